@@ -154,10 +154,8 @@ struct bgl_ctx {
                                   // runs, [2] allocation-free iterations (read by bgl_ctx_sync)
     int *h_flag = nullptr;        // pinned mirror
     unsigned char *noalloc_scratch = nullptr;   // device address of the allocation-free scratch array
-    // autotuner choices: exact-repulsion targets per thread by log2 of the pairs
-    std::mutex tune_mu;
-    std::map<int, int> tune_exact;
     // measured exact/FMM choice by component size octave (fmm_min_nodes = -1)
+    std::mutex tune_mu;
     std::map<int, bool> tune_fmm;
 };
 

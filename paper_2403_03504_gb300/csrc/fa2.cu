@@ -31,13 +31,13 @@ namespace bgl {
 
 namespace {
 
-// pairs of a thread's targets summed with packed FP32x2 arithmetic in the
-// exact kernel (the rest scalar)
-#ifndef BGL_EXACT_PACKED
-#define BGL_EXACT_PACKED 2
+constexpr int EX_THREADS = 128, EX_WARPS = EX_THREADS / 32;
+constexpr int EX_STAGE = 1024;                 // sources summed before they enter the compensated total
+constexpr int64_t EX_SPLIT_MAX_N = 1 << 16;    // components up to this size: a block per stage (partial sums in memory)
+#ifndef BGL_EXACT_WIDE_WARPS
+#define BGL_EXACT_WIDE_WARPS 3000              // warps at two targets per lane from which a run takes two
 #endif
-constexpr int EX_THREADS = 256;                // a tile is EX_THREADS x R targets, R = 1, 2 or 4 (autotuned)
-constexpr int EX_STILE = 1024;                 // sources per shared-memory stage
+constexpr int ATT_LANE_DEG = 8;                // attraction: nodes up to this degree by one lane each
 constexpr int HEAVY_DEG = 128;
 constexpr int HEAVY_CHUNK = 2048;              // adjacency entries per block for high-degree nodes
 constexpr int RED_TILE = 256;                  // nodes per swing/traction tile (one per thread)
@@ -49,82 +49,372 @@ struct Tile {
 };
 
 
-// K1 (exact): repulsion of every target in the tile from every node of its component
-template <int EX_R>
-__global__ void __launch_bounds__(EX_THREADS) exact_repulsion_kernel(
-    const Tile *__restrict__ tiles, const int64_t *__restrict__ comp_off, int64_t c0, const float2 *__restrict__ xy,
-    const float *__restrict__ mass, int64_t qbase, float kr, const float2 *__restrict__ fa, float2 *__restrict__ f) {
-    __shared__ float4 src[EX_STILE];
-    const Tile t = tiles[blockIdx.x];
-    const int64_t s_begin = comp_off[c0 + t.comp], s_end = comp_off[c0 + t.comp + 1];
-    float zx[EX_R], zy[EX_R], sx[EX_R], sy[EX_R], cx[EX_R], cy[EX_R];
-#pragma unroll
-    for (int r = 0; r < EX_R; ++r) {
-        int64_t q = t.t0 + threadIdx.x + r * EX_THREADS;
-        float2 p = q < t.t1 ? xy[q - qbase] : make_float2(0.f, 0.f);
-        zx[r] = p.x;
-        zy[r] = p.y;
-        sx[r] = sy[r] = cx[r] = cy[r] = 0.f;
-    }
-    for (int64_t s0 = s_begin; s0 < s_end; s0 += EX_STILE) {
-        const int cnt = (int)(s_end - s0 < EX_STILE ? s_end - s0 : EX_STILE);
-        __syncthreads();
-        for (int k = threadIdx.x; k < cnt; k += EX_THREADS) {
-            float2 p = xy[s0 + k - qbase];
-            src[k] = make_float4(p.x, p.y, mass[s0 + k], 0.f);
+// Swing and traction sums of a component (Section 3.2).  One order for
+// every kernel that makes them (here and the fused FMM iteration's
+// combine_kernel), so that a component gets the same s_G whatever runs it:
+// FP32 over 32 consecutive nodes (a butterfly), FP64 over the eight such
+// groups of a 256-node tile, then thread t of 256 over the tiles t, t + 256,
+// ..., a butterfly in each warp, and the warps in order.  (FP64 issue is
+// scarce on this part, so it is kept off the per-node path.)
+struct SwingArgs {
+    const float2 *fprev;      // F_{t-1} (null in the exact kernel: forces only)
+    int variant;
+    double tau;
+    double2 *partial;         // one per 256-node tile (swing_traction_kernel)
+    float2 *group;            // one per 32 nodes (exact kernel)
+    const int32_t *tile_off;  // per component: its first tile, [ncomp + 1] (equal: no tiles here)
+    double *sg;               // [ncomp]
+    unsigned *counter;        // [ncomp] tiles of each component done, zero between launches
+    double *stats;            // optional, component 0
+    int *iter;                // iteration counter for stats
+};
+
+// s_G from the component's sums, by one thread of its last block to finish
+__device__ __forceinline__ void swing_finish(const SwingArgs &a, int comp, double swg, double trc) {
+    const double s_new = fa2_global_speed(swg, trc, a.sg[comp], a.tau);
+    a.sg[comp] = s_new;
+    if (comp == 0) {
+        if (a.stats) {
+            const int it = *a.iter;
+            a.stats[3 * it] = swg;
+            a.stats[3 * it + 1] = trc;
+            a.stats[3 * it + 2] = s_new;
         }
-        __syncthreads();
-        float ax[EX_R], ay[EX_R];
+        *a.iter += 1;
+    }
+    a.counter[comp] = 0u;
+}
+
+__device__ __forceinline__ void warp_sum2(float &x, float &y) {
 #pragma unroll
-        for (int r = 0; r < EX_R; ++r) ax[r] = ay[r] = 0.f;
-        {
-            // targets 2k, 2k + 1 (k < R2) in packed FP32x2 (negated targets
-            // and sums, bitwise the scalar pair's result), the rest scalar
-            constexpr int R2 = EX_R / 2 < BGL_EXACT_PACKED ? EX_R / 2 : BGL_EXACT_PACKED;
-            float2 nzx[R2 > 0 ? R2 : 1], nzy[R2 > 0 ? R2 : 1], gx[R2 > 0 ? R2 : 1], gy[R2 > 0 ? R2 : 1];
+    for (int o = 16; o > 0; o >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+}
+__device__ __forceinline__ void warp_sum2(double &x, double &y) {
 #pragma unroll
-            for (int k = 0; k < R2; ++k) {
-                nzx[k] = make_float2(-zx[2 * k], -zx[2 * k + 1]);
-                nzy[k] = make_float2(-zy[2 * k], -zy[2 * k + 1]);
-                gx[k] = gy[k] = make_float2(0.f, 0.f);
+    for (int o = 16; o > 0; o >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+}
+
+// One block of the exact sum: EX_THREADS R targets of a component (a tile)
+// against one stage of its sources, or against all of them, or the tile's
+// attraction and gravity (component-order positions).
+struct ExBlock {
+    int32_t t0, nt;           // targets [t0, t0 + nt)
+    int32_t s0, s1;           // sources [s0, s1) (empty: attraction and gravity)
+    int32_t comp, tile;       // component relative to c0, tile index (over all components)
+    int32_t k, parts;         // part k of `parts` partial sums of the tile
+    int32_t part, n;          // the tile's first partial sum in units of a tile's targets; component size
+};
+
+struct ExArgs {
+    const ExBlock *blk;
+    int first;                // block 0 of the launch (past the attraction blocks: repulsion only)
+    bool att;
+    const float2 *xy;         // xy[q - qbase]
+    const float *mass;        // mass[q]
+    const int64_t *coff;
+    const int32_t *cadj;
+    int64_t qbase, fbase;     // f[q - fbase], fa and fprev likewise
+    float kr, kg;
+    float2 *part;             // partial sums
+    unsigned *arrive;         // [tiles] blocks of the tile done, zero between launches
+    float2 *fa;               // attraction and gravity
+    float2 *f;
+    SwingArgs sw;
+};
+
+// Attraction and gravity of a tile: -sum_{j adjacent} (p_i - p_j) - kg m_i p_i,
+// in the order of attraction_gravity_kernel (one after another up to
+// HEAVY_DEG entries, chunks of HEAVY_CHUNK above).  A lane sums a node of up
+// to ATT_LANE_DEG entries; for one of up to HEAVY_DEG the warp loads 32
+// entries at a time and adds them in order through shuffles (one thread
+// loading them took 10 us for a node of 120); the rest the block takes.
+template <int R>
+__device__ void tile_attraction(const ExArgs &a, const ExBlock &b) {
+    __shared__ float2 hred[8];
+    __shared__ int hlist[EX_THREADS * R], nh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float2 *__restrict__ xy = a.xy - a.qbase;
+    if (threadIdx.x == 0) nh = 0;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = (warp * R + r) * 32 + lane;
+        const int q = b.t0 + i;
+        const bool ok = i < b.nt;
+        const int64_t e0 = ok ? a.coff[q] : 0, deg = ok ? a.coff[q + 1] - e0 : 0;
+        const float2 p = ok ? xy[q] : make_float2(0.f, 0.f);
+        float ax = 0.f, ay = 0.f;
+        if (deg <= ATT_LANE_DEG) {
+            float2 o[ATT_LANE_DEG];
+#pragma unroll
+            for (int e = 0; e < ATT_LANE_DEG; ++e) o[e] = e < deg ? xy[a.cadj[e0 + e]] : p;
+#pragma unroll
+            for (int e = 0; e < ATT_LANE_DEG; ++e) {
+                if (e < deg) {
+                    ax -= p.x - o[e].x;
+                    ay -= p.y - o[e].y;
+                }
             }
+        }
+        if (deg > HEAVY_DEG) hlist[atomicAdd(&nh, 1)] = i;          // (nodes are independent: any order)
+        unsigned mid = __ballot_sync(0xffffffffu, deg > ATT_LANE_DEG && deg <= HEAVY_DEG);
+        while (mid) {
+            const int l = __ffs(mid) - 1;
+            mid &= mid - 1;
+            const int64_t f0 = __shfl_sync(0xffffffffu, e0, l);
+            const int d = __shfl_sync(0xffffffffu, (int)deg, l);
+            const float px = __shfl_sync(0xffffffffu, p.x, l), py = __shfl_sync(0xffffffffu, p.y, l);
+            float2 t[HEAVY_DEG / 32];
+#pragma unroll
+            for (int c = 0; c < HEAVY_DEG / 32; ++c) {
+                const int e = c * 32 + lane;
+                const float2 o = e < d ? xy[a.cadj[f0 + e]] : make_float2(px, py);
+                t[c] = make_float2(px - o.x, py - o.y);
+            }
+            float sx = 0.f, sy = 0.f;
+#pragma unroll
+            for (int c = 0; c < HEAVY_DEG / 32; ++c) {
+                const int m = min(32, d - c * 32);
+#pragma unroll 8
+                for (int j = 0; j < m; ++j) {
+                    sx -= __shfl_sync(0xffffffffu, t[c].x, j);
+                    sy -= __shfl_sync(0xffffffffu, t[c].y, j);
+                }
+            }
+            if (lane == l) {
+                ax = sx;
+                ay = sy;
+            }
+        }
+        if (ok && deg <= HEAVY_DEG) {
+            const float km = a.kg * a.mass[q];
+            a.fa[q - a.fbase] = make_float2(ax - km * p.x, ay - km * p.y);
+        }
+    }
+    __syncthreads();
+    for (int h = 0; h < nh; ++h) {
+        const int q = b.t0 + hlist[h];
+        const int64_t e0 = a.coff[q], e1 = a.coff[q + 1];
+        const float2 p = xy[q];
+        float sx = 0.f, sy = 0.f;                                   // (thread 0)
+        for (int64_t c0 = e0; c0 < e1; c0 += HEAVY_CHUNK) {
+            const int64_t c1 = min(e1, c0 + HEAVY_CHUNK);
+            // 256 strided sums, two a thread
+#pragma unroll
+            for (int u = 0; u < 256 / EX_THREADS; ++u) {
+                float ax = 0.f, ay = 0.f;
+                for (int64_t e = c0 + u * EX_THREADS + threadIdx.x; e < c1; e += 256) {
+                    const float2 o = xy[a.cadj[e]];
+                    ax -= p.x - o.x;
+                    ay -= p.y - o.y;
+                }
+                warp_sum2(ax, ay);
+                if (lane == 0) hred[u * EX_WARPS + warp] = make_float2(ax, ay);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                float cx = 0.f, cy = 0.f;
+                for (int w = 0; w < 8; ++w) {
+                    cx += hred[w].x;
+                    cy += hred[w].y;
+                }
+                sx += cx;
+                sy += cy;
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            const float km = a.kg * a.mass[q];
+            a.fa[q - a.fbase] = make_float2(sx - km * p.x, sy - km * p.y);
+        }
+    }
+}
+
+// K1 (exact), with K2 and K3 of its targets: F_rep (+ attraction + gravity,
+// and the tile's swing and traction).
+//
+// Bound by the MUFU: one reciprocal a pair, 16 pairs per clock and SM.  A
+// target's sum is a chain over its sources (in stages of 1,024, each stage's
+// sum entering a compensated total), so what can be spread over the chip is
+// targets times stages: a block takes EX_THREADS R targets and one stage,
+// and the tile's last block to finish adds the stages in order, adds the
+// attraction (a block of its own in the same launch) and sums swing and
+// traction.  R = 1 for few warps (each then has a scheduler to itself), R = 2
+// in packed FP32x2 arithmetic for many (less issue per pair); the sums are
+// the same bit for bit.  One block per 512 targets with all their sources
+// took 116 us for 2,821 nodes (6 blocks on 152 SMs).
+template <int R>
+__global__ void __launch_bounds__(EX_THREADS) exact_kernel(ExArgs a) {
+    __shared__ float4 src[EX_STAGE];
+    __shared__ double ws[8], wt[8];
+    __shared__ bool last;
+    constexpr int TT = EX_THREADS * R;
+    const ExBlock b = a.blk[a.first + blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float2 *__restrict__ xy = a.xy - a.qbase;
+    float sx[R], sy[R];
+    if (b.s0 == b.s1) {
+        tile_attraction<R>(a, b);
+    } else {
+        float zx[R], zy[R], cx[R], cy[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = (warp * R + r) * 32 + lane;
+            const float2 p = i < b.nt ? xy[b.t0 + i] : make_float2(0.f, 0.f);
+            zx[r] = p.x;
+            zy[r] = p.y;
+            sx[r] = sy[r] = cx[r] = cy[r] = 0.f;
+        }
+        const bool work = warp * R * 32 < b.nt;
+        for (int s0 = b.s0; s0 < b.s1; s0 += EX_STAGE) {
+            const int cnt = min(b.s1 - s0, EX_STAGE);
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < EX_STAGE / EX_THREADS; ++k) {
+                const int j = k * EX_THREADS + threadIdx.x;
+                if (j < cnt) {
+                    const float2 p = xy[s0 + j];
+                    src[j] = make_float4(p.x, p.y, a.mass[s0 + j], 0.f);
+                }
+            }
+            __syncthreads();
+            if (!work) continue;
+            float ax[R], ay[R];
+            if constexpr (R == 1) {
+                ax[0] = ay[0] = 0.f;
+#pragma unroll 8
+                for (int j = 0; j < cnt; ++j) p2p_pair(zx[0], zy[0], src[j], ax[0], ay[0]);
+            } else {
+                float2 nzx[R / 2], nzy[R / 2], gx[R / 2], gy[R / 2];
+#pragma unroll
+                for (int k = 0; k < R / 2; ++k) {
+                    nzx[k] = make_float2(-zx[2 * k], -zx[2 * k + 1]);
+                    nzy[k] = make_float2(-zy[2 * k], -zy[2 * k + 1]);
+                    gx[k] = gy[k] = make_float2(0.f, 0.f);
+                }
 #pragma unroll 4
-            for (int j = 0; j < cnt; ++j) {
-                const float4 q = src[j];
+                for (int j = 0; j < cnt; ++j) {
+                    const float4 q = src[j];
 #pragma unroll
-                for (int k = 0; k < R2; ++k) p2p_pair2(nzx[k], nzy[k], q, gx[k], gy[k]);
+                    for (int k = 0; k < R / 2; ++k) p2p_pair2(nzx[k], nzy[k], q, gx[k], gy[k]);
+                }
 #pragma unroll
-                for (int r = 2 * R2; r < EX_R; ++r) p2p_pair(zx[r], zy[r], q, ax[r], ay[r]);
+                for (int k = 0; k < R / 2; ++k) {
+                    ax[2 * k] = -gx[k].x;
+                    ax[2 * k + 1] = -gx[k].y;
+                    ay[2 * k] = -gy[k].x;
+                    ay[2 * k + 1] = -gy[k].y;
+                }
             }
+            // each stage's sum enters a compensated (Kahan) running total
 #pragma unroll
-            for (int k = 0; k < R2; ++k) {
-                ax[2 * k] = -gx[k].x;
-                ax[2 * k + 1] = -gx[k].y;
-                ay[2 * k] = -gy[k].x;
-                ay[2 * k + 1] = -gy[k].y;
+            for (int r = 0; r < R; ++r) {
+                float y = ax[r] - cx[r];
+                float s = sx[r] + y;
+                cx[r] = (s - sx[r]) - y;
+                sx[r] = s;
+                y = ay[r] - cy[r];
+                s = sy[r] + y;
+                cy[r] = (s - sy[r]) - y;
+                sy[r] = s;
             }
-        }
-        // blocked accumulation: each stage's partial sum enters a
-        // compensated (Kahan) running total
-#pragma unroll
-        for (int r = 0; r < EX_R; ++r) {
-            float y = ax[r] - cx[r];
-            float s = sx[r] + y;
-            cx[r] = (s - sx[r]) - y;
-            sx[r] = s;
-            y = ay[r] - cy[r];
-            s = sy[r] + y;
-            cy[r] = (s - sy[r]) - y;
-            sy[r] = s;
         }
     }
+    const unsigned blocks = (unsigned)b.parts + (a.att ? 1u : 0u);
+    if (blocks > 1) {
+        float2 *part = a.part + (size_t)b.part * TT;
+        if (b.s0 != b.s1) {
 #pragma unroll
-    for (int r = 0; r < EX_R; ++r) {
-        int64_t q = t.t0 + threadIdx.x + r * EX_THREADS;
-        if (q >= t.t1) continue;
-        float km = kr * mass[q];
-        const float2 a = fa ? fa[q - qbase] : make_float2(0.f, 0.f);
-        f[q - qbase] = make_float2(fmaf(km, sx[r], a.x), fmaf(km, sy[r], a.y));
+            for (int r = 0; r < R; ++r)
+                part[b.k * TT + (warp * R + r) * 32 + lane] = make_float2(sx[r], sy[r]);
+        }
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&a.arrive[b.tile], 1u) == blocks - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) a.arrive[b.tile] = 0u;
+        float cx[R], cy[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) sx[r] = sy[r] = cx[r] = cy[r] = 0.f;
+        for (int k = 0; k < b.parts; ++k) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float2 v = __ldcg(&part[k * TT + (warp * R + r) * 32 + lane]);
+                float y = v.x - cx[r];
+                float s = sx[r] + y;
+                cx[r] = (s - sx[r]) - y;
+                sx[r] = s;
+                y = v.y - cy[r];
+                s = sy[r] + y;
+                cy[r] = (s - sy[r]) - y;
+                sy[r] = s;
+            }
+        }
+    }
+    const bool swing = a.sw.fprev != nullptr;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = (warp * R + r) * 32 + lane;
+        float sw = 0.f, tr = 0.f;
+        if (i < b.nt) {
+            const int64_t q = b.t0 + i;
+            const float m = a.mass[q], km = a.kr * m;
+            const float2 t = a.att ? __ldcg(&a.fa[q - a.fbase]) : make_float2(0.f, 0.f);
+            const float2 F = make_float2(fmaf(km, sx[r], t.x), fmaf(km, sy[r], t.y));
+            a.f[q - a.fbase] = F;
+            if (swing) fa2_swing_terms(F, a.sw.fprev[q - a.fbase], m, a.sw.variant, sw, tr);
+        }
+        if (swing) {
+            warp_sum2(sw, tr);
+            if (lane == 0) a.sw.group[(size_t)b.tile * (TT / 32) + warp * R + r] = make_float2(sw, tr);
+        }
+    }
+    if (!swing) return;
+    __threadfence();
+    __syncthreads();
+    const int tile0 = a.sw.tile_off[b.comp];
+    if (threadIdx.x == 0)
+        last = atomicAdd(&a.sw.counter[b.comp], 1u) == (unsigned)(a.sw.tile_off[b.comp + 1] - tile0) - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const float2 *group = a.sw.group + (size_t)tile0 * (TT / 32);
+    const int ng = (b.n + 31) / 32, nt = (ng + 7) / 8;
+#pragma unroll
+    for (int u = 0; u < 256 / EX_THREADS; ++u) {
+        double swg = 0.0, trc = 0.0;
+        for (int k = u * EX_THREADS + (int)threadIdx.x; k < nt; k += 256) {
+            double s = 0.0, t = 0.0;
+            for (int w = 8 * k; w < min(8 * k + 8, ng); ++w) {
+                const float2 v = __ldcg(&group[w]);         // written by other blocks: bypass L1
+                s += (double)v.x;
+                t += (double)v.y;
+            }
+            swg += s;
+            trc += t;
+        }
+        warp_sum2(swg, trc);
+        if (lane == 0) {
+            ws[u * EX_WARPS + warp] = swg;
+            wt[u * EX_WARPS + warp] = trc;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double swg = 0.0, trc = 0.0;
+        for (int w = 0; w < 8; ++w) {
+            swg += ws[w];
+            trc += wt[w];
+        }
+        swing_finish(a.sw, b.comp, swg, trc);
     }
 }
 
@@ -221,74 +511,41 @@ __global__ void heavy_rows_kernel(const int32_t *__restrict__ heavy, const int64
     rows[2 * i + 1] = coff[heavy[i] + 1];
 }
 
-struct RedArgs {
-    const Tile *tiles;        // node tiles, each inside one component
-    const int64_t *tile_off;  // per component: first tile, [ncomp+1]
-    int ncomp;
-    const float2 *f, *fprev;
-    const float *mass;
-    int64_t qbase;
-    int variant;
-    double tau;
-    double2 *partial;         // [ntiles]
-    double *sg;               // [ncomp]
-    unsigned *counter;        // [ncomp] tiles of each component done, zero between launches
-    double *stats;            // optional, component 0
-    int *iter;                // iteration counter for stats
-};
-
-// K3: swing / traction sums (Section 3.2) and the global speed of each component
-__global__ void swing_traction_kernel(RedArgs a) {
-    __shared__ double ws[32], wt[32];
+// K3 for the FMM's components (the exact kernel sums its own): tiles of 256
+// consecutive nodes of a component, one node per thread.
+__global__ void swing_traction_kernel(SwingArgs a, const Tile *__restrict__ tiles, const float2 *__restrict__ f,
+                                      const float *__restrict__ mass, int64_t fbase) {
+    __shared__ double ws[8], wt[8];
     __shared__ bool last;
-    const Tile t = a.tiles[blockIdx.x];
-    // FP32 within a warp (32 terms), FP64 across warps, tiles and components
-    // (FP64 issue is scarce on this part, so it is kept off the per-node
-    // path).  The order is the fused FMM iteration's (combine_kernel): tiles
-    // of 256 consecutive nodes of a component, one node per thread, so a
-    // component gets the same s_G whether it is iterated alone or with others.
+    const Tile t = tiles[blockIdx.x];
     float sw = 0.f, tr = 0.f;
     const int i = threadIdx.x;
     if (i < (int)(t.t1 - t.t0)) {
         const int64_t q = t.t0 + i;
-        fa2_swing_terms(a.f[q - a.qbase], a.fprev[q - a.qbase], a.mass[q], a.variant, sw, tr);
+        fa2_swing_terms(f[q - fbase], a.fprev[q - fbase], mass[q], a.variant, sw, tr);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        sw += __shfl_xor_sync(0xffffffffu, sw, o);
-        tr += __shfl_xor_sync(0xffffffffu, tr, o);
-    }
+    warp_sum2(sw, tr);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) { ws[warp] = (double)sw; wt[warp] = (double)tr; }
     __syncthreads();
+    const int c = t.comp, k0 = a.tile_off[c], nk = a.tile_off[c + 1] - k0;
     if (threadIdx.x == 0) {
         double s = 0.0, u = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { s += ws[w]; u += wt[w]; }
+        for (int w = 0; w < 8; ++w) { s += ws[w]; u += wt[w]; }
         a.partial[blockIdx.x] = make_double2(s, u);
         __threadfence();
-        const unsigned ntc = (unsigned)(a.tile_off[t.comp + 1] - a.tile_off[t.comp]);
-        last = atomicAdd(&a.counter[t.comp], 1u) == ntc - 1;
+        last = atomicAdd(&a.counter[c], 1u) == (unsigned)nk - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // the component's last tile to finish adds its tile sums in the fused
-    // iteration's order (combine_kernel's last block, also 256 threads):
-    // thread t sums the tiles t, t + 256, ... in order, a butterfly in each
-    // warp, then the warps' results in warp order
-    const int c = t.comp;
-    const int64_t k0 = a.tile_off[c], nk = a.tile_off[c + 1] - k0;
     double swg = 0.0, trc = 0.0;
-    for (int64_t k = threadIdx.x; k < nk; k += blockDim.x) {
+    for (int k = threadIdx.x; k < nk; k += 256) {
         const double2 v = __ldcg(&a.partial[k0 + k]);   // written by other blocks: bypass L1
         swg += v.x;
         trc += v.y;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        swg += __shfl_xor_sync(0xffffffffu, swg, o);
-        trc += __shfl_xor_sync(0xffffffffu, trc, o);
-    }
+    warp_sum2(swg, trc);
     __syncthreads();
     if (lane == 0) {
         ws[warp] = swg;
@@ -298,29 +555,32 @@ __global__ void swing_traction_kernel(RedArgs a) {
     if (threadIdx.x == 0) {
         swg = 0.0;
         trc = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        for (int w = 0; w < 8; ++w) {
             swg += ws[w];
             trc += wt[w];
         }
-        const double s_new = fa2_global_speed(swg, trc, a.sg[c], a.tau);
-        a.sg[c] = s_new;
-        if (c == 0) {
-            if (a.stats) {
-                const int it = *a.iter;
-                a.stats[3 * it] = swg;
-                a.stats[3 * it + 1] = trc;
-                a.stats[3 * it + 2] = s_new;
-            }
-            *a.iter += 1;
-        }
-        a.counter[c] = 0u;
+        swing_finish(a, c, swg, trc);
     }
 }
 
-// K4: node speeds and the position update
+// Control of the device-side loop: count the iteration and keep looping
+// while below `iters` (count null: no loop).
+struct LoopCtl {
+    cudaGraphConditionalHandle h = 0;
+    int *count = nullptr;
+    int iters = 0;
+};
+__device__ __forceinline__ void loop_step(const LoopCtl &l) {
+    const int k = ++*l.count;
+    cudaGraphSetConditional(l.h, k < l.iters ? 1u : 0u);
+}
+
+// K4: node speeds and the position update; the first thread also steps the loop
 __global__ void update_kernel(const float2 *__restrict__ f, float2 *__restrict__ fprev, float2 *__restrict__ xy,
                               const int32_t *__restrict__ node_comp, const double *__restrict__ sg, int64_t q0,
-                              int64_t q1, int64_t qbase, int64_t c0, float ks, float ksmax, int *bad) {
+                              int64_t q1, int64_t qbase, int64_t c0, float ks, float ksmax, int *bad,
+                              LoopCtl loop) {
+    if (loop.count && blockIdx.x == 0 && threadIdx.x == 0) loop_step(loop);
     int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= q1) return;
     const float2 F = f[q - qbase], P = fprev[q - qbase];
@@ -334,88 +594,102 @@ inline unsigned nblocks(int64_t n, int t) { return (unsigned)std::max<int64_t>(1
 
 }  // namespace
 
-static void launch_exact(int r, int ntiles, const Tile *tiles, const int64_t *comp_off, int64_t c0, const float2 *xy,
-                         const float *mass, int64_t qbase, float kr, const float2 *fa, float2 *f, cudaStream_t s) {
-    if (r == 1)
-        exact_repulsion_kernel<1><<<ntiles, EX_THREADS, 0, s>>>(tiles, comp_off, c0, xy, mass, qbase, kr, fa, f);
-    else if (r == 4)
-        exact_repulsion_kernel<4><<<ntiles, EX_THREADS, 0, s>>>(tiles, comp_off, c0, xy, mass, qbase, kr, fa, f);
-    else
-        exact_repulsion_kernel<2><<<ntiles, EX_THREADS, 0, s>>>(tiles, comp_off, c0, xy, mass, qbase, kr, fa, f);
-    BGL_LAUNCH_CHECK();
-}
+// Blocks of the exact sum over the given components (indices >= c0): for each
+// tile of EX_THREADS R targets one for its attraction, and one for each stage
+// of its sources, or for all of them in a component of more than
+// EX_SPLIT_MAX_N nodes (the partial sums of more would take n^2 / 128 bytes,
+// and it has tiles enough).
+struct ExactSum {
+    DevBuf<ExBlock> blk;
+    DevBuf<float2> part, group;
+    DevBuf<unsigned> arrive;
+    std::vector<int32_t> tile_off;    // per component of [c0, c1): its first tile
+    int R = 1, n_blk = 0, n_tiles = 0;     // blocks of the sum (the tiles' attraction blocks come before them)
 
-// tiles of EX_THREADS * r targets over the given components (indices >= c0)
-static std::vector<Tile> exact_tiles(const bgl_graph *g, int64_t c0, const std::vector<int64_t> &comps, int r) {
-    std::vector<Tile> ex;
-    const int64_t tile = (int64_t)EX_THREADS * r;
-    for (int64_t c : comps) {
-        const int64_t a = g->h_comp_off[c], b = g->h_comp_off[c + 1];
-        for (int64_t t = a; t < b; t += tile) ex.push_back(Tile{(int32_t)(c - c0), 0, t, std::min(b, t + tile)});
-    }
-    return ex;
-}
-
-// Autotuner of the exact tiles: the first time a context meets a set of
-// exact components of a given scale (log2 of the pairs of one evaluation),
-// each R in {1, 2, 4} is timed on one evaluation (after one warm-up launch),
-// and the fastest is kept for that scale.  Small sets (under 2^24 pairs)
-// take R = 2 untimed.
-static int exact_tile_choice(bgl_graph *g, const bgl_params *p, const std::vector<int64_t> &comps) {
-    if (comps.empty()) return 2;
-    double pairs = 0.0;
-    for (int64_t c : comps) {
-        const double n = (double)(g->h_comp_off[c + 1] - g->h_comp_off[c]);
-        pairs += n * n;
-    }
-    if (pairs < (double)(1 << 24)) return 2;
-    const int scale = (int)std::log2(pairs);
-    bgl_ctx *ctx = g->ctx;
-    {
-        std::lock_guard<std::mutex> lk(ctx->tune_mu);
-        auto it = ctx->tune_exact.find(scale);
-        if (it != ctx->tune_exact.end()) return it->second;
-    }
-    cudaStream_t s = ctx->stream;
-    const int64_t c0 = comps.front();
-    const int64_t q0 = g->h_comp_off[c0], q1 = g->h_comp_off[comps.back() + 1];
-    DevBuf<float2> xy(ctx->alloc, q1 - q0), f(ctx->alloc, q1 - q0);
-    init_positions(g, p, xy.p, q0, q1);
-    cudaEvent_t e0, e1;
-    BGL_CUDA(cudaEventCreate(&e0));
-    BGL_CUDA(cudaEventCreate(&e1));
-    int best = 2;
-    float best_ms = 1e30f;
-    try {
-        for (int r : {1, 2, 4}) {
-            const std::vector<Tile> ex = exact_tiles(g, c0, comps, r);
-            DevBuf<Tile> tiles(ctx->alloc, ex.size());
-            BGL_CUDA(cudaMemcpyAsync(tiles.p, ex.data(), sizeof(Tile) * ex.size(), cudaMemcpyHostToDevice, s));
-            launch_exact(r, (int)ex.size(), tiles.p, g->comp_off.p, c0, xy.p, g->mass.p, q0, (float)p->kr, nullptr,
-                         f.p, s);
-            BGL_CUDA(cudaEventRecord(e0, s));
-            launch_exact(r, (int)ex.size(), tiles.p, g->comp_off.p, c0, xy.p, g->mass.p, q0, (float)p->kr, nullptr,
-                         f.p, s);
-            BGL_CUDA(cudaEventRecord(e1, s));
-            BGL_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            BGL_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-            if (ms < best_ms) {
-                best_ms = ms;
-                best = r;
-            }
+    // reps: every tile so many times (each copy writes the same forces)
+    void make(bgl_graph *g, int64_t c0, int64_t c1, const std::vector<int64_t> &comps, int reps = 1) {
+        auto parts_of = [](int64_t n) { return n <= EX_SPLIT_MAX_N ? (n + EX_STAGE - 1) / EX_STAGE : int64_t(1); };
+        int64_t wide = 0;
+        for (int64_t c : comps) {
+            const int64_t n = g->h_comp_off[c + 1] - g->h_comp_off[c];
+            wide += (n + 63) / 64 * parts_of(n) * reps;
         }
-    } catch (...) {
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        throw;
+        R = wide >= BGL_EXACT_WIDE_WARPS ? 2 : 1;
+        const int64_t tt = EX_THREADS * R;
+        std::vector<ExBlock> att, sum;
+        tile_off.assign(c1 - c0 + 1, 0);
+        int32_t tile = 0, units = 0;
+        size_t next = 0;
+        for (int64_t c = c0; c < c1; ++c) {
+            tile_off[c - c0] = tile;
+            if (next >= comps.size() || comps[next] != c) continue;
+            ++next;
+            const int64_t a = g->h_comp_off[c], n = g->h_comp_off[c + 1] - a, parts = parts_of(n);
+            for (int r = 0; r < reps; ++r)
+                for (int64_t t = 0; t < n; t += tt, ++tile, units += (int32_t)parts) {
+                    ExBlock b;
+                    b.t0 = (int32_t)(a + t);
+                    b.nt = (int32_t)std::min(tt, n - t);
+                    b.s0 = b.s1 = 0;
+                    b.comp = (int32_t)(c - c0);
+                    b.tile = tile;
+                    b.k = -1;
+                    b.parts = (int32_t)parts;
+                    b.part = units;
+                    b.n = (int32_t)n;
+                    att.push_back(b);
+                    for (int64_t k = 0; k < parts; ++k) {
+                        b.k = (int32_t)k;
+                        b.s0 = (int32_t)(a + k * EX_STAGE);
+                        b.s1 = (int32_t)(a + (k + 1 < parts ? (k + 1) * EX_STAGE : n));
+                        sum.push_back(b);
+                    }
+                }
+        }
+        tile_off[c1 - c0] = tile;
+        n_blk = (int)sum.size();
+        n_tiles = tile;
+        if (!n_blk) return;
+        att.insert(att.end(), sum.begin(), sum.end());
+        Allocator *A = g->ctx->alloc;
+        cudaStream_t s = g->ctx->stream;
+        blk.reset(A, att.size());
+        part.reset(A, (size_t)units * tt);
+        group.reset(A, (size_t)tile * (tt / 32));
+        arrive.reset(A, tile);
+        BGL_CUDA(cudaMemcpyAsync(blk.p, att.data(), sizeof(ExBlock) * att.size(), cudaMemcpyHostToDevice, s));
+        BGL_CUDA(cudaMemsetAsync(arrive.p, 0, sizeof(unsigned) * tile, s));
+        BGL_CUDA(cudaStreamSynchronize(s));      // att goes out of scope
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    std::lock_guard<std::mutex> lk(ctx->tune_mu);
-    ctx->tune_exact[scale] = best;
-    return best;
-}
+
+    // F_rep, or with fa (scratch) the total force; swing and traction where sw.fprev is set
+    void launch(const bgl_graph *g, const bgl_params *p, const float2 *xy, int64_t qbase, float2 *f, int64_t fbase,
+                float2 *fa, const SwingArgs &sw, cudaStream_t s) const {
+        if (!n_blk) return;
+        ExArgs a;
+        a.blk = blk.p;
+        a.att = fa != nullptr;
+        a.first = a.att ? 0 : n_tiles;
+        a.xy = xy;
+        a.mass = g->mass.p;
+        a.coff = g->coff.p;
+        a.cadj = g->cadj.p;
+        a.qbase = qbase;
+        a.fbase = fbase;
+        a.kr = (float)p->kr;
+        a.kg = (float)p->kg;
+        a.part = part.p;
+        a.arrive = arrive.p;
+        a.fa = fa;
+        a.f = f;
+        a.sw = sw;
+        a.sw.group = group.p;
+        const unsigned blocks = (unsigned)(n_blk + (a.att ? n_tiles : 0));
+        if (R == 1) exact_kernel<1><<<blocks, EX_THREADS, 0, s>>>(a);
+        else exact_kernel<2><<<blocks, EX_THREADS, 0, s>>>(a);
+        BGL_LAUNCH_CHECK();
+    }
+};
 
 bool use_fmm(const bgl_params *p, int64_t n) {
     if (p->repulsion == BGL_REP_FMM) return true;
@@ -450,13 +724,11 @@ static bool use_fmm_for(bgl_graph *g, const bgl_params *p, int64_t c) {
     const int64_t q0 = g->h_comp_off[c], q1 = g->h_comp_off[c + 1];
     DevBuf<float2> xy(ctx->alloc, n), f(ctx->alloc, n);
     init_positions(g, p, xy.p, q0, q1);
-    const std::vector<Tile> one = exact_tiles(g, c, std::vector<int64_t>{c}, 2);
-    // repeated until there are four tiles per SM (each copy writes the same forces)
-    const int reps = std::max<int>(1, (4 * ctx->num_sms + (int)one.size() - 1) / (int)one.size());
-    std::vector<Tile> ex;
-    for (int r = 0; r < reps; ++r) ex.insert(ex.end(), one.begin(), one.end());
-    DevBuf<Tile> tiles(ctx->alloc, ex.size());
-    BGL_CUDA(cudaMemcpyAsync(tiles.p, ex.data(), sizeof(Tile) * ex.size(), cudaMemcpyHostToDevice, s));
+    // repeated until there are eight blocks per SM (each copy writes the same forces)
+    ExactSum ex;
+    ex.make(g, c, c + 1, {c});
+    const int reps = std::max<int>(1, (8 * ctx->num_sms + ex.n_blk - 1) / ex.n_blk);
+    ex.make(g, c, c + 1, {c}, reps);
     FmmPlan *pl = fmm_create(g, p, c);
     cudaEvent_t e[4] = {nullptr, nullptr, nullptr, nullptr};
     float ms_fmm = 0.f, ms_exact = 0.f;
@@ -466,9 +738,9 @@ static bool use_fmm_for(bgl_graph *g, const bgl_params *p, int64_t c) {
         BGL_CUDA(cudaEventRecord(e[0], s));
         fmm_repulsion(pl, xy.p, q0, f.p, q0);
         BGL_CUDA(cudaEventRecord(e[1], s));
-        launch_exact(2, (int)ex.size(), tiles.p, g->comp_off.p, c, xy.p, g->mass.p, q0, (float)p->kr, nullptr, f.p, s);
+        ex.launch(g, p, xy.p, q0, f.p, q0, nullptr, SwingArgs{}, s);
         BGL_CUDA(cudaEventRecord(e[2], s));
-        launch_exact(2, (int)ex.size(), tiles.p, g->comp_off.p, c, xy.p, g->mass.p, q0, (float)p->kr, nullptr, f.p, s);
+        ex.launch(g, p, xy.p, q0, f.p, q0, nullptr, SwingArgs{}, s);
         BGL_CUDA(cudaEventRecord(e[3], s));
         BGL_CUDA(cudaEventSynchronize(e[3]));
         BGL_CUDA(cudaEventElapsedTime(&ms_fmm, e[0], e[1]));
@@ -499,10 +771,11 @@ struct Fa2Run {
     const bgl_params *p;
     float2 *xy;
     int64_t qbase, c0, c1, q0, q1;
-    DevBuf<Tile> ex_tiles, red_tiles;
-    int ex_r = 2;                 // targets per thread of the exact tiles
-    DevBuf<int64_t> red_tile_off;
-    int n_ex_tiles = 0, n_red_tiles = 0;
+    ExactSum exact;
+    DevBuf<Tile> red_tiles;       // swing/traction tiles of the FMM's components
+    DevBuf<int32_t> red_tile_off, ex_tile_off;
+    int n_red_tiles = 0;
+    int64_t q_fmm = 0;            // end of the last FMM component (the attraction kernel's range is [q0, q_fmm))
     DevBuf<float2> f, fprev, fa;
     DevBuf<double2> partial;
     DevBuf<double> sg;
@@ -527,7 +800,7 @@ struct Fa2Run {
         if (!fused) {
             const char *v = std::getenv("BGL_FUSED_ITERATION");
             if (v && v[0] == '0') return;
-            if (fmm.size() != 1 || n_ex_tiles != 0 || c1 - c0 != 1) return;
+            if (fmm.size() != 1 || exact.n_blk != 0 || c1 - c0 != 1) return;
         }
         FmmFuse fz;
         fz.fprev = fprev.p;
@@ -550,36 +823,42 @@ struct Fa2Run {
         q0 = g->h_comp_off[c0];
         q1 = g->h_comp_off[c1];
         const int64_t n = q1 - q0;
-        std::vector<Tile> ex, red;
+        std::vector<Tile> red;
         std::vector<int64_t> ex_comps;
-        std::vector<int64_t> roff(1, 0);
+        std::vector<int32_t> roff(1, 0);
+        q_fmm = q0;
         for (int64_t c = c0; c < c1; ++c) {
             int64_t a = g->h_comp_off[c], b = g->h_comp_off[c + 1];
             if (use_fmm_for(g, p, c)) {
                 fmm.push_back(fmm_create(g, p, c));
                 fmm_comp.push_back(c);
+                q_fmm = b;
+                for (int64_t t = a; t < b; t += RED_TILE)
+                    red.push_back(Tile{(int32_t)(c - c0), 0, t, std::min(b, t + RED_TILE)});
             } else {
                 ex_comps.push_back(c);
             }
-            for (int64_t t = a; t < b; t += RED_TILE) red.push_back(Tile{(int32_t)(c - c0), 0, t, std::min(b, t + RED_TILE)});
-            roff.push_back((int64_t)red.size());
+            roff.push_back((int32_t)red.size());
         }
-        ex_r = exact_tile_choice(g, p, ex_comps);
-        ex = exact_tiles(g, c0, ex_comps, ex_r);
-        n_ex_tiles = (int)ex.size();
+        if (!ex_comps.empty()) {
+            exact.make(g, c0, c1, ex_comps);
+            ex_tile_off.reset(A, exact.tile_off.size());
+            BGL_CUDA(cudaMemcpyAsync(ex_tile_off.p, exact.tile_off.data(), sizeof(int32_t) * exact.tile_off.size(),
+                                     cudaMemcpyHostToDevice, s));
+        }
         n_red_tiles = (int)red.size();
-        ex_tiles.reset(A, ex.size());
-        red_tiles.reset(A, red.size());
-        red_tile_off.reset(A, roff.size());
-        if (!ex.empty())
-            BGL_CUDA(cudaMemcpyAsync(ex_tiles.p, ex.data(), sizeof(Tile) * ex.size(), cudaMemcpyHostToDevice, s));
-        BGL_CUDA(cudaMemcpyAsync(red_tiles.p, red.data(), sizeof(Tile) * red.size(), cudaMemcpyHostToDevice, s));
-        BGL_CUDA(cudaMemcpyAsync(red_tile_off.p, roff.data(), sizeof(int64_t) * roff.size(), cudaMemcpyHostToDevice, s));
-        f.reset(A, n);
+        if (n_red_tiles > 0) {
+            red_tiles.reset(A, red.size());
+            red_tile_off.reset(A, roff.size());
+            BGL_CUDA(cudaMemcpyAsync(red_tiles.p, red.data(), sizeof(Tile) * red.size(), cudaMemcpyHostToDevice, s));
+            BGL_CUDA(cudaMemcpyAsync(red_tile_off.p, roff.data(), sizeof(int32_t) * roff.size(),
+                                     cudaMemcpyHostToDevice, s));
+            partial.reset(A, red.size());
+        }
         fa.reset(A, n);
+        f.reset(A, n);
         fprev.reset(A, n);
         BGL_CUDA(cudaMemsetAsync(fprev.p, 0, sizeof(float2) * n, s));
-        partial.reset(A, red.size());
         std::vector<double> ones(c1 - c0, 1.0);
         sg.reset(A, c1 - c0);
         BGL_CUDA(cudaMemcpyAsync(sg.p, ones.data(), sizeof(double) * ones.size(), cudaMemcpyHostToDevice, s));
@@ -588,18 +867,35 @@ struct Fa2Run {
         iter.reset(A, 1);
         BGL_CUDA(cudaMemsetAsync(iter.p, 0, sizeof(int), s));
         loop.reset(A, 1);
-        // nodes of high degree: chunks of HEAVY_CHUNK adjacency entries
-        DevBuf<int32_t> flag(A, n), fscan(A, n), tot(A, 1);
-        heavy_flag_kernel<<<nblocks(n, 256), 256, 0, s>>>(g->coff.p, q0, n, flag.p);
+        if (!fmm.empty()) heavy_setup();
+        BGL_CUDA(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+        BGL_CUDA(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
+        BGL_CUDA(cudaEventCreateWithFlags(&ev_fa, cudaEventDisableTiming));
+        BGL_CUDA(cudaStreamSynchronize(s));
+    }
+    ~Fa2Run() {
+        for (auto *pl : fmm) fmm_destroy(pl);
+        if (ev_fork) cudaEventDestroy(ev_fork);
+        if (ev_fa) cudaEventDestroy(ev_fa);
+        if (side) cudaStreamDestroy(side);
+    }
+
+    // the FMM components' nodes of high degree: chunks of HEAVY_CHUNK adjacency entries
+    void heavy_setup() {
+        Allocator *A = g->ctx->alloc;
+        cudaStream_t s = g->ctx->stream;
+        const int64_t nf = q_fmm - q0;
+        DevBuf<int32_t> flag(A, nf), fscan(A, nf), tot(A, 1);
+        heavy_flag_kernel<<<nblocks(nf, 256), 256, 0, s>>>(g->coff.p, q0, nf, flag.p);
         BGL_LAUNCH_CHECK();
-        scan_exclusive_i32(g->ctx, flag.p, fscan.p, n, tot.p);
+        scan_exclusive_i32(g->ctx, flag.p, fscan.p, nf, tot.p);
         int32_t nh = 0;
         BGL_CUDA(cudaMemcpyAsync(&nh, tot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         BGL_CUDA(cudaStreamSynchronize(s));
         std::vector<HeavyChunk> hc;
         if (nh > 0) {
             DevBuf<int32_t> heavy(A, nh);
-            heavy_list_kernel<<<nblocks(n, 256), 256, 0, s>>>(flag.p, fscan.p, q0, n, heavy.p);
+            heavy_list_kernel<<<nblocks(nf, 256), 256, 0, s>>>(flag.p, fscan.p, q0, nf, heavy.p);
             BGL_LAUNCH_CHECK();
             DevBuf<int64_t> hrow(A, 2 * (size_t)nh);
             heavy_rows_kernel<<<nblocks(nh, 256), 256, 0, s>>>(heavy.p, g->coff.p, nh, hrow.p);
@@ -625,16 +921,6 @@ struct Fa2Run {
         BGL_CUDA(cudaMemsetAsync(chunk_arrive.p, 0, sizeof(int) * std::max<int32_t>(nh, 1), s));
         if (!hc.empty())
             BGL_CUDA(cudaMemcpyAsync(chunks.p, hc.data(), sizeof(HeavyChunk) * hc.size(), cudaMemcpyHostToDevice, s));
-        BGL_CUDA(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
-        BGL_CUDA(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
-        BGL_CUDA(cudaEventCreateWithFlags(&ev_fa, cudaEventDisableTiming));
-        BGL_CUDA(cudaStreamSynchronize(s));
-    }
-    ~Fa2Run() {
-        for (auto *pl : fmm) fmm_destroy(pl);
-        if (ev_fork) cudaEventDestroy(ev_fork);
-        if (ev_fa) cudaEventDestroy(ev_fa);
-        if (side) cudaStreamDestroy(side);
     }
 
     // device-side failures of the FMM (bounded waits, capacities)
@@ -647,20 +933,35 @@ struct Fa2Run {
         }
     }
 
-    // K1 + K2: f <- F (what 0) or F_rep (what 1).  K2 runs on the side
-    // stream from the start; the repulsion kernels that write f last wait
-    // for it (event ev_fa) and add fa.
-    void forces(int what) {
+    SwingArgs swing_args(double *d_stats) const {
+        SwingArgs a;
+        a.fprev = fprev.p;
+        a.variant = p->swing_variant;
+        a.tau = p->tau;
+        a.partial = partial.p;
+        a.group = nullptr;
+        a.tile_off = red_tile_off.p;
+        a.sg = sg.p;
+        a.counter = counter.p;
+        a.stats = d_stats;
+        a.iter = iter.p;
+        return a;
+    }
+
+    // K1 + K2: f <- F (what 0) or F_rep (what 1).  The FMM's K2 runs on the
+    // side stream from the start; its kernels that write f last wait for it
+    // (event ev_fa) and add fa.  The exact kernel adds its targets' K2 and,
+    // with `sw`, sums their K3.
+    void forces(int what, const SwingArgs *sw = nullptr) {
         cudaStream_t s = g->ctx->stream;
         const bool att = what == 0;
-        if (att) {
+        if (att && !fmm.empty()) {
             BGL_RANGE("ForceAtlas2: attraction and gravity (Section 3.2)");
             BGL_CUDA(cudaEventRecord(ev_fork, s));
             BGL_CUDA(cudaStreamWaitEvent(side, ev_fork, 0));
-            int64_t n = q1 - q0;
-            int64_t nl = nblocks(n, 256);
+            int64_t nl = nblocks(q_fmm - q0, 256);
             attraction_gravity_kernel<<<(unsigned)(nl + n_chunks), 256, 0, side>>>(
-                xy, g->mass.p, g->coff.p, g->cadj.p, q0, q1, qbase, (float)p->kg, chunks.p, nl, chunk_part.p,
+                xy, g->mass.p, g->coff.p, g->cadj.p, q0, q_fmm, qbase, (float)p->kg, chunks.p, nl, chunk_part.p,
                 chunk_arrive.p, fa.p - (q0 - qbase));
             BGL_LAUNCH_CHECK();
             BGL_CUDA(cudaEventRecord(ev_fa, side));
@@ -669,16 +970,20 @@ struct Fa2Run {
             BGL_RANGE("ForceAtlas2: repulsion by the FMM (Section 3.2.1)");
             fmm_repulsion(fmm[k], xy, qbase, f.p, q0, att ? fa.p : nullptr, att ? ev_fa : nullptr);
         }
-        if (att) BGL_CUDA(cudaStreamWaitEvent(s, ev_fa, 0));
-        if (n_ex_tiles > 0) {
+        if (att && !fmm.empty()) BGL_CUDA(cudaStreamWaitEvent(s, ev_fa, 0));
+        if (exact.n_blk > 0) {
             BGL_RANGE("ForceAtlas2: exact repulsion (Section 3.2)");
-            launch_exact(ex_r, n_ex_tiles, ex_tiles.p, g->comp_off.p, c0, xy, g->mass.p, qbase, (float)p->kr,
-                         att ? fa.p - (q0 - qbase) : nullptr, f.p - (q0 - qbase), s);
+            SwingArgs a{};
+            if (sw) {
+                a = *sw;
+                a.tile_off = ex_tile_off.p;
+            }
+            exact.launch(g, p, xy, qbase, f.p, q0, att ? fa.p : nullptr, a, s);
         }
     }
 
-    // one full iteration (K1..K4)
-    void iteration(double *d_stats) {
+    // one full iteration (K1..K4); loop: the device-side loop's control, done by K4
+    void iteration(double *d_stats, const LoopCtl &loop_ctl = LoopCtl{}) {
         BGL_RANGE("ForceAtlas2 iteration: forces, swing/traction, update (Section 3.2)");
         cudaStream_t s = g->ctx->stream;
         if (fused) {
@@ -688,42 +993,27 @@ struct Fa2Run {
             fmm_update_root(fmm[0], xy, qbase, f.p, fprev.p, q0);
             return;
         }
-        forces(0);
-        RedArgs a;
-        a.tiles = red_tiles.p;
-        a.tile_off = red_tile_off.p;
-        a.ncomp = (int)(c1 - c0);
-        a.f = f.p - (q0 - qbase);
-        a.fprev = fprev.p - (q0 - qbase);
-        a.mass = g->mass.p;
-        a.qbase = qbase;
-        a.variant = p->swing_variant;
-        a.tau = p->tau;
-        a.partial = partial.p;
-        a.sg = sg.p;
-        a.counter = counter.p;
-        a.stats = d_stats;
-        a.iter = iter.p;
+        const SwingArgs a = swing_args(d_stats);
+        forces(0, &a);
         {
             BGL_RANGE("ForceAtlas2: swing and traction (Section 3.2)");
-            swing_traction_kernel<<<n_red_tiles, 256, 0, s>>>(a);
-            BGL_LAUNCH_CHECK();
+            if (n_red_tiles > 0) {
+                swing_traction_kernel<<<n_red_tiles, 256, 0, s>>>(a, red_tiles.p, f.p, g->mass.p, q0);
+                BGL_LAUNCH_CHECK();
+            }
         }
         BGL_RANGE("ForceAtlas2: node update (Section 3.2)");
         update_kernel<<<nblocks(q1 - q0, 256), 256, 0, s>>>(f.p - (q0 - qbase), fprev.p - (q0 - qbase), xy,
                                                             g->node_comp.p, sg.p, q0, q1, qbase, c0, (float)p->ks,
-                                                            (float)p->ksmax, g->ctx->d_flag + 1);
+                                                            (float)p->ksmax, g->ctx->d_flag + 1, loop_ctl);
         BGL_LAUNCH_CHECK();
     }
 };
 
 namespace {
 
-// End of a loop iteration: count it and keep looping while below `iters`.
-__global__ void loop_ctrl_kernel(cudaGraphConditionalHandle h, int *count, int iters) {
-    const int k = ++*count;
-    cudaGraphSetConditional(h, k < iters ? 1u : 0u);
-}
+// End of a loop iteration (fused runs, whose last kernel is the FMM's).
+__global__ void loop_ctrl_kernel(LoopCtl loop) { loop_step(loop); }
 
 }  // namespace
 
@@ -839,9 +1129,15 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
         BGL_CUDA(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
         ctx->alloc->forbid = true;
         try {
-            run.iteration(d_stats);
-            loop_ctrl_kernel<<<1, 1, 0, s>>>(h, run.loop.p, iters);
-            BGL_LAUNCH_CHECK();
+            LoopCtl ctl;
+            ctl.h = h;
+            ctl.count = run.loop.p;
+            ctl.iters = iters;
+            run.iteration(d_stats, ctl);
+            if (run.fused) {
+                loop_ctrl_kernel<<<1, 1, 0, s>>>(ctl);
+                BGL_LAUNCH_CHECK();
+            }
         } catch (...) {
             ctx->alloc->forbid = false;
             cudaGraph_t tmp = nullptr;
