@@ -33,6 +33,7 @@ namespace {
 
 constexpr int EX_THREADS = 128, EX_WARPS = EX_THREADS / 32;
 constexpr int EX_STAGE = 1024;                 // sources summed before they enter the compensated total
+constexpr int EX_AHEAD = 8;                    // sources a warp with one target a lane takes together
 constexpr int64_t EX_SPLIT_MAX_N = 1 << 16;    // components up to this size: a block per stage (partial sums in memory)
 #ifndef BGL_EXACT_WIDE_WARPS
 #define BGL_EXACT_WIDE_WARPS 3000              // warps at two targets per lane from which a run takes two
@@ -251,7 +252,7 @@ __device__ void tile_attraction(const ExArgs &a, const ExBlock &b) {
 // took 116 us for 2,821 nodes (6 blocks on 152 SMs).
 template <int R>
 __global__ void __launch_bounds__(EX_THREADS) exact_kernel(ExArgs a) {
-    __shared__ float4 src[EX_STAGE];
+    __shared__ float4 src[EX_STAGE + EX_AHEAD];
     __shared__ double ws[8], wt[8];
     __shared__ bool last;
     constexpr int TT = EX_THREADS * R;
@@ -287,9 +288,32 @@ __global__ void __launch_bounds__(EX_THREADS) exact_kernel(ExArgs a) {
             if (!work) continue;
             float ax[R], ay[R];
             if constexpr (R == 1) {
+                // a warp has a scheduler to itself here: eight sources at a
+                // time, their reciprocals in flight together, the next eight
+                // loaded meanwhile; the sums in source order
                 ax[0] = ay[0] = 0.f;
-#pragma unroll 8
-                for (int j = 0; j < cnt; ++j) p2p_pair(zx[0], zy[0], src[j], ax[0], ay[0]);
+                constexpr int B = EX_AHEAD;
+                float4 q[B];
+#pragma unroll
+                for (int k = 0; k < B; ++k) q[k] = src[k];
+                int j = 0;
+                for (; j + B <= cnt; j += B) {
+                    float dx[B], dy[B], w[B];
+#pragma unroll
+                    for (int k = 0; k < B; ++k) {
+                        dx[k] = zx[0] - q[k].x;
+                        dy[k] = zy[0] - q[k].y;
+                        w[k] = q[k].z * rcp_approx(fmaf(dx[k], dx[k], fmaf(dy[k], dy[k], 1e-30f)));
+                    }
+#pragma unroll
+                    for (int k = 0; k < B; ++k) q[k] = src[j + B + k];
+#pragma unroll
+                    for (int k = 0; k < B; ++k) {
+                        ax[0] = fmaf(w[k], dx[k], ax[0]);
+                        ay[0] = fmaf(w[k], dy[k], ay[0]);
+                    }
+                }
+                for (; j < cnt; ++j) p2p_pair(zx[0], zy[0], src[j], ax[0], ay[0]);
             } else {
                 float2 nzx[R / 2], nzy[R / 2], gx[R / 2], gy[R / 2];
 #pragma unroll
@@ -575,12 +599,16 @@ __device__ __forceinline__ void loop_step(const LoopCtl &l) {
     cudaGraphSetConditional(l.h, k < l.iters ? 1u : 0u);
 }
 
-// K4: node speeds and the position update; the first thread also steps the loop
+// K4: node speeds and the position update; the first thread also steps the
+// loop (LOOP; a kernel without it can be profiled)
+template <bool LOOP>
 __global__ void update_kernel(const float2 *__restrict__ f, float2 *__restrict__ fprev, float2 *__restrict__ xy,
                               const int32_t *__restrict__ node_comp, const double *__restrict__ sg, int64_t q0,
                               int64_t q1, int64_t qbase, int64_t c0, float ks, float ksmax, int *bad,
                               LoopCtl loop) {
-    if (loop.count && blockIdx.x == 0 && threadIdx.x == 0) loop_step(loop);
+    if constexpr (LOOP) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) loop_step(loop);
+    }
     int64_t q = q0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= q1) return;
     const float2 F = f[q - qbase], P = fprev[q - qbase];
@@ -1003,9 +1031,9 @@ struct Fa2Run {
             }
         }
         BGL_RANGE("ForceAtlas2: node update (Section 3.2)");
-        update_kernel<<<nblocks(q1 - q0, 256), 256, 0, s>>>(f.p - (q0 - qbase), fprev.p - (q0 - qbase), xy,
-                                                            g->node_comp.p, sg.p, q0, q1, qbase, c0, (float)p->ks,
-                                                            (float)p->ksmax, g->ctx->d_flag + 1, loop_ctl);
+        (loop_ctl.count ? update_kernel<true> : update_kernel<false>)<<<nblocks(q1 - q0, 256), 256, 0, s>>>(
+            f.p - (q0 - qbase), fprev.p - (q0 - qbase), xy, g->node_comp.p, sg.p, q0, q1, qbase, c0, (float)p->ks,
+            (float)p->ksmax, g->ctx->d_flag + 1, loop_ctl);
         BGL_LAUNCH_CHECK();
     }
 };
@@ -1090,11 +1118,53 @@ static void run_iterations_host(Fa2Run &run, int iters, double *d_stats, const S
     if (ctx->h_flag[1]) fail(BGL_ENUMERIC, "fa2: a position became non-finite");
 }
 
+// Iterations per turn of the device-side loop.  A turn costs some 4 us beside
+// its kernels: of a 25 us iteration of exact sums four to a turn save 3.5 us
+// (871 nodes: 24.8 us an iteration with one, 22.6 two, 21.5 four, 20.9 eight),
+// but every captured iteration also costs the instantiation of its kernels:
+// an FMM iteration of nineteen takes 30 us longer to instantiate than it saves
+// in ten turns (8,888 nodes: 106.0 and 104.0 us an iteration with one and two).
+static int loop_unroll(const Fa2Run &run) { return run.fmm.empty() ? 4 : 1; }
+
+// `n` iterations captured on s into graph `into` (null: a new graph, which
+// is returned); loop: stepped by the last one.  Adds the kernels to `kernels`.
+static cudaGraph_t capture_iterations(Fa2Run &run, double *d_stats, int n, cudaGraph_t into, const LoopCtl &loop,
+                                      int64_t &kernels) {
+    bgl_ctx *ctx = run.g->ctx;
+    cudaStream_t s = ctx->stream;
+    const int64_t before = launch_count();
+    if (into) {
+        BGL_CUDA(cudaStreamBeginCaptureToGraph(s, into, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    } else {
+        BGL_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    }
+    ctx->alloc->forbid = true;
+    cudaGraph_t captured = nullptr;
+    try {
+        for (int k = 0; k < n; ++k) run.iteration(d_stats, k + 1 < n ? LoopCtl{} : loop);
+        if (run.fused && loop.count) {
+            loop_ctrl_kernel<<<1, 1, 0, s>>>(loop);
+            BGL_LAUNCH_CHECK();
+        }
+    } catch (...) {
+        ctx->alloc->forbid = false;
+        cudaStreamEndCapture(s, &captured);
+        if (captured && !into) cudaGraphDestroy(captured);
+        throw;
+    }
+    ctx->alloc->forbid = false;
+    BGL_CUDA(cudaStreamEndCapture(s, &captured));
+    // captured launches run only when the graph does
+    kernels = launch_count() - before;
+    count_launches(-kernels);
+    return captured;
+}
+
 // All `iters` iterations of `run` in one graph launch: the graph holds a
-// WHILE conditional node whose body is one captured iteration followed by a
-// one-thread kernel that counts the iterations and clears the condition
-// after the last, so the loop runs on the device without the host.
-// Nothing may allocate while the capture is open.
+// WHILE conditional node whose body is some captured iterations, the last
+// kernel of which counts them and clears the condition after the last, so
+// the loop runs on the device without the host; the iterations that are left
+// over come before it.  Nothing may allocate while a capture is open.
 static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWork &side = SideWork()) {
     bgl_ctx *ctx = run.g->ctx;
     cudaStream_t s = ctx->stream;
@@ -1115,48 +1185,29 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
     BGL_CUDA(cudaGraphCreate(&graph, 0));
     int64_t kernels = 0;
     try {
-        cudaGraphConditionalHandle h;
-        BGL_CUDA(cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault));
-        cudaGraphNodeParams cp = {};
-        cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = h;
-        cp.conditional.type = cudaGraphCondTypeWhile;
-        cp.conditional.size = 1;
-        cudaGraphNode_t cnode;
-        BGL_CUDA(cudaGraphAddNode(&cnode, graph, nullptr, nullptr, 0, &cp));
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
-        const int64_t before = launch_count();
-        BGL_CUDA(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-        ctx->alloc->forbid = true;
-        try {
-            LoopCtl ctl;
-            ctl.h = h;
-            ctl.count = run.loop.p;
-            ctl.iters = iters;
-            run.iteration(d_stats, ctl);
-            if (run.fused) {
-                loop_ctrl_kernel<<<1, 1, 0, s>>>(ctl);
-                BGL_LAUNCH_CHECK();
-            }
-        } catch (...) {
-            ctx->alloc->forbid = false;
-            cudaGraph_t tmp = nullptr;
-            cudaStreamEndCapture(s, &tmp);
-            throw;
+        const int unroll = loop_unroll(run), turns = iters / unroll, rest = iters - turns * unroll;
+        cudaGraphNode_t rnode = nullptr;
+        if (rest > 0) {
+            cudaGraph_t child = capture_iterations(run, d_stats, rest, nullptr, LoopCtl{}, kernels);
+            const cudaError_t e = cudaGraphAddChildGraphNode(&rnode, graph, nullptr, 0, child);
+            cudaGraphDestroy(child);
+            BGL_CUDA(e);
         }
-        ctx->alloc->forbid = false;
-        cudaGraph_t captured = nullptr;
-        BGL_CUDA(cudaStreamEndCapture(s, &captured));
-        // captured launches run only when the graph does
-        count_launches(before - launch_count());
-        size_t nn = 0;
-        BGL_CUDA(cudaGraphGetNodes(body, nullptr, &nn));
-        std::vector<cudaGraphNode_t> nodes(nn);
-        if (nn) BGL_CUDA(cudaGraphGetNodes(body, nodes.data(), &nn));
-        for (auto nd : nodes) {
-            cudaGraphNodeType t;
-            BGL_CUDA(cudaGraphNodeGetType(nd, &t));
-            if (t == cudaGraphNodeTypeKernel) ++kernels;
+        if (turns > 0) {
+            LoopCtl ctl;
+            BGL_CUDA(cudaGraphConditionalHandleCreate(&ctl.h, graph, 1, cudaGraphCondAssignDefault));
+            ctl.count = run.loop.p;
+            ctl.iters = turns;
+            cudaGraphNodeParams cp = {};
+            cp.type = cudaGraphNodeTypeConditional;
+            cp.conditional.handle = ctl.h;
+            cp.conditional.type = cudaGraphCondTypeWhile;
+            cp.conditional.size = 1;
+            cudaGraphNode_t cnode;
+            BGL_CUDA(cudaGraphAddNode(&cnode, graph, rnode ? &rnode : nullptr, nullptr, rnode ? 1 : 0, &cp));
+            int64_t per_turn = 0;
+            capture_iterations(run, d_stats, unroll, cp.conditional.phGraph_out[0], ctl, per_turn);
+            kernels += per_turn * turns;
         }
         if (side) {
             // the side work, captured on the run's side stream (it may fork
@@ -1186,7 +1237,7 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
         throw;
     }
     cudaGraphDestroy(graph);
-    count_launches(kernels * iters);
+    count_launches(kernels);
     try {
         if (run.fused) fmm_root(run.fmm[0], run.xy, run.qbase);
         BGL_CUDA(cudaGraphLaunch(exec, s));
