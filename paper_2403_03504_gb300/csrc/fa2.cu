@@ -33,7 +33,6 @@ namespace {
 
 constexpr int EX_THREADS = 128, EX_WARPS = EX_THREADS / 32;
 constexpr int EX_STAGE = 1024;                 // sources summed before they enter the compensated total
-constexpr int EX_AHEAD = 8;                    // sources a warp with one target a lane takes together
 constexpr int64_t EX_SPLIT_MAX_N = 1 << 16;    // components up to this size: a block per stage (partial sums in memory)
 #ifndef BGL_EXACT_WIDE_WARPS
 #define BGL_EXACT_WIDE_WARPS 3000              // warps at two targets per lane from which a run takes two
@@ -252,7 +251,7 @@ __device__ void tile_attraction(const ExArgs &a, const ExBlock &b) {
 // took 116 us for 2,821 nodes (6 blocks on 152 SMs).
 template <int R>
 __global__ void __launch_bounds__(EX_THREADS) exact_kernel(ExArgs a) {
-    __shared__ float4 src[EX_STAGE + EX_AHEAD];
+    __shared__ float4 src[EX_STAGE + P2P_AHEAD];
     __shared__ double ws[8], wt[8];
     __shared__ bool last;
     constexpr int TT = EX_THREADS * R;
@@ -288,32 +287,9 @@ __global__ void __launch_bounds__(EX_THREADS) exact_kernel(ExArgs a) {
             if (!work) continue;
             float ax[R], ay[R];
             if constexpr (R == 1) {
-                // a warp has a scheduler to itself here: eight sources at a
-                // time, their reciprocals in flight together, the next eight
-                // loaded meanwhile; the sums in source order
                 ax[0] = ay[0] = 0.f;
-                constexpr int B = EX_AHEAD;
-                float4 q[B];
-#pragma unroll
-                for (int k = 0; k < B; ++k) q[k] = src[k];
-                int j = 0;
-                for (; j + B <= cnt; j += B) {
-                    float dx[B], dy[B], w[B];
-#pragma unroll
-                    for (int k = 0; k < B; ++k) {
-                        dx[k] = zx[0] - q[k].x;
-                        dy[k] = zy[0] - q[k].y;
-                        w[k] = q[k].z * rcp_approx(fmaf(dx[k], dx[k], fmaf(dy[k], dy[k], 1e-30f)));
-                    }
-#pragma unroll
-                    for (int k = 0; k < B; ++k) q[k] = src[j + B + k];
-#pragma unroll
-                    for (int k = 0; k < B; ++k) {
-                        ax[0] = fmaf(w[k], dx[k], ax[0]);
-                        ay[0] = fmaf(w[k], dy[k], ay[0]);
-                    }
-                }
-                for (; j < cnt; ++j) p2p_pair(zx[0], zy[0], src[j], ax[0], ay[0]);
+                p2p_chain(zx[0], zy[0], src, cnt,
+                          [](float dx, float dy) { return fmaf(dx, dx, fmaf(dy, dy, 1e-30f)); }, ax[0], ay[0]);
             } else {
                 float2 nzx[R / 2], nzy[R / 2], gx[R / 2], gy[R / 2];
 #pragma unroll

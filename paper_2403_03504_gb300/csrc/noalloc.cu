@@ -13,24 +13,32 @@
 //
 // The kernels are variants of the ones in fa2.cu that need no host-built
 // tile list and no per-call buffers: one component, targets tiled by block
-// index, hub rows summed by the node's own thread.  The formulas of every
-// force term, of the swing/traction sums and of the update are the same;
-// the order and precision of the sums differ (here every thread sums its
-// swing/traction terms in FP64 over tiles of 2,048 nodes and a hub's
-// attraction in one loop, where fa2.cu sums in FP32 within a warp over tiles
-// of 1,024 nodes and splits hub rows into 2,048-entry chunks), so the two
-// agree within rounding, not bitwise.  A position that becomes non-finite
-// sets the context's d_flag[2], which bgl_ctx_sync reports.
+// index, the stages of a tile's sources spread over a thread-block cluster
+// whose blocks hand their sums over in distributed shared memory.  The
+// formulas of every force term, of the swing/traction sums and of the update
+// are the same; the order and precision of the sums differ (here every thread
+// sums its swing/traction terms in FP64 over tiles of 2,048 nodes and a hub's
+// attraction is summed entry after entry, where fa2.cu sums in FP32 within a
+// warp over tiles of 256 nodes and splits hub rows into 2,048-entry chunks),
+// so the two agree within rounding, not bitwise.  A position that becomes
+// non-finite sets the context's d_flag[2], which bgl_ctx_sync reports.
+#include <algorithm>
+
+#include <cooperative_groups.h>
+
 #include "bgl_internal.cuh"
+#include "p2p.cuh"
 
 namespace bgl {
 
 namespace {
 
-constexpr int NA_THREADS = 256;
-constexpr int NA_R = 2;                           // targets per thread
-constexpr int NA_TILE = NA_THREADS * NA_R;        // targets per block
+namespace cg = cooperative_groups;
+
+constexpr int NA_TILE = 128;                      // targets per cluster, one a thread
+constexpr int NA_CLUSTER = 8;                     // blocks per cluster (the portable maximum)
 constexpr int NA_STILE = 1024;                    // sources per shared-memory stage
+constexpr int NA_LANE_DEG = 8;                    // nodes up to this degree: attraction by one lane
 constexpr int NA_RED_TILE = 2048;                 // nodes per swing/traction tile
 constexpr int64_t NA_MAX_NODES = BGL_NOALLOC_MAX_NODES;
 constexpr int NA_MAX_TILES = (int)(NA_MAX_NODES / NA_RED_TILE);
@@ -43,87 +51,134 @@ constexpr size_t NOALLOC_SCRATCH_BYTES = NA_COUNTER_BYTES + sizeof(double2) * NA
 // cudaGetSymbolAddress (noalloc_scratch_address, stored in the context).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
 
-__device__ __forceinline__ float na_rcp(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// repulsion of targets [blockIdx.x * NA_TILE, ...) from all n nodes
-__global__ void __launch_bounds__(NA_THREADS) na_repulsion_kernel(const float2 *__restrict__ xy,
-                                                                 const float *__restrict__ mass, int64_t n, float kr,
-                                                                 float2 *__restrict__ f) {
-    __shared__ float4 src[NA_STILE];
-    const int64_t t0 = (int64_t)blockIdx.x * NA_TILE;
-    float xi[NA_R], yi[NA_R], sx[NA_R], sy[NA_R], cx[NA_R], cy[NA_R];
+// Forces of the cluster's NA_TILE targets: repulsion from all n nodes, plus
+// attraction and gravity.
+//
+// A target's repulsion is a chain over its sources (each 1,024-source stage's
+// sum enters a compensated total), so the cluster's blocks take the stages in
+// turn; block 0 adds their sums in order out of the others' shared memory
+// (two buffers, so one barrier a round).  A cluster has a block per stage and
+// one more, up to NA_CLUSTER: on a small component more would only share SMs
+// with the ones that work.  The blocks without a stage, or all of them,
+// share the attraction, entry after entry:
+// a lane for a node of few entries, for the others the warp loads 32 entries
+// at a time and adds them in order through shuffles.  No memory is needed
+// beyond the blocks' own.  One block per 512 targets with all stages, and a
+// kernel with one thread per node for the attraction, took 99.6 and 15.5 us
+// for 2,821 nodes.
+__global__ void __launch_bounds__(NA_TILE)
+    na_force_kernel(const float2 *__restrict__ xy, const float *__restrict__ mass, const int64_t *__restrict__ off,
+                    const int32_t *__restrict__ adj, int64_t n, float kr, float kg, float2 *__restrict__ f) {
+    __shared__ float4 src[NA_STILE + P2P_AHEAD];
+    __shared__ float2 part[2][NA_TILE];
+    __shared__ float2 satt[NA_TILE];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), blocks = (int)cluster.num_blocks();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t t0 = (int64_t)(blockIdx.x / (unsigned)blocks) * NA_TILE;
+    const int64_t stages = (n + NA_STILE - 1) / NA_STILE;
+    // attraction: shared by the blocks without a stage, or by all of them
+    const int first = stages < blocks ? (int)stages : 0;
+    const int share = (NA_TILE + blocks - first - 1) / (blocks - first);
+    if (rank >= first) {
+        const int per_warp = (share + NA_TILE / 32 - 1) / (NA_TILE / 32);
+        const int node = warp * per_warp + lane;         // lanes below per_warp own a node
+        const int i = (rank - first) * share + node;
+        const int64_t q = t0 + i;
+        const bool own = lane < per_warp && node < share && i < NA_TILE, ok = own && q < n;
+        const int64_t e0 = ok ? off[q] : 0, deg = ok ? off[q + 1] - e0 : 0;
+        const float2 p = ok ? xy[q] : make_float2(0.f, 0.f);
+        float ax = 0.f, ay = 0.f;
+        if (deg <= NA_LANE_DEG) {
+            float2 o[NA_LANE_DEG];
 #pragma unroll
-    for (int r = 0; r < NA_R; ++r) {
-        int64_t q = t0 + threadIdx.x + r * NA_THREADS;
-        float2 p = q < n ? xy[q] : make_float2(0.f, 0.f);
-        xi[r] = p.x;
-        yi[r] = p.y;
-        sx[r] = sy[r] = cx[r] = cy[r] = 0.f;
-    }
-    for (int64_t s0 = 0; s0 < n; s0 += NA_STILE) {
-        const int cnt = (int)(n - s0 < NA_STILE ? n - s0 : NA_STILE);
-        __syncthreads();
-        for (int k = threadIdx.x; k < cnt; k += NA_THREADS) {
-            float2 p = xy[s0 + k];
-            src[k] = make_float4(p.x, p.y, mass[s0 + k], 0.f);
-        }
-        __syncthreads();
-        float ax[NA_R], ay[NA_R];
+            for (int e = 0; e < NA_LANE_DEG; ++e) o[e] = e < deg ? xy[adj[e0 + e]] : p;
 #pragma unroll
-        for (int r = 0; r < NA_R; ++r) ax[r] = ay[r] = 0.f;
-#pragma unroll 4
-        for (int j = 0; j < cnt; ++j) {
-            const float4 s = src[j];
-#pragma unroll
-            for (int r = 0; r < NA_R; ++r) {
-                float dx = xi[r] - s.x, dy = yi[r] - s.y;
-                float r2 = fmaf(dx, dx, dy * dy);
-                float w = s.z * na_rcp(fmaxf(r2, 1e-30f));   // the node itself adds 0
-                ax[r] = fmaf(w, dx, ax[r]);
-                ay[r] = fmaf(w, dy, ay[r]);
+            for (int e = 0; e < NA_LANE_DEG; ++e) {
+                if (e < deg) {
+                    ax -= p.x - o[e].x;
+                    ay -= p.y - o[e].y;
+                }
             }
         }
+        unsigned more = __ballot_sync(0xffffffffu, deg > NA_LANE_DEG);
+        while (more) {
+            const int l = __ffs(more) - 1;
+            more &= more - 1;
+            const int64_t f0 = __shfl_sync(0xffffffffu, e0, l), d = __shfl_sync(0xffffffffu, deg, l);
+            const float px = __shfl_sync(0xffffffffu, p.x, l), py = __shfl_sync(0xffffffffu, p.y, l);
+            float sx = 0.f, sy = 0.f;
+            constexpr int C = 4;                         // loads of four rounds in flight
+            for (int64_t c0 = 0; c0 < d; c0 += 32 * C) {
+                float2 t[C];
 #pragma unroll
-        for (int r = 0; r < NA_R; ++r) {   // compensated running total of the stage sums
-            float y = ax[r] - cx[r];
-            float s = sx[r] + y;
-            cx[r] = (s - sx[r]) - y;
-            sx[r] = s;
-            y = ay[r] - cy[r];
-            s = sy[r] + y;
-            cy[r] = (s - sy[r]) - y;
-            sy[r] = s;
+                for (int c = 0; c < C; ++c) {
+                    const int64_t e = c0 + c * 32 + lane;
+                    const float2 o = e < d ? xy[adj[f0 + e]] : make_float2(px, py);
+                    t[c] = make_float2(px - o.x, py - o.y);
+                }
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const int m = (int)min((int64_t)32, d - c0 - c * 32);
+#pragma unroll 8
+                    for (int j = 0; j < m; ++j) {
+                        sx -= __shfl_sync(0xffffffffu, t[c].x, j);
+                        sy -= __shfl_sync(0xffffffffu, t[c].y, j);
+                    }
+                }
+            }
+            if (lane == l) {
+                ax = sx;
+                ay = sy;
+            }
+        }
+        if (own) satt[node] = make_float2(ax, ay);
+    }
+    const int64_t q = t0 + threadIdx.x;
+    const float2 z = q < n ? xy[q] : make_float2(0.f, 0.f);
+    float sx = 0.f, sy = 0.f, cx = 0.f, cy = 0.f;        // block 0: the running total
+    int buf = 0;
+    for (int64_t k0 = 0; k0 < stages; k0 += blocks, buf ^= 1) {
+        const int64_t s0 = (k0 + rank) * NA_STILE;
+        const int cnt = (int)(s0 >= n ? 0 : (n - s0 < NA_STILE ? n - s0 : NA_STILE));
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < NA_STILE / NA_TILE; ++k) {
+            const int j = k * NA_TILE + threadIdx.x;
+            if (j < cnt) {
+                const float2 p = xy[s0 + j];
+                src[j] = make_float4(p.x, p.y, mass[s0 + j], 0.f);
+            }
+        }
+        __syncthreads();
+        float ax = 0.f, ay = 0.f;
+        // (the node itself adds 0)
+        p2p_chain(z.x, z.y, src, cnt, [](float dx, float dy) { return fmaxf(fmaf(dx, dx, dy * dy), 1e-30f); }, ax, ay);
+        part[buf][threadIdx.x] = make_float2(ax, ay);
+        cluster.sync();
+        if (rank == 0) {
+            const int m = (int)(stages - k0 < blocks ? stages - k0 : blocks);
+            for (int r = 0; r < m; ++r) {                // compensated running total of the stage sums
+                const float2 v = cluster.map_shared_rank(&part[0][0], r)[buf * NA_TILE + threadIdx.x];
+                float y = v.x - cx;
+                float t = sx + y;
+                cx = (t - sx) - y;
+                sx = t;
+                y = v.y - cy;
+                t = sy + y;
+                cy = (t - sy) - y;
+                sy = t;
+            }
         }
     }
-#pragma unroll
-    for (int r = 0; r < NA_R; ++r) {
-        int64_t q = t0 + threadIdx.x + r * NA_THREADS;
-        if (q >= n) continue;
-        float km = kr * mass[q];
-        f[q] = make_float2(km * sx[r], km * sy[r]);
+    if (rank == 0 && q < n) {
+        const float m = mass[q], km = kr * m;
+        const float2 a = cluster.map_shared_rank(&satt[0], first + threadIdx.x / share)[threadIdx.x % share];
+        const float2 fr = make_float2(__fmul_rn(km, sx), __fmul_rn(km, sy));   // rounded before the attraction
+        const float kgm = kg * m;
+        f[q] = make_float2((fr.x + a.x) - kgm * z.x, (fr.y + a.y) - kgm * z.y);
     }
-}
-
-// attraction and gravity added to f, one thread per node
-__global__ void na_attraction_gravity_kernel(const float2 *__restrict__ xy, const float *__restrict__ mass,
-                                             const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                                             int64_t n, float kg, float2 *__restrict__ f) {
-    int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    float2 p = xy[q];
-    float ax = 0.f, ay = 0.f;
-    for (int64_t e = off[q]; e < off[q + 1]; ++e) {
-        float2 o = xy[adj[e]];
-        ax -= p.x - o.x;
-        ay -= p.y - o.y;
-    }
-    float km = kg * mass[q];
-    float2 fr = f[q];
-    f[q] = make_float2((fr.x + ax) - km * p.x, (fr.y + ay) - km * p.y);
+    cluster.sync();                                      // no block leaves while block 0 reads its memory
 }
 
 // swing / traction partial sums per tile into the static scratch; the last
@@ -137,15 +192,26 @@ __global__ void na_swing_traction_kernel(const float2 *__restrict__ f, const flo
     double2 *partial = reinterpret_cast<double2 *>(scratch + NA_COUNTER_BYTES);
     const int64_t t0 = (int64_t)blockIdx.x * NA_RED_TILE;
     const int64_t t1 = t0 + NA_RED_TILE < n ? t0 + NA_RED_TILE : n;
+    // the tile's loads in flight together, then each thread's terms in order
+    constexpr int PER = NA_RED_TILE / 256;
+    float2 F[PER], P[PER];
+    float m[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int64_t q = t0 + k * 256 + threadIdx.x;
+        F[k] = q < t1 ? f[q] : make_float2(0.f, 0.f);
+        P[k] = q < t1 ? fprev[q] : make_float2(0.f, 0.f);
+        m[k] = variant == 1 && q < t1 ? mass[q] : 0.f;
+    }
     double sw = 0.0, tr = 0.0;
-    for (int64_t q = t0 + threadIdx.x; q < t1; q += blockDim.x) {
-        float2 F = f[q], P = fprev[q];
-        float s = sqrtf((F.x - P.x) * (F.x - P.x) + (F.y - P.y) * (F.y - P.y));
-        float u = sqrtf((F.x + P.x) * (F.x + P.x) + (F.y + P.y) * (F.y + P.y));
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (t0 + k * 256 + (int64_t)threadIdx.x >= t1) break;
+        const float s = sqrtf((F[k].x - P[k].x) * (F[k].x - P[k].x) + (F[k].y - P[k].y) * (F[k].y - P[k].y));
+        const float u = sqrtf((F[k].x + P[k].x) * (F[k].x + P[k].x) + (F[k].y + P[k].y) * (F[k].y + P[k].y));
         if (variant == 1) {
-            float m = mass[q];
-            sw += (double)m * s;
-            tr += 0.5 * (double)m * u;
+            sw += (double)m[k] * s;
+            tr += 0.5 * (double)m[k] * u;
         } else {
             sw += s;
             tr += u;
@@ -173,13 +239,17 @@ __global__ void na_swing_traction_kernel(const float2 *__restrict__ f, const flo
         last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!last || threadIdx.x != 0) return;
+    if (!last) return;
     __threadfence();
+    // the tiles' sums fetched together, then added in order
+    __shared__ double2 tiles[NA_MAX_TILES];
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) tiles[k] = __ldcg(&partial[k]);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     double swg = 0.0, trc = 0.0;
     for (unsigned k = 0; k < gridDim.x; ++k) {
-        double2 v = __ldcg(&partial[k]);
-        swg += v.x;
-        trc += v.y;
+        swg += tiles[k].x;
+        trc += tiles[k].y;
     }
     double g = *sg;
     double s_new = swg > 0.0 ? tau * trc / swg : 1.5 * g;
@@ -189,7 +259,10 @@ __global__ void na_swing_traction_kernel(const float2 *__restrict__ f, const flo
 }
 
 __global__ void na_update_kernel(const float2 *__restrict__ f, float2 *__restrict__ fprev, float2 *__restrict__ xy,
-                                 const double *__restrict__ sg, int64_t n, float ks, float ksmax, int *bad) {
+                                 const double *__restrict__ sg, int64_t n, float ks, float ksmax, int *bad,
+                                 unsigned char *scratch) {
+    // the arrival counter of the next call starts at zero whatever ran before
+    if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<unsigned *>(scratch) = 0u;
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
     float2 F = f[q], P = fprev[q];
@@ -229,17 +302,25 @@ void fa2_iteration_noalloc(bgl_ctx *c, int64_t n, const int64_t *d_off, const in
     unsigned char *scratch = c->noalloc_scratch;
     BGL_REQUIRE(scratch != nullptr, "noalloc: the context has no scratch address");
     cudaStream_t s = c->stream;
-    // the arrival counter must start at zero; the partial sums are overwritten
-    BGL_CUDA(cudaMemsetAsync(scratch, 0, sizeof(unsigned), s));
-    na_repulsion_kernel<<<na_blocks(n, NA_TILE), NA_THREADS, 0, s>>>(d_xy, d_mass, n, (float)p->kr, d_f);
-    BGL_LAUNCH_CHECK();
-    na_attraction_gravity_kernel<<<na_blocks(n, 256), 256, 0, s>>>(d_xy, d_mass, d_off, d_adj, n, (float)p->kg, d_f);
+    const unsigned blocks = (unsigned)std::min<int64_t>(NA_CLUSTER, (n + NA_STILE - 1) / NA_STILE + 1);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(na_blocks(n, NA_TILE) * blocks);
+    cfg.blockDim = dim3(NA_TILE);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    BGL_CUDA(cudaLaunchKernelEx(&cfg, na_force_kernel, (const float2 *)d_xy, d_mass, d_off, d_adj, n, (float)p->kr,
+                                (float)p->kg, d_f));
     BGL_LAUNCH_CHECK();
     na_swing_traction_kernel<<<na_blocks(n, NA_RED_TILE), 256, 0, s>>>(d_f, d_fprev, d_mass, n, p->swing_variant,
                                                                        p->tau, d_sg, scratch);
     BGL_LAUNCH_CHECK();
     na_update_kernel<<<na_blocks(n, 256), 256, 0, s>>>(d_f, d_fprev, d_xy, d_sg, n, (float)p->ks, (float)p->ksmax,
-                                                       c->d_flag + 2);
+                                                       c->d_flag + 2, scratch);
     BGL_LAUNCH_CHECK();
 }
 

@@ -39,4 +39,67 @@ __device__ __forceinline__ void p2p_pair2(float2 nzx, float2 nzy, const float4 &
     gy = __ffma2_rn(w, dy, gy);
 }
 
+// Sources a warp takes together in p2p_chain; src holds this many readable
+// entries past the last source.
+constexpr int P2P_AHEAD = 8;
+
+// f += the pairs of one target with src[0 .. cnt) in order, for a warp that
+// has its scheduler to itself: the terms of eight sources are worked out
+// (their reciprocals in flight together, the next eight sources loading)
+// while those of the eight before are added, so that neither the MUFU's
+// latency nor the chain of additions is waited for.  Bit for bit the sums of
+// p2p_pair in a loop.  r2_of(dx, dy) is the guarded squared distance.
+template <class R2>
+__device__ __forceinline__ void p2p_chain(float zx, float zy, const float4 *src, int cnt, R2 r2_of, float &fx,
+                                          float &fy) {
+    constexpr int B = P2P_AHEAD;
+    const int full = cnt / B;
+    if (full > 0) {
+        float4 q[B];
+        float dx[B], dy[B], w[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) q[k] = src[k];
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            dx[k] = zx - q[k].x;
+            dy[k] = zy - q[k].y;
+            w[k] = q[k].z * rcp_approx(r2_of(dx[k], dy[k]));
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k) q[k] = src[B + k];
+#pragma unroll 2
+        for (int b = 1; b < full; ++b) {
+            const float4 *next = src + (b + 1) * B;
+            float ex[B], ey[B], v[B];
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                ex[k] = zx - q[k].x;
+                ey[k] = zy - q[k].y;
+                v[k] = q[k].z * rcp_approx(r2_of(ex[k], ey[k]));
+                q[k] = next[k];
+                fx = fmaf(w[k], dx[k], fx);
+                fy = fmaf(w[k], dy[k], fy);
+            }
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                dx[k] = ex[k];
+                dy[k] = ey[k];
+                w[k] = v[k];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            fx = fmaf(w[k], dx[k], fx);
+            fy = fmaf(w[k], dy[k], fy);
+        }
+    }
+    for (int j = full * B; j < cnt; ++j) {
+        const float4 q = src[j];
+        const float dx = zx - q.x, dy = zy - q.y;
+        const float w = q.z * rcp_approx(r2_of(dx, dy));
+        fx = fmaf(w, dx, fx);
+        fy = fmaf(w, dy, fy);
+    }
+}
+
 }  // namespace bgl
