@@ -208,9 +208,13 @@ void layout_device(bgl_graph *g, const bgl_params *p, float *d_xy_out) {
         ks.clear();
     };
     try {
+        // the classes of larger components, whose chains of node steps are the
+        // longest, get their SMs first
+        int lowest = 0, highest = 0;
+        BGL_CUDA(cudaDeviceGetStreamPriorityRange(&lowest, &highest));
         for (int i = 0; i < nk; ++i) {
             cudaStream_t st;
-            BGL_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+            BGL_CUDA(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, std::min(lowest, highest + i)));
             ks.push_back(st);
         }
         for (int i = 0; i < nk + 1; ++i) {
@@ -221,6 +225,7 @@ void layout_device(bgl_graph *g, const bgl_params *p, float *d_xy_out) {
         // small components: Kamada-Kawai, one stream per size class, forked
         // from and joined back to stream s
         SideWork kk_work = [&](cudaStream_t s) {
+            kk_enqueue_distances(kk.get(), s);
             BGL_CUDA(cudaEventRecord(kev[nk], s));
             for (int i = 0; i < nk; ++i) {
                 BGL_CUDA(cudaStreamWaitEvent(ks[i], kev[nk], 0));
