@@ -228,7 +228,7 @@ void radix_sort_u32_ws(bgl_ctx *c, SortWorkspace &ws, uint32_t *keys, uint32_t *
 int sort_workspace_error(bgl_ctx *c, SortWorkspace &ws);
 // The same sort in two halves, so that a caller's kernel can count the digit
 // histograms while it makes the keys: radix_sort_u32_ws_begin clears the
-// counts and returns them; every block of the caller's kernel (256 threads)
+// counts and returns them; every block of the caller's kernel (OS_THREADS)
 // then calls os_block_hist (sort_hist.cuh) on its keys; and
 // radix_sort_u32_ws_scatter runs the four passes.
 struct OsHist {
@@ -237,7 +237,7 @@ struct OsHist {
     unsigned *counter;   // arrival count of the blocks (reset by the last block)
     unsigned *tickets;   // 4 pass tickets
     uint32_t *status;    // 4 x ntiles x 256 look-back status words
-    int64_t ntiles;      // tiles of 256 x 16 keys
+    int64_t ntiles;      // tiles of 4,096 keys
 };
 // With clear = false the caller zeroes hist and tickets in a kernel that
 // runs before its histogram kernel, and each block of the histogram kernel

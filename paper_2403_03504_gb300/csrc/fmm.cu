@@ -410,21 +410,21 @@ __global__ void bbox_kernel(const float2 *__restrict__ xy, int n, float4 *__rest
 
 constexpr int KEY_ITEMS = OS_ITEMS;      // one key block per radix tile
 
-__global__ void __launch_bounds__(256) keys_kernel(const float2 *__restrict__ xy, int n, const Root *__restrict__ root,
+__global__ void __launch_bounds__(OS_THREADS) keys_kernel(const float2 *__restrict__ xy, int n, const Root *__restrict__ root,
                                                    uint32_t *__restrict__ key, uint32_t *__restrict__ idx, OsHist h) {
     const float ox = root->oxf, oy = root->oyf, sc = root->scale;
-    const int i0 = blockIdx.x * 256 * KEY_ITEMS + threadIdx.x;
+    const int i0 = blockIdx.x * OS_TILE + threadIdx.x;
     uint32_t k[KEY_ITEMS];
     unsigned valid = 0;
     float2 p[KEY_ITEMS];
 #pragma unroll
     for (int r = 0; r < KEY_ITEMS; ++r) {
-        const int i = i0 + r * 256;
+        const int i = i0 + r * OS_THREADS;
         p[r] = i < n ? xy[i] : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int r = 0; r < KEY_ITEMS; ++r) {
-        const int i = i0 + r * 256;
+        const int i = i0 + r * OS_THREADS;
         const float fx = floorf((p[r].x - ox) * sc), fy = floorf((p[r].y - oy) * sc);
         const int qx = (int)fminf(fmaxf(fx, 0.f), 65535.f), qy = (int)fminf(fmaxf(fy, 0.f), 65535.f);
         k[r] = spread_bits((uint32_t)qx) | (spread_bits((uint32_t)qy) << 1);
@@ -434,7 +434,6 @@ __global__ void __launch_bounds__(256) keys_kernel(const float2 *__restrict__ xy
             valid |= 1u << r;
         }
     }
-    static_assert(256 * KEY_ITEMS == OS_TILE, "a key block is one radix tile");
     os_clear_status(h, blockIdx.x);
     os_block_hist<KEY_ITEMS>(k, valid, h);
 }
@@ -1597,9 +1596,57 @@ int stage_chunk(const Tree &T, float4 *buf, int &ui, int &off, int ue, int lane)
     return padded;
 }
 
+// The U list staged chunk by chunk (stage_chunk)
+struct Stager {
+    int ui, off, ue;
+    __device__ __forceinline__ Stager(const Tree &, int us, int ue_, int) : ui(us), off(0), ue(ue_) {}
+    __device__ __forceinline__ bool more() const { return ui < ue; }
+    __device__ __forceinline__ int chunk(const Tree &T, float4 *buf, int lane) {
+        return stage_chunk(T, buf, ui, off, ue, lane);
+    }
+};
+
+// The same chunks with the point ranges of 32 U entries fetched at once, a
+// lane each: one chain of dependent loads for a whole list instead of one an
+// entry (twelve of the 32 us that the near field of 225 leaves took).
+struct WideStager {
+    int us, i, nu, off;      // list [us, us + nu), entry i next, `off` of its points done
+    int cs, len;             // the lane's entry of the 32 around i
+    __device__ __forceinline__ void fetch(const Tree &T, int lane) {
+        const int k = (i & ~31) + lane;
+        const int C = k < nu ? T.lidx[us + k] : -1;
+        cs = C >= 0 ? T.bstart[C] : 0;
+        len = C >= 0 ? T.bend[C] - cs : 0;
+    }
+    __device__ __forceinline__ WideStager(const Tree &T, int us_, int ue, int lane)
+        : us(us_), i(0), nu(ue - us_), off(0) {
+        fetch(T, lane);
+    }
+    __device__ __forceinline__ bool more() const { return i < nu; }
+    __device__ __forceinline__ int chunk(const Tree &T, float4 *buf, int lane) {
+        int cnt = 0;
+        while (i < nu && cnt < NEAR_SRC) {
+            const int s = __shfl_sync(0xffffffffu, cs, i & 31), n = __shfl_sync(0xffffffffu, len, i & 31);
+            const int take = min(n - off, NEAR_SRC - cnt);
+            for (int k = lane; k < take; k += 32) cp_async16(buf + cnt + k, T.pts + s + off + k);
+            cnt += take;
+            off += take;
+            if (off == n) {
+                ++i;
+                off = 0;
+                if ((i & 31) == 0 && i < nu) fetch(T, lane);
+            }
+        }
+        cp_async_commit();
+        const int padded = (cnt + NEAR_SPLIT - 1) & ~(NEAR_SPLIT - 1);
+        if (lane < padded - cnt) buf[cnt + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return padded;
+    }
+};
+
 // Pairs of the targets tb + t + 8 r (r < R) of lane (t, h) with the staged
 // sources h, h + NEAR_SPLIT, ...
-template <int R>
+template <int R, class Stage>
 __device__ __forceinline__ void near_tile(const Tree &T, LeafArgs &la, float4 (*buf)[NEAR_SRC], int tb, int ntc,
                                           int us, int ue, int lane) {
     const int t = lane % NEAR_LPS, h = lane / NEAR_LPS;
@@ -1624,11 +1671,12 @@ __device__ __forceinline__ void near_tile(const Tree &T, LeafArgs &la, float4 (*
         gx[k] = gy[k] = make_float2(0.f, 0.f);
     }
 #endif
-    int ui = us, off = 0, cur = 0;
-    int cnt = stage_chunk(T, buf[0], ui, off, ue, lane);
+    Stage stage(T, us, ue, lane);
+    int cur = 0;
+    int cnt = stage.chunk(T, buf[0], lane);
     while (cnt > 0) {
         // next chunk in flight while this one is summed
-        const int nxt = ui < ue ? stage_chunk(T, buf[cur ^ 1], ui, off, ue, lane) : (cp_async_commit(), 0);
+        const int nxt = stage.more() ? stage.chunk(T, buf[cur ^ 1], lane) : (cp_async_commit(), 0);
         cp_async_wait_one();
         __syncwarp();
         const float4 *src = buf[cur] + h;
@@ -1685,56 +1733,83 @@ __device__ __forceinline__ void near_tile(const Tree &T, LeafArgs &la, float4 (*
 // It also empties the child slots of this evaluation's boxes for the next
 // tree (the emit kernel fills only the slots of children that exist; the
 // plan starts with all slots empty).
-__global__ void combine_kernel(LeafArgs la, int n) {
+//
+// Bound by memory latency; a block takes COMBINE_TILES tiles of 256 points,
+// their loads in flight together.  One tile a block (2,173 blocks, each with
+// a fence and an arrival at one counter) took 16.8 us for 556,277 points.
+constexpr int COMBINE_TILES = 4;
+
+__global__ void __launch_bounds__(256) combine_kernel(LeafArgs la, int n) {
     if (aborted(la.e.T.err)) return;
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
     const Tree &T = la.e.T;
-    for (int b = o, B = min(T.levoff[NLEV], T.Bmax); b < B; b += gridDim.x * blockDim.x)
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x, B = min(T.levoff[NLEV], T.Bmax); b < B;
+         b += gridDim.x * blockDim.x)
         T.bchild[b] = make_int4(-1, -1, -1, -1);
-    float sw = 0.f, tr = 0.f;
-    if (o < n) {
+    const int o0 = blockIdx.x * (256 * COMBINE_TILES) + threadIdx.x;
+    float2 nr[COMBINE_TILES], E[COMBINE_TILES], a[COMBINE_TILES], P[COMBINE_TILES];
+    float m[COMBINE_TILES];
+#pragma unroll
+    for (int k = 0; k < COMBINE_TILES; ++k) {
+        const int o = o0 + 256 * k;
+        const bool ok = o < n;
         const int64_t q = la.q0 + o - la.fbase;
-        const float2 nr = la.f[q];
-        const float2 E = la.ef[o];
-        const float km = la.kr * la.mass[o];
-        const float2 a = la.fa ? la.fa[q] : make_float2(0.f, 0.f);
-        const float2 F = make_float2(fmaf(km, nr.x + E.x, a.x), fmaf(km, nr.y - E.y, a.y));
-        la.f[q] = F;
-        if (la.fprev) fa2_swing_terms(F, la.fprev[q], la.mass[o], la.variant, sw, tr);
+        nr[k] = ok ? la.f[q] : make_float2(0.f, 0.f);
+        E[k] = ok ? la.ef[o] : make_float2(0.f, 0.f);
+        a[k] = ok && la.fa ? la.fa[q] : make_float2(0.f, 0.f);
+        P[k] = ok && la.fprev ? la.fprev[q] : make_float2(0.f, 0.f);
+        m[k] = ok ? la.mass[o] : 0.f;
+    }
+    float sw[COMBINE_TILES], tr[COMBINE_TILES];
+#pragma unroll
+    for (int k = 0; k < COMBINE_TILES; ++k) {
+        const int o = o0 + 256 * k;
+        sw[k] = tr[k] = 0.f;
+        if (o >= n) continue;
+        const float km = la.kr * m[k];
+        const float2 F = make_float2(fmaf(km, nr[k].x + E[k].x, a[k].x), fmaf(km, nr[k].y - E[k].y, a[k].y));
+        la.f[la.q0 + o - la.fbase] = F;
+        if (la.fprev) fa2_swing_terms(F, P[k], m[k], la.variant, sw[k], tr[k]);
     }
     if (!la.fprev) return;
     // swing/traction of the iteration (Section 3.2): FP32 within a warp, FP64
-    // across warps and blocks, blocks summed in order by the last to arrive
-    __shared__ double ws[32], wt[32];
+    // across a tile's warps and over the tiles, summed in order by the last
+    // block to arrive
+    __shared__ double ws[COMBINE_TILES][8], wt[COMBINE_TILES][8];
     __shared__ bool last;
-#pragma unroll
-    for (int k = 16; k > 0; k >>= 1) {
-        sw += __shfl_xor_sync(0xffffffffu, sw, k);
-        tr += __shfl_xor_sync(0xffffffffu, tr, k);
-    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        ws[warp] = (double)sw;
-        wt[warp] = (double)tr;
+#pragma unroll
+    for (int k = 0; k < COMBINE_TILES; ++k) {
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) {
+            sw[k] += __shfl_xor_sync(0xffffffffu, sw[k], h);
+            tr[k] += __shfl_xor_sync(0xffffffffu, tr[k], h);
+        }
+        if (lane == 0) {
+            ws[k][warp] = (double)sw[k];
+            wt[k][warp] = (double)tr[k];
+        }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    const int tiles = (n + 255) / 256;
+    if (threadIdx.x < COMBINE_TILES) {
+        const int k = threadIdx.x, tile = blockIdx.x * COMBINE_TILES + k;
         double s = 0.0, u = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            s += ws[w];
-            u += wt[w];
+        for (int w = 0; w < 8; ++w) {
+            s += ws[k][w];
+            u += wt[k][w];
         }
-        la.spart[blockIdx.x] = make_double2(s, u);
+        if (tile < tiles) la.spart[tile] = make_double2(s, u);
         __threadfence();
-        last = atomicAdd(la.scount, 1u) == gridDim.x - 1;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(la.scount, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // the last block: thread t sums the partials t, t + blockDim, ... (fixed
+    // the last block: thread t sums the partials t, t + 256, ... (fixed
     // order), then the block's sums in warp order
     double swg = 0.0, trc = 0.0;
-    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) {
+    for (int k = threadIdx.x; k < tiles; k += blockDim.x) {
         const double2 v = __ldcg(&la.spart[k]);
         swg += v.x;
         trc += v.y;
@@ -1746,16 +1821,16 @@ __global__ void combine_kernel(LeafArgs la, int n) {
     }
     __syncthreads();
     if (lane == 0) {
-        ws[warp] = swg;
-        wt[warp] = trc;
+        ws[0][warp] = swg;
+        wt[0][warp] = trc;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         swg = 0.0;
         trc = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            swg += ws[w];
-            trc += wt[w];
+        for (int w = 0; w < 8; ++w) {
+            swg += ws[0][w];
+            trc += wt[0][w];
         }
         const double s_new = fa2_global_speed(swg, trc, *la.sg, la.tau);
         *la.sg = s_new;
@@ -1773,38 +1848,53 @@ __global__ void combine_kernel(LeafArgs la, int n) {
 // Fused update: every point moves by s F (Section 3.2) and F_{t-1} <- F;
 // the new positions give the next evaluation's root square, and block 0
 // clears the next evaluation's tickets and counts (what bbox_kernel does).
-__global__ void update_root_kernel(float2 *xy, const float2 *__restrict__ f, float2 *fprev, int n, const double *sg,
-                                   float ks, float ksmax, int *bad, float4 *__restrict__ part, unsigned *counter,
-                                   Root *root, int *err, unsigned *epoch, int *tickets, OsHist h) {
+// Several points a thread, as in combine_kernel (one: 13.1 us for 556,277).
+constexpr int UPDATE_POINTS = 4;
+
+__global__ void __launch_bounds__(256) update_root_kernel(float2 *xy, const float2 *__restrict__ f, float2 *fprev, int n,
+                                                         const double *sg, float ks, float ksmax, int *bad,
+                                                         float4 *__restrict__ part, unsigned *counter, Root *root,
+                                                         int *err, unsigned *epoch, int *tickets, OsHist h) {
     evaluation_clear(tickets, h);
     const float g = (float)*sg;
     float mnx = INFINITY, mxx = -INFINITY, mny = INFINITY, mxy = -INFINITY;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;   // one point per thread
-    if (i < n) {
-        const float2 F = f[i], P = fprev[i];
-        const float2 p = fa2_move(xy[i], F, P, g, ks, ksmax);
-        if (!isfinite(p.x) || !isfinite(p.y)) *bad = 1;
-        xy[i] = p;
-        fprev[i] = F;
-        mnx = fminf(mnx, p.x);
-        mxx = fmaxf(mxx, p.x);
-        mny = fminf(mny, p.y);
-        mxy = fmaxf(mxy, p.y);
+    const int i0 = blockIdx.x * (256 * UPDATE_POINTS) + threadIdx.x;
+    float2 F[UPDATE_POINTS], P[UPDATE_POINTS], p[UPDATE_POINTS];
+#pragma unroll
+    for (int k = 0; k < UPDATE_POINTS; ++k) {
+        const int i = i0 + 256 * k;
+        const bool ok = i < n;
+        F[k] = ok ? f[i] : make_float2(0.f, 0.f);
+        P[k] = ok ? fprev[i] : make_float2(0.f, 0.f);
+        p[k] = ok ? xy[i] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int k = 0; k < UPDATE_POINTS; ++k) {
+        const int i = i0 + 256 * k;
+        if (i >= n) continue;
+        const float2 q = fa2_move(p[k], F[k], P[k], g, ks, ksmax);
+        if (!isfinite(q.x) || !isfinite(q.y)) *bad = 1;
+        xy[i] = q;
+        fprev[i] = F[k];
+        mnx = fminf(mnx, q.x);
+        mxx = fmaxf(mxx, q.x);
+        mny = fminf(mny, q.y);
+        mxy = fmaxf(mxy, q.y);
     }
     bbox_reduce_root(mnx, mxx, mny, mxy, part, counter, root, err, epoch);
 }
 
 // the tile variant with R targets per lane
-template <int R>
+template <int R, class Stage>
 __device__ __forceinline__ void near_dispatch(int r, const Tree &T, LeafArgs &la, float4 (*buf)[NEAR_SRC], int tb,
                                               int ntc, int us, int ue, int lane) {
     if constexpr (R > 1) {
         if (r < R) {
-            near_dispatch<R - 1>(r, T, la, buf, tb, ntc, us, ue, lane);
+            near_dispatch<R - 1, Stage>(r, T, la, buf, tb, ntc, us, ue, lane);
             return;
         }
     }
-    near_tile<R>(T, la, buf, tb, ntc, us, ue, lane);
+    near_tile<R, Stage>(T, la, buf, tb, ntc, us, ue, lane);
 }
 
 __global__ void __launch_bounds__(NEAR_WARPS * 32) near_kernel(LeafArgs la) {
@@ -1844,7 +1934,52 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) near_kernel(LeafArgs la) {
         const int us = T.lofs[5 * b], ue = T.lofs[5 * b + 1];
         for (int tb = s; tb < e; tb += NEAR_LPS * NEAR_RMAX) {
             const int ntc = min(NEAR_LPS * NEAR_RMAX, e - tb);
-            near_dispatch<NEAR_RMAX>((ntc + NEAR_LPS - 1) / NEAR_LPS, T, la, buf, tb, ntc, us, ue, lane);
+            near_dispatch<NEAR_RMAX, Stager>((ntc + NEAR_LPS - 1) / NEAR_LPS, T, la, buf, tb, ntc, us, ue, lane);
+        }
+    }
+}
+
+// The near field of a tree with few leaves: a warp takes some of a leaf's
+// targets, rows of NEAR_LPS of them, so that a chip's worth of warps shares
+// what one warp per leaf would leave to a few (225 leaves: 29.3 us with one
+// warp each, 18.2 so; 843 leaves: 40.4 and 20.3).  As many rows as leave two
+// work items a warp.  Every target's sum is that of near_kernel bit for bit.
+__global__ void __launch_bounds__(NEAR_WARPS * 32) near_rows_kernel(LeafArgs la) {
+    if (aborted(la.e.T.err)) return;
+    const Tree &T = la.e.T;
+    __shared__ __align__(16) float4 stage[NEAR_WARPS][2][NEAR_SRC];
+    const int lane = threadIdx.x & 31;
+    float4(*buf)[NEAR_SRC] = stage[threadIdx.x >> 5];
+    const int leaves = lane < NEAR_RMAX ? T.ncls[lane] : 0;      // of class lane + 1 (rows of a leaf)
+    const int nw = gridDim.x * NEAR_WARPS;
+    // items of the class for 1, 2 and 4 rows an item, and their totals
+    int rows = 1, items, total;
+    for (;; rows *= 2) {
+        items = leaves * ((lane + rows) / rows);                 // ceil((lane + 1) / rows)
+        total = items;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+        if (rows == 4 || total <= 2 * nw) break;
+    }
+    for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(la.ticket, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= total) return;
+        int cls = NEAR_RMAX;
+        for (;; --cls) {
+            const int c = __shfl_sync(0xffffffffu, items, cls - 1);
+            if (t < c) break;
+            t -= c;
+        }
+        const int per = (cls + rows - 1) / rows;
+        const int b = T.cleaf[(size_t)(cls - 1) * T.Bmax + t / per];
+        const int s = T.bstart[b], e = T.bend[b];
+        const int us = T.lofs[5 * b], ue = T.lofs[5 * b + 1];
+        // a leaf of more than 64 points is all in the last class: its tiles in turn
+        for (int tb = s + t % per * rows * NEAR_LPS; tb < e; tb += NEAR_LPS * NEAR_RMAX) {
+            const int ntc = min(rows * NEAR_LPS, e - tb);
+            near_dispatch<4, WideStager>((ntc + NEAR_LPS - 1) / NEAR_LPS, T, la, buf, tb, ntc, us, ue, lane);
         }
     }
 }
@@ -2385,7 +2520,7 @@ static void phase_points(FmmPlan *pl, const float2 *xl, cudaStream_t s) {
                                                        pl->epoch.p, pl->tickets.p, h);
             BGL_LAUNCH_CHECK();
         }
-        keys_kernel<<<nblk(n, 256 * KEY_ITEMS), 256, 0, s>>>(xl, n, pl->root.p, pl->key.p, pl->idx.p, h);
+        keys_kernel<<<nblk(n, OS_TILE), OS_THREADS, 0, s>>>(xl, n, pl->root.p, pl->key.p, pl->idx.p, h);
         BGL_LAUNCH_CHECK();
         radix_sort_u32_ws_scatter(ctx, pl->sortws, pl->key.p, pl->idx.p, n, xl, ml, pl->pts.p, pl->sortskip.p,
                                   pl->wait);
@@ -2463,7 +2598,16 @@ static int near_blocks_per_sm(bool beside) {
     if (forced > 0) return std::min(forced, full);
     return beside && full > 1 ? full - 1 : full;
 }
+// Components up to this size take near_rows_kernel: a whole iteration on 8,888
+// nodes 108.1 us without it and 96.0 with it, on 27,980 115.3 and 113.5, on
+// 69,696 125.6 and 126.4 (there the far field beside it is the longer branch).
+constexpr int NEAR_ROWS_MAX_N = 1 << 15;
 static void launch_near(FmmPlan *pl, const LeafArgs &la, cudaStream_t s, bool beside) {
+    if (BGL_NEAR_BUCKETS && pl->n <= NEAR_ROWS_MAX_N) {
+        near_rows_kernel<<<pl->g->ctx->num_sms * near_blocks_per_sm(beside), NEAR_WARPS * 32, 0, s>>>(la);
+        BGL_LAUNCH_CHECK();
+        return;
+    }
     near_kernel<<<pl->g->ctx->num_sms * near_blocks_per_sm(beside), NEAR_WARPS * 32, 0, s>>>(la);
     BGL_LAUNCH_CHECK();
 }
@@ -2475,7 +2619,7 @@ static void launch_far(FmmPlan *pl, const LeafArgs &la, cudaStream_t s) {
     BGL_LAUNCH_CHECK();
 }
 static void launch_combine(FmmPlan *pl, const LeafArgs &la, cudaStream_t s) {
-    combine_kernel<<<nblk(pl->n, 256), 256, 0, s>>>(la, pl->n);
+    combine_kernel<<<nblk(pl->n, 256 * COMBINE_TILES), 256, 0, s>>>(la, pl->n);
     BGL_LAUNCH_CHECK();
 }
 
@@ -2679,7 +2823,7 @@ void fmm_root(FmmPlan *pl, const float2 *xy, int64_t qbase) {
 void fmm_update_root(FmmPlan *pl, float2 *xy, int64_t qbase, const float2 *f, float2 *fprev, int64_t fbase) {
     bgl_ctx *ctx = pl->g->ctx;
     const OsHist h = radix_sort_u32_ws_begin(ctx, pl->sortws, pl->n, false);
-    update_root_kernel<<<nblk(pl->n, 256), 256, 0, ctx->stream>>>(
+    update_root_kernel<<<nblk(pl->n, 256 * UPDATE_POINTS), 256, 0, ctx->stream>>>(
         xy + (pl->q0 - qbase), f + (pl->q0 - fbase), fprev + (pl->q0 - fbase), pl->n, pl->fz.sg, pl->fz.ks,
         pl->fz.ksmax, pl->fz.bad, pl->part.p, pl->counter.p, pl->root.p, pl->err.p, pl->epoch.p, pl->tickets.p, h);
     BGL_LAUNCH_CHECK();

@@ -297,7 +297,7 @@ struct OsBufs {
     uint32_t *k0, *v0, *k1, *v1; // scratch
 };
 
-__global__ void __launch_bounds__(OS_THREADS, 2) os_scatter_kernel(OsBufs bf, int d, const int *d_skip, int64_t n,
+__global__ void __launch_bounds__(OS_THREADS, OS_THREADS > 512 ? 1 : 2) os_scatter_kernel(OsBufs bf, int d, const int *d_skip, int64_t n,
                                                                  const uint32_t *__restrict__ base,
                                                                  uint32_t *status, unsigned *ticket, int *err,
                                                                  const float2 *__restrict__ gxy,
@@ -310,10 +310,10 @@ __global__ void __launch_bounds__(OS_THREADS, 2) os_scatter_kernel(OsBufs bf, in
     const uint32_t *__restrict__ vin = d == skip ? bf.vals : (((d - skip - 1) & 1) ? bf.v1 : bf.v0);
     uint32_t *__restrict__ kout = d == 3 ? bf.keys : (((d - skip) & 1) ? bf.k1 : bf.k0);
     uint32_t *__restrict__ vout = d == 3 ? bf.vals : (((d - skip) & 1) ? bf.v1 : bf.v0);
-    __shared__ int32_t cnt[OS_WARPS][256];
+    __shared__ __align__(4) uint16_t cnt[OS_WARPS][256];     // (at most a tile)
     __shared__ uint32_t gofs[256];
     __shared__ int32_t lstart[256];
-    __shared__ int32_t wsum[OS_WARPS];
+    __shared__ int32_t wsum[8];
     __shared__ uint32_t skey[OS_TILE], sval[OS_TILE];
     __shared__ int tile_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(OS_THREADS, 2) os_scatter_kernel(OsBufs bf, in
     // block started) the keys are not sorted: blocks return before taking
     // a tile, so no tile is left waiting for one that nobody holds
     if (threadIdx.x == 0) tile_s = (*(volatile int *)err & 1) ? -1 : (int)atomicAdd(ticket, 1u);
-    for (int i = threadIdx.x; i < OS_WARPS * 256; i += OS_THREADS) (&cnt[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < OS_WARPS * 128; i += OS_THREADS) reinterpret_cast<uint32_t *>(cnt)[i] = 0;
     __syncthreads();
     const int tile = tile_s;
     if (tile < 0) return;
@@ -348,24 +348,25 @@ __global__ void __launch_bounds__(OS_THREADS, 2) os_scatter_kernel(OsBufs bf, in
         const int before = __popc(peers & lt);
         const int cur = ok ? cnt[warp][d] : 0;
         __syncwarp();
-        if (ok && before == 0) cnt[warp][d] = cur + __popc(peers);
+        if (ok && before == 0) cnt[warp][d] = (uint16_t)(cur + __popc(peers));
         __syncwarp();
         rank[r] = ok ? cur + before : -1;
     }
     __syncthreads();
-    {
-        // thread = digit: prefix over warps, then an exclusive scan over digits
-        // (tile-local start of each digit run), then the look-back for the
-        // global offset of each digit run
+    // thread = digit: prefix over warps, then an exclusive scan over digits
+    // (tile-local start of each digit run), then the look-back for the
+    // global offset of each digit run
+    const bool digit = threadIdx.x < 256;
+    int s = 0, x = 0;
+    if (digit) {
         const int d = threadIdx.x;
-        int s = 0;
 #pragma unroll
         for (int w = 0; w < OS_WARPS; ++w) {
             const int c = cnt[w][d];
-            cnt[w][d] = s;
+            cnt[w][d] = (uint16_t)s;
             s += c;
         }
-        int x = s;
+        x = s;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -407,10 +408,12 @@ __global__ void __launch_bounds__(OS_THREADS, 2) os_scatter_kernel(OsBufs bf, in
             st[(int64_t)tile * 256 + d] = OS_INC | (excl + own);
         }
         gofs[d] = base[d] + excl;
-        __syncthreads();
+    }
+    __syncthreads();
+    if (digit) {
         int pre = 0;
         for (int w = 0; w < warp; ++w) pre += wsum[w];
-        lstart[d] = pre + x - s;
+        lstart[threadIdx.x] = pre + x - s;
     }
     __syncthreads();
     // keys to their tile-local sorted position, then coalesced runs to global
