@@ -146,13 +146,13 @@ struct Tree {
     int *bstart, *bend, *blevel, *bparent;
     uint32_t *bkey;
     int8_t *bleaf;
-    int4 *bchild;
+    int4 *bchild;             // per box its children, 2 index + leaf (-1: none)
     int2 *bmeta;              // per box {x | y << 16 at its level, level | leaf << 8}: one load
     int *levoff;              // [NLEV + 1], levoff[NLEV] = number of boxes
     int *lofs;                // [5 * Bmax] per box: starts of U, V, W, X and the end, in lidx
     int *lidx;                // list entries (each box's lists in one chunk)
     int *pool;                // entries handed out so far (zero at the start of an evaluation)
-    ulonglong2 *hkv;          // box hash table: {key tagged with the evaluation epoch, box index}
+    ulonglong2 *hkv;          // box hash table: {key tagged with the evaluation epoch, box index | leaf << 32}
     int hmask;                // table size - 1 (a power of two)
     const unsigned *epoch;    // evaluation counter (1..2^24-1)
     int lcap;                 // capacity of lidx
@@ -251,7 +251,8 @@ __device__ __forceinline__ unsigned hash_slot(unsigned long long k, int mask) {
     return (unsigned)k & (unsigned)mask;
 }
 
-__device__ void hash_insert(ulonglong2 *hkv, int mask, unsigned epoch, int L, uint32_t prefix, int box, int *err) {
+__device__ void hash_insert(ulonglong2 *hkv, int mask, unsigned epoch, int L, uint32_t prefix, int box, bool leaf,
+                            int *err) {
     const unsigned long long k = hash_key(epoch, L, prefix);
     unsigned s = hash_slot(k, mask);
     for (int probe = 0; probe <= mask; ++probe) {
@@ -259,7 +260,7 @@ __device__ void hash_insert(ulonglong2 *hkv, int mask, unsigned epoch, int L, ui
         while ((cur >> 40) != epoch) {             // empty (stale): try to claim it
             const unsigned long long prev = atomicCAS(&hkv[s].x, cur, k);
             if (prev == cur) {
-                hkv[s].y = (unsigned long long)(unsigned)box;
+                hkv[s].y = (unsigned long long)(unsigned)box | ((unsigned long long)leaf << 32);
                 return;
             }
             cur = prev;
@@ -269,30 +270,35 @@ __device__ void hash_insert(ulonglong2 *hkv, int mask, unsigned epoch, int L, ui
     atomicOr(err, 4);                              // table full (cannot happen at twice the box capacity)
 }
 
-// box index of (L, prefix) in this evaluation, or -1
-__device__ __forceinline__ int hash_find(const Tree &T, unsigned epoch, int L, uint32_t prefix) {
+// value of (L, prefix) in this evaluation (box index | leaf << 32), or -1
+__device__ __forceinline__ long long hash_find_value(const Tree &T, unsigned epoch, int L, uint32_t prefix) {
     const unsigned long long k = hash_key(epoch, L, prefix);
     unsigned s = hash_slot(k, T.hmask);
     for (int probe = 0; probe <= T.hmask; ++probe) {
         const ulonglong2 cur = __ldcg(&T.hkv[s]);
-        if (cur.x == k) return (int)cur.y;
+        if (cur.x == k) return (long long)cur.y;
         if ((cur.x >> 40) != epoch) return -1;
         s = (s + 1) & (unsigned)T.hmask;
     }
     return -1;
 }
+__device__ __forceinline__ int hash_find(const Tree &T, unsigned epoch, int L, uint32_t prefix) {
+    return (int)hash_find_value(T, epoch, L, prefix);
+}
 
 // The box at level L covering cell (cx, cy) of level L, else the coarser
-// leaf covering it, else -1 (empty cell or outside the root square).
-__device__ int cover(const Tree &T, unsigned epoch, int L, int cx, int cy) {
+// leaf covering it, else -1 (empty cell or outside the root square); its
+// level | leaf << 8 in `info`.
+__device__ int cover(const Tree &T, unsigned epoch, int L, int cx, int cy, int &info) {
     if (cx < 0 || cy < 0 || cx >= (1 << L) || cy >= (1 << L)) return -1;
     for (int l = L; l >= 0; --l) {
         const int d = L - l;
         const uint32_t pre = spread_bits((uint32_t)(cx >> d)) | (spread_bits((uint32_t)(cy >> d)) << 1);
-        const int A = hash_find(T, epoch, l, pre);
-        if (A < 0) continue;
-        if (l == L) return A;
-        return (T.bmeta[A].y & 256) ? A : -1;
+        const long long v = hash_find_value(T, epoch, l, pre);
+        if (v < 0) continue;
+        const bool leaf = (v >> 32) != 0;
+        info = l | (leaf ? 256 : 0);
+        return l == L || leaf ? (int)v : -1;
     }
     return -1;
 }
@@ -438,6 +444,16 @@ __global__ void __launch_bounds__(OS_THREADS) keys_kernel(const float2 *__restri
     os_block_hist<KEY_ITEMS>(k, valid, h);
 }
 
+
+__device__ __forceinline__ int warp_incl_scan(int v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    return v;
+}
 
 // ---------------------------------------------------------------- tree build
 
@@ -599,8 +615,10 @@ __global__ void __launch_bounds__(SCAN_THREADS) tree_scan_kernel(int *tcnt, int 
 //     before_{L-1}(i) if that one starts at i too, else before_{L-1}(i) - 1;
 //   the box of level L holding point i - 1 ends (c(i) < L <= lambda(i-1)):
 //     index before_L(i) - 1, end i; every box holding point n - 1 ends at n.
-// Each new box also takes its child slot in the parent and its entry in
-// the hash table.  Levels above the deepest leaf level met in the tile
+// Each new box also takes its child slot in the parent.  The entries in the
+// hash table come last, the tile's boxes a thread each: a thread that entered
+// its boxes as it made them waited for a probe and an exchange at each, up to
+// four a level (11.3 us in a tree of 301 boxes).  Levels above the deepest leaf level met in the tile
 // (of its points and of the point before it) hold no box start or end.
 __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const int8_t *__restrict__ cl,
                                                                 const int8_t *__restrict__ lam,
@@ -609,7 +627,8 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const i
     constexpr int NW = TREE_THREADS / 32;
     constexpr int R = TREE_TILE / TREE_THREADS;        // rounds per warp
     constexpr int PW = TREE_TILE / NW;                 // points per warp
-    __shared__ int wcount[NLEV][NW];
+    __shared__ int wcount[NLEV][NW];   // boxes of the level in each warp, then in the warps before it
+    __shared__ int lcount[NLEV + 1];   // the tile's boxes of the levels before
     __shared__ int smax;
     __shared__ int stc[NLEV];          // the tile's offset at every level, loaded once
     if (threadIdx.x == 0) smax = 0;
@@ -663,6 +682,21 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const i
         if (lane == 0) wcount[L][warp] = tot;
     }
     __syncthreads();
+    if (warp == 0) {
+        int tot = 0;
+        if (lane <= Lmax) {
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const int c = wcount[lane][w];
+                wcount[lane][w] = tot;
+                tot += c;
+            }
+        }
+        const int upto = warp_incl_scan(tot);
+        if (lane <= Lmax) lcount[lane + 1] = upto;
+        if (lane == 0) lcount[0] = 0;
+    }
+    __syncthreads();
     int pb[R];            // before_{L-1}(i), then whether a box of level L - 1 starts at i
     bool pf[R];
 #pragma unroll
@@ -671,8 +705,7 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const i
         pf[r] = false;
     }
     for (int L = 0; L <= Lmax; ++L) {
-        int base = stc[L];
-        for (int w = 0; w < warp; ++w) base += wcount[L][w];
+        int base = stc[L] + wcount[L][warp];
         if (!((lm >> L) & 1u)) {
             // no start or end at this level: before_L(i) = base for every point
 #pragma unroll
@@ -699,11 +732,10 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const i
                 int par = -1;
                 if (L >= 1) {
                     par = pf[r] ? pb[r] : pb[r] - 1;
-                    if (par >= 0 && par < b) ((int *)&T.bchild[par])[P & 3u] = b;
+                    if (par >= 0 && par < b) ((int *)&T.bchild[par])[P & 3u] = 2 * b + (L == la[r] ? 1 : 0);
                     else atomicOr(T.err, ERR_BOX_OVERFLOW);
                 }
                 T.bparent[b] = par;
-                hash_insert(T.hkv, T.hmask, epoch, L, P, b, T.err);
             }
             // the box of level L holding point i - 1 ends at i
             if (i < T.n && c[r] < L && L <= lp[r] && before >= 1 && before - 1 < Bmax) T.bend[before - 1] = i;
@@ -714,6 +746,13 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const i
             pf[r] = f;
             base += __popc(bl);
         }
+    }
+    __syncthreads();                   // the tile's boxes are written
+    for (int i = threadIdx.x; i < lcount[Lmax + 1]; i += TREE_THREADS) {
+        int L = 0;
+        while (i >= lcount[L + 1]) ++L;
+        const int b = stc[L] + i - lcount[L];
+        if (b < Bmax) hash_insert(T.hkv, T.hmask, epoch, L, T.bkey[b], b, T.bleaf[b] != 0, T.err);
     }
 }
 
@@ -761,7 +800,7 @@ __device__ void lists_uw(const Tree &T, int b, int2 mb, const int *nbb, int k, i
     while (sp > 0) {
         const int D = stack[--sp];
         const int4 ch = T.bchild[D];
-        const int cs[4] = {ch.x, ch.y, ch.z, ch.w};
+        const int cs[4] = {ch.x >> 1, ch.y >> 1, ch.z >> 1, ch.w >> 1};
         int2 mc[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) mc[q] = cs[q] >= 0 ? T.bmeta[cs[q]] : make_int2(0, 0);
@@ -785,91 +824,74 @@ __device__ void lists_uw(const Tree &T, int b, int2 mb, const int *nbb, int k, i
     }
 }
 
-// (ov[q] for child q, -1 where it is absent or adjacent; cv = how many are set)
-__device__ __forceinline__ void lists_v(const Tree &T, int2 mb, int A, int k, int (&ov)[4], int &cv) {
+// (ov[q] for child q, -1 where it is absent or adjacent; cv = how many are
+// set; A the box of the parent's cell (ax, ay), info its level and leaf flag)
+__device__ __forceinline__ void lists_v(const Tree &T, int2 mb, int A, int info, int ax, int ay, int k, int (&ov)[4],
+                                        int &cv) {
     cv = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) ov[q] = -1;
     const int L = meta_level(mb);
-    if (L < 2 || k == 4) return;
-    if (A < 0) return;
-    const int2 ma = T.bmeta[A];
-    if (meta_level(ma) != L - 1 || meta_leaf(ma)) return;
+    if (L < 2 || k == 4 || A < 0 || info != L - 1) return;       // (an internal box of the parent's level)
     const int bx = mx_(mb.x), by = my_(mb.x);
     const int4 ch = T.bchild[A];
     const int cs[4] = {ch.x, ch.y, ch.z, ch.w};
-    int cc[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) cc[q] = cs[q] >= 0 ? T.bmeta[cs[q]].x : 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const int C = cs[q];
-        if (C < 0) continue;
-        const int dx = mx_(cc[q]) - bx, dy = my_(cc[q]) - by;
+        if (cs[q] < 0) continue;
+        const int dx = 2 * ax + (q & 1) - bx, dy = 2 * ay + (q >> 1) - by;
         if (abs(dx) <= 1 && abs(dy) <= 1) continue;
-        ov[q] = (C << 6) | ((dx + 3) * 7 + (dy + 3));
+        ov[q] = ((cs[q] >> 1) << 6) | ((dx + 3) * 7 + (dy + 3));
         ++cv;
     }
 }
 
-// (dup: an earlier cell of the parent had the same box)
-__device__ void lists_x(const Tree &T, int2 mb, int A, int k, bool dup, int *ox, int &cx) {
-    cx = 0;
+// (dup: an earlier cell of the parent had the same box; A covers the
+// parent's cell (ax, ay))
+__device__ __forceinline__ bool lists_x(int2 mb, int A, int info, int ax, int ay, int k, bool dup) {
     const int L = meta_level(mb);
-    if (L < 2 || k == 4) return;
-    if (A < 0 || dup) return;
-    const int2 ma = T.bmeta[A];
-    if (!meta_leaf(ma)) return;
-    if (adjacent_xy(ma.x, meta_level(ma), mb.x, L)) return;
-    if (ox) ox[0] = A;
-    cx = 1;
+    if (L < 2 || k == 4 || A < 0 || dup || !(info & 256)) return false;
+    const int l = info & 255, d = L - 1 - l;
+    return !adjacent_xy((ax >> d) | ((ay >> d) << 16), l, mb.x, L);
 }
 
 // Warp-wide breadth-first descent from the internal same-level neighbours
-// of leaf (cb, L) (front[0 .. nf)): every child that touches the leaf is a
-// U entry if it is a leaf and joins the next frontier otherwise; every child
-// that does not touch it is a W entry.  The frontier is taken 32 boxes at a
-// time, a lane per box; one warp scan of packed class counts orders the
-// outputs (level by level, frontier order, child order).  Entries go to
-// su[nu ..] and sw[nw ..] while they fit in LST_CAP; returns false if any
-// list or frontier exceeded its staging capacity (the counts stay exact).
+// of leaf (cb, L) (front[0 .. nf), their coordinates in frontc): every child
+// that touches the leaf is a U entry if it is a leaf and joins the next
+// frontier otherwise; every child that does not touch it is a W entry.  The
+// frontier is taken 32 boxes at a time, a lane per box, all of one level, so
+// a child's place follows from its parent's; one warp scan of packed class
+// counts orders the outputs (level by level, frontier order, child order).
+// Entries go to su[nu ..] and sw[nw ..] while they fit in LST_CAP; returns
+// false if any list or frontier exceeded its staging capacity (the counts
+// stay exact).
 constexpr int LST_CAP = 256;
 constexpr int FRONT_CAP = 128;
 
-__device__ __forceinline__ int warp_incl_scan(int v) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
-    }
-    return v;
-}
-
-__device__ bool descend(const Tree &T, int cb, int L, int *front, int nf, int *su, int &nu, int *sw, int &nw,
-                        int lane) {
-    int *cur = front, *nxt = front + FRONT_CAP;
+__device__ bool descend(const Tree &T, int cb, int L, int *front, int *frontc, int nf, int *su, int &nu, int *sw,
+                        int &nw, int lane) {
+    int *cur = front, *nxt = front + FRONT_CAP, *curc = frontc, *nxtc = frontc + FRONT_CAP;
     bool ok = true;
-    while (nf > 0) {
+    for (int lv = L + 1; nf > 0; ++lv) {
         int nn = 0;
         for (int base = 0; base < nf; base += 32) {
             const int i = base + lane;
-            int cs[4] = {-1, -1, -1, -1};
+            int cs[4] = {-1, -1, -1, -1}, cc[4] = {0, 0, 0, 0};
             unsigned cls = 0;       // 2 bits per child: 0 none, 1 U, 2 W, 3 frontier
             if (i < nf) {
                 const int4 ch = T.bchild[cur[i]];
+                const int pc = curc[i];
                 cs[0] = ch.x;
                 cs[1] = ch.y;
                 cs[2] = ch.z;
                 cs[3] = ch.w;
-                int2 mc[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) mc[q] = cs[q] >= 0 ? T.bmeta[cs[q]] : make_int2(0, 0);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (cs[q] < 0) continue;
-                    const unsigned c = adjacent_xy(mc[q].x, mc[q].y & 255, cb, L) ? (mc[q].y & 256 ? 1u : 3u) : 2u;
+                    cc[q] = (2 * mx_(pc) + (q & 1)) | ((2 * my_(pc) + (q >> 1)) << 16);
+                    const unsigned c = adjacent_xy(cc[q], lv, cb, L) ? (cs[q] & 1 ? 1u : 3u) : 2u;
                     cls |= c << (2 * q);
+                    cs[q] >>= 1;
                 }
             }
             // counts packed 10 bits per class (at most 4 per lane, 128 per warp)
@@ -892,7 +914,10 @@ __device__ bool descend(const Tree &T, int cb, int L, int *front, int nf, int *s
                     if (pw < LST_CAP) sw[pw] = cs[q];
                     ++pw;
                 } else if (c == 3u) {
-                    if (pf < FRONT_CAP) nxt[pf] = cs[q];
+                    if (pf < FRONT_CAP) {
+                        nxt[pf] = cs[q];
+                        nxtc[pf] = cc[q];
+                    }
                     ++pf;
                 }
             }
@@ -904,6 +929,9 @@ __device__ bool descend(const Tree &T, int cb, int L, int *front, int nf, int *s
         int *t = cur;
         cur = nxt;
         nxt = t;
+        t = curc;
+        curc = nxtc;
+        nxtc = t;
         nf = nn;
         if (nf > FRONT_CAP) {
             ok = false;
@@ -929,11 +957,11 @@ constexpr int LIST_WARPS = 8;
 __global__ void __launch_bounds__(LIST_WARPS * 32) nbr_lists_kernel(Tree T) {
     if (aborted(T.err)) return;
     __shared__ int s_u[LIST_WARPS][LST_CAP], s_w[LIST_WARPS][LST_CAP];
-    __shared__ int s_front[LIST_WARPS][2 * FRONT_CAP];
+    __shared__ int s_front[LIST_WARPS][2 * FRONT_CAP], s_frontc[LIST_WARPS][2 * FRONT_CAP];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int role = lane / 9, k = lane % 9;
     const unsigned lt = (1u << lane) - 1u;
-    int *su = s_u[wib], *sw = s_w[wib], *front = s_front[wib];
+    int *su = s_u[wib], *sw = s_w[wib], *front = s_front[wib], *frontc = s_frontc[wib];
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int B = min(T.levoff[NLEV], T.Bmax);
@@ -944,44 +972,46 @@ __global__ void __launch_bounds__(LIST_WARPS * 32) nbr_lists_kernel(Tree T) {
         const bool leaf = meta_leaf(mb);
         const int bx = mx_(mb.x), by = my_(mb.x);
         const int p = b == 0 ? -1 : T.bparent[b];
-        int mine = -1;
+        int mine = -1, minfo = 0;
         if (lane < 9) {
-            mine = lane == 4 ? b : cover(T, epoch, L, bx + lane % 3 - 1, by + lane / 3 - 1);
+            minfo = L | (leaf ? 256 : 0);
+            mine = lane == 4 ? b : cover(T, epoch, L, bx + lane % 3 - 1, by + lane / 3 - 1, minfo);
         } else if (lane < 18 && p >= 0) {
             const int j = lane - 9;
-            mine = j == 4 ? p : cover(T, epoch, L - 1, (bx >> 1) + j % 3 - 1, (by >> 1) + j / 3 - 1);
+            minfo = L - 1;
+            mine = j == 4 ? p : cover(T, epoch, L - 1, (bx >> 1) + j % 3 - 1, (by >> 1) + j / 3 - 1, minfo);
         }
         // lane (role, k): the box of cell k around b (role 0) or around its parent (roles 1, 2)
-        const int A = __shfl_sync(0xffffffffu, mine, role == 0 ? k : 9 + k);
+        const int from = role == 0 ? k : 9 + k;
+        const int A = __shfl_sync(0xffffffffu, mine, from), info = __shfl_sync(0xffffffffu, minfo, from);
+        const int ax = (bx >> 1) + k % 3 - 1, ay = (by >> 1) + k / 3 - 1;   // cell k around the parent
         // a cell whose box an earlier cell of the same group already had (k = 4 excluded)
         const bool grp = role <= 2 && k != 4 && A >= 0;
-        const unsigned long long tag =
-            grp ? ((unsigned long long)role << 32) | (unsigned)A : (1ull << 40) + (unsigned)lane;
+        const unsigned tag = grp ? ((unsigned)role << 28) | (unsigned)A : 0xC0000000u + (unsigned)lane;   // A < 2^25
         const bool dup = (__match_any_sync(0xffffffffu, tag) & lt) != 0u;
         // V (lanes 9-17, up to 4 each) and X (lanes 18-26, up to 1 each) in registers
         int ve[4] = {-1, -1, -1, -1};
         int cv = 0, xe = -1;
-        if (role == 1 && p >= 0) lists_v(T, mb, A, k, ve, cv);
-        else if (role == 2 && p >= 0) {
-            int cx = 0;
-            lists_x(T, mb, A, k, dup, &xe, cx);
-            if (!cx) xe = -1;
-        }
+        if (role == 1 && p >= 0) lists_v(T, mb, A, info, ax, ay, k, ve, cv);
+        else if (role == 2 && p >= 0 && lists_x(mb, A, info, ax, ay, k, dup)) xe = A;
         // direct U entries and the frontier (lanes 0-8 of a leaf)
         int du = -1, fr = -1;
         if (leaf && role == 0) {
             if (k == 4) du = b;
             else if (A >= 0 && !dup) {
-                if (meta_leaf(T.bmeta[A])) du = A;
+                if (info & 256) du = A;
                 else fr = A;
             }
         }
         const unsigned bu = __ballot_sync(0xffffffffu, du >= 0), bf = __ballot_sync(0xffffffffu, fr >= 0);
         if (du >= 0) su[__popc(bu & lt)] = du;
-        if (fr >= 0) front[__popc(bf & lt)] = fr;
+        if (fr >= 0) {
+            front[__popc(bf & lt)] = fr;
+            frontc[__popc(bf & lt)] = (bx + k % 3 - 1) | ((by + k / 3 - 1) << 16);
+        }
         int nu = __popc(bu), nw = 0;
         __syncwarp();
-        const bool staged = bf == 0u || descend(T, mb.x, L, front, __popc(bf), su, nu, sw, nw, lane);
+        const bool staged = bf == 0u || descend(T, mb.x, L, front, frontc, __popc(bf), su, nu, sw, nw, lane);
         int nbb[9];
         if (!staged) {
             // overflow: exact counts by the per-lane walk
@@ -1359,7 +1389,7 @@ __global__ void __launch_bounds__(256) up_kernel(ExpArgs a) {
             __syncwarp();
             int last = 0;
             const int4 ch = T.bchild[pb];
-            const int cs[4] = {ch.x, ch.y, ch.z, ch.w};
+            const int cs[4] = {ch.x >> 1, ch.y >> 1, ch.z >> 1, ch.w >> 1};
             if (lane == 0) {
                 const int nch = (ch.x >= 0) + (ch.y >= 0) + (ch.z >= 0) + (ch.w >= 0);
                 const int old = atomicAdd(&a.arrive[pb], 1);
