@@ -13,12 +13,14 @@
 // arrival order.  Results do not depend on what else runs: every kernel is
 // deterministic and per-request state is private to its worker.
 //
-// k-hop extraction on the device: frontier expansion edge-parallel (a
-// thread per frontier edge, its frontier node by binary search over the
-// degree prefix sums), visited marks stamped with a per-worker counter (never
-// cleared), then the visited nodes sorted by id (local id = rank, so the
-// subgraph does not depend on the order of discovery) and the induced edges
-// listed per node in adjacency order.
+// k-hop extraction on the device, without the host between the hops: the
+// frontier's bounds stay in device memory, a hop is one kernel over its nodes
+// and one over the entries of those of high degree; visited marks are
+// stamped with a per-worker counter (never cleared).  The visited nodes in
+// ascending id (local id = rank, so the subgraph does not depend on the order
+// of discovery) and their degree prefix sums come from one scan over the
+// marks, and the induced edges, listed per node in adjacency order, from a
+// count and a fill over the entries.
 #include <chrono>
 #include <condition_variable>
 #include <deque>
@@ -51,41 +53,211 @@ __global__ void kh_iota_kernel(int32_t *__restrict__ dst, int64_t count) {
     if (i < count) dst[i] = (int32_t)i;
 }
 
-__global__ void kh_seed_kernel(int32_t *stamp, int32_t *vis, int32_t seed, int32_t epoch) {
+constexpr int KH_LANE_DEG = 8;         // frontier nodes up to this degree: one thread
+constexpr int KH_HUB_DEG = 1024;       // above this degree: the whole grid
+constexpr int KH_TILE = 4096;          // nodes per tile of the scan over the marks
+constexpr int KH_CHUNK = 2048;         // adjacency entries per block of the edge kernels
+
+// state of an extraction on the device
+struct KhState {
+    unsigned long long count;          // nodes visited
+    unsigned long long f0, f1;         // the frontier: visit list entries [f0, f1)
+    unsigned long long entries;        // adjacency entries of the visited nodes
+    unsigned long long edges;          // induced edges
+    unsigned hubs, arrive;
+};
+
+__global__ void kh_seed_kernel(int32_t *stamp, int32_t *vis, int32_t seed, int32_t epoch, KhState *st) {
     stamp[seed] = epoch;
     vis[0] = seed;
+    st->count = 1;
+    st->f0 = 0;
+    st->f1 = 1;
+    st->entries = st->edges = 0;
+    st->hubs = st->arrive = 0u;
 }
 
-__global__ void kh_deg_kernel(const int32_t *__restrict__ front, int64_t nf, const int64_t *__restrict__ off,
-                              int64_t *__restrict__ deg) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nf) deg[i] = off[front[i] + 1] - off[front[i]];
+// w joins the visit list if it was not in it (one count for the lanes of the
+// warp that come here together)
+__device__ __forceinline__ void kh_visit(int32_t w, int32_t *stamp, int32_t epoch, int32_t *vis, int64_t cap,
+                                         KhState *st) {
+    if (stamp[w] == epoch || atomicExch(&stamp[w], epoch) == epoch) return;
+    const unsigned m = __activemask();
+    const int lane = threadIdx.x & 31, lead = __ffs(m) - 1;
+    unsigned long long at = 0;
+    if (lane == lead) at = atomicAdd(&st->count, (unsigned long long)__popc(m));
+    at = __shfl_sync(m, at, lead) + __popc(m & ((1u << lane) - 1u));
+    if ((int64_t)at < cap) vis[at] = w;
 }
 
-// one thread per edge of the frontier; new nodes appended to vis[base ..]
-__global__ void kh_expand_kernel(const int32_t *__restrict__ front, int64_t nf, const int64_t *__restrict__ dscan,
-                                 int64_t E, const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                                 int32_t *stamp, int32_t epoch, int32_t *vis, int64_t base, int64_t cap,
-                                 unsigned long long *cnt) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= E) return;
-    int64_t lo = 0, hi = nf;           // largest i with dscan[i] <= e
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (dscan[mid] <= e) lo = mid;
-        else hi = mid;
+// A hop: the neighbours of the frontier's nodes of up to KH_HUB_DEG entries
+// (a thread for a few, the warp for more); the others go to `hubs`.
+__global__ void __launch_bounds__(KH_TPB) kh_hop_kernel(const int64_t *__restrict__ off,
+                                                       const int32_t *__restrict__ adj, int32_t *stamp,
+                                                       int32_t epoch, int32_t *vis, int64_t cap, int32_t *hubs,
+                                                       KhState *st) {
+    const int64_t f0 = (int64_t)st->f0, f1 = (int64_t)st->f1;
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * KH_TPB;
+    for (int64_t i0 = f0 + (int64_t)blockIdx.x * KH_TPB + (threadIdx.x & ~31); i0 < f1; i0 += step) {
+        const int64_t i = i0 + lane;
+        int64_t e0 = 0, deg = 0;
+        if (i < f1) {
+            const int32_t v = vis[i];
+            e0 = off[v];
+            deg = off[v + 1] - e0;
+            if (deg > KH_HUB_DEG) {
+                hubs[atomicAdd(&st->hubs, 1u)] = v;
+                deg = 0;
+            }
+        }
+        if (deg <= KH_LANE_DEG)
+            for (int64_t e = e0; e < e0 + deg; ++e) kh_visit(adj[e], stamp, epoch, vis, cap, st);
+        __syncwarp();
+        unsigned mid = __ballot_sync(0xffffffffu, deg > KH_LANE_DEG);
+        while (mid) {
+            const int l = __ffs(mid) - 1;
+            mid &= mid - 1;
+            const int64_t b = __shfl_sync(0xffffffffu, e0, l), d = __shfl_sync(0xffffffffu, deg, l);
+            for (int64_t e = lane; e < d; e += 32) kh_visit(adj[b + e], stamp, epoch, vis, cap, st);
+            __syncwarp();
+        }
     }
-    const int32_t f = front[lo];
-    const int32_t w = adj[off[f] + (e - dscan[lo])];
-    if (stamp[w] == epoch) return;
-    if (atomicExch(&stamp[w], epoch) == epoch) return;
-    const unsigned long long idx = atomicAdd(cnt, 1ull);
-    if (base + (int64_t)idx < cap) vis[base + idx] = w;
 }
 
-__global__ void kh_local_kernel(const int32_t *__restrict__ vis, int64_t n, int32_t *__restrict__ local) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) local[vis[r]] = (int32_t)r;
+// The hop's hubs, entries over the whole grid; the last block to finish makes
+// the next frontier.
+__global__ void __launch_bounds__(KH_TPB) kh_hub_kernel(const int64_t *__restrict__ off,
+                                                       const int32_t *__restrict__ adj, int32_t *stamp,
+                                                       int32_t epoch, int32_t *vis, int64_t cap,
+                                                       const int32_t *__restrict__ hubs, KhState *st) {
+    const unsigned nh = st->hubs;
+    for (unsigned h = 0; h < nh; ++h) {
+        const int32_t v = hubs[h];
+        const int64_t e1 = off[v + 1];
+        for (int64_t e = off[v] + (int64_t)blockIdx.x * KH_TPB + threadIdx.x; e < e1; e += (int64_t)gridDim.x * KH_TPB)
+            kh_visit(adj[e], stamp, epoch, vis, cap, st);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x != 0 || atomicAdd(&st->arrive, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    const unsigned long long n = *(volatile unsigned long long *)&st->count;
+    st->f0 = st->f1;
+    st->f1 = n < (unsigned long long)cap ? n : (unsigned long long)cap;
+    st->hubs = 0u;
+    st->arrive = 0u;
+}
+
+// exclusive sums of (x, y) over the block (every thread of KH_TPB calls it);
+// the totals to (tx, ty)
+__device__ __forceinline__ void kh_block_scan(int &x, long long &y, int &tx, long long &ty) {
+    __shared__ int wx[KH_TPB / 32];
+    __shared__ long long wy[KH_TPB / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int x0 = x;
+    const long long y0 = y;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, x, o);
+        const long long b = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) {
+            x += a;
+            y += b;
+        }
+    }
+    __syncthreads();
+    if (lane == 31) {
+        wx[warp] = x;
+        wy[warp] = y;
+    }
+    __syncthreads();
+    int px = 0;
+    long long py = 0;
+    tx = 0;
+    ty = 0;
+#pragma unroll
+    for (int w = 0; w < KH_TPB / 32; ++w) {
+        if (w == warp) {
+            px = tx;
+            py = ty;
+        }
+        tx += wx[w];
+        ty += wy[w];
+    }
+    x += px - x0;
+    y += py - y0;
+}
+
+// Scan over the marks of the resident graph's nodes, KH_TILE a block,
+// consecutive nodes a thread: first pass (vis null) the tiles' visited nodes
+// and adjacency entries, second the visited nodes in ascending id with their
+// ranks and entry prefix sums.
+__global__ void __launch_bounds__(KH_TPB) kh_mark_kernel(const int32_t *__restrict__ stamp, int32_t epoch, int64_t n_res,
+                                                        const int64_t *__restrict__ off, longlong2 *tiles,
+                                                        int32_t *vis, int32_t *local, int64_t *ds, int64_t cap) {
+    constexpr int PER = KH_TILE / KH_TPB;
+    const int64_t v0 = (int64_t)blockIdx.x * KH_TILE + (int64_t)threadIdx.x * PER;
+    unsigned mark = 0;
+    long long deg = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+        if (v0 + k < n_res && stamp[v0 + k] == epoch) mark |= 1u << k;
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+        if ((mark >> k) & 1u) deg += off[v0 + k + 1] - off[v0 + k];
+    int x = __popc(mark), tx;
+    long long y = deg, ty;
+    kh_block_scan(x, y, tx, ty);
+    if (!vis) {
+        if (threadIdx.x == 0) tiles[blockIdx.x] = make_longlong2(tx, ty);
+        return;
+    }
+    const longlong2 base = tiles[blockIdx.x];
+    int64_t r = base.x + x, e = base.y + y;
+    for (; mark; mark &= mark - 1) {
+        const int64_t v = v0 + __ffs(mark) - 1;
+        if (r < cap) {
+            vis[r] = (int32_t)v;
+            ds[r] = e;
+        }
+        local[v] = (int32_t)r;
+        ++r;
+        e += off[v + 1] - off[v];
+    }
+}
+
+// one block: the tiles' exclusive sums in place, the totals to st (of the
+// marks: count is already there; of the edge chunks: edges)
+__global__ void __launch_bounds__(KH_TPB) kh_tiles_kernel(longlong2 *tiles, int64_t n, KhState *st, int edges) {
+    constexpr int PER = 8;
+    long long cx = 0, cy = 0;
+    for (int64_t b = 0; b < n; b += KH_TPB * PER) {
+        const int64_t k0 = b + (int64_t)threadIdx.x * PER;
+        longlong2 t[PER];
+        int x = 0, tx;
+        long long y = 0, ty;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            t[k] = k0 + k < n ? tiles[k0 + k] : make_longlong2(0, 0);
+            x += (int)t[k].x;
+            y += t[k].y;
+        }
+        kh_block_scan(x, y, tx, ty);
+        long long ex = cx + x, ey = cy + y;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            if (k0 + k < n) tiles[k0 + k] = make_longlong2(ex, ey);
+            ex += t[k].x;
+            ey += t[k].y;
+        }
+        cx += tx;
+        cy += ty;
+    }
+    if (threadIdx.x == 0) {
+        if (edges) st->edges = (unsigned long long)cx;
+        else st->entries = (unsigned long long)cy;
+    }
 }
 
 // Induced edges (r, local[w]) with local[w] > r, one thread per adjacency
@@ -103,74 +275,97 @@ __device__ __forceinline__ int64_t kh_owner(const int64_t *__restrict__ ds, int6
     return lo;
 }
 
-// node r and neighbour w of entry e = blockIdx.x * blockDim.x + threadIdx.x
-// (false past E); the block's node range found once
-__device__ __forceinline__ bool kh_entry(const int32_t *__restrict__ vis, int64_t n, const int64_t *__restrict__ ds,
-                                         int64_t E, const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                                         int64_t &r, int32_t &w) {
+// First pass (u null): the edges of each chunk of KH_CHUNK entries; second:
+// the edges, at the chunk's offset.
+__global__ void __launch_bounds__(KH_TPB) kh_edge_kernel(const int32_t *__restrict__ vis, int64_t n,
+                                                        const int64_t *__restrict__ ds, int64_t E,
+                                                        const int64_t *__restrict__ off,
+                                                        const int32_t *__restrict__ adj,
+                                                        const int32_t *__restrict__ stamp, int32_t epoch,
+                                                        const int32_t *__restrict__ local, longlong2 *chunks,
+                                                        int32_t *u, int32_t *v) {
+    constexpr int PER = KH_CHUNK / KH_TPB;
     __shared__ int64_t rr[2];
-    const int64_t k0 = (int64_t)blockIdx.x * blockDim.x;
-    if (threadIdx.x < 2) rr[threadIdx.x] = kh_owner(ds, 0, n - 1, threadIdx.x == 0 ? k0 : min(E, k0 + (int64_t)blockDim.x) - 1);
+    __shared__ int wc[PER][KH_TPB / 32];
+    const int64_t k0 = (int64_t)blockIdx.x * KH_CHUNK;
+    if (threadIdx.x < 2)
+        rr[threadIdx.x] = kh_owner(ds, 0, n - 1, threadIdx.x == 0 ? k0 : min(E, k0 + (int64_t)KH_CHUNK) - 1);
     __syncthreads();
-    const int64_t e = k0 + threadIdx.x;
-    if (e >= E) return false;
-    r = kh_owner(ds, rr[0], rr[1], e);
-    w = adj[off[vis[r]] + (e - ds[r])];
-    return true;
-}
-
-__global__ void kh_edge_flag_kernel(const int32_t *__restrict__ vis, int64_t n, const int64_t *__restrict__ ds,
-                                    int64_t E, const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                                    const int32_t *__restrict__ stamp, int32_t epoch,
-                                    const int32_t *__restrict__ local, int32_t *__restrict__ keep) {
-    if ((int64_t)blockIdx.x * blockDim.x >= E) return;
-    int64_t r;
-    int32_t w;
-    if (!kh_entry(vis, n, ds, E, off, adj, r, w)) return;
-    keep[(int64_t)blockIdx.x * blockDim.x + threadIdx.x] = stamp[w] == epoch && local[w] > r ? 1 : 0;
-}
-
-__global__ void kh_edge_fill_kernel(const int32_t *__restrict__ vis, int64_t n, const int64_t *__restrict__ ds,
-                                    int64_t E, const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                                    const int32_t *__restrict__ stamp, int32_t epoch,
-                                    const int32_t *__restrict__ local, const int32_t *__restrict__ kpos,
-                                    int32_t *__restrict__ u, int32_t *__restrict__ v) {
-    if ((int64_t)blockIdx.x * blockDim.x >= E) return;
-    int64_t r;
-    int32_t w;
-    if (!kh_entry(vis, n, ds, E, off, adj, r, w)) return;
-    if (stamp[w] == epoch && local[w] > r) {
-        const int64_t k = kpos[(int64_t)blockIdx.x * blockDim.x + threadIdx.x];
-        u[k] = (int32_t)r;
-        v[k] = local[w];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t r[PER], w[PER];
+    unsigned keep = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int64_t e = k0 + k * KH_TPB + threadIdx.x;
+        r[k] = e < E ? (int32_t)kh_owner(ds, rr[0], rr[1], e) : -1;
+        w[k] = e < E ? adj[off[vis[r[k]]] + (e - ds[r[k]])] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (r[k] < 0 || stamp[w[k]] != epoch) continue;
+        w[k] = local[w[k]];
+        if (w[k] > r[k]) keep |= 1u << k;
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const unsigned b = __ballot_sync(0xffffffffu, (keep >> k) & 1u);
+        if (lane == 0) wc[k][warp] = __popc(b);
+    }
+    __syncthreads();
+    int before = 0, total = 0;          // edges of earlier rounds, then of earlier warps of the round
+    if (!u) {
+        if (threadIdx.x != 0) return;
+        for (int k = 0; k < PER; ++k)
+            for (int x = 0; x < KH_TPB / 32; ++x) total += wc[k][x];
+        chunks[blockIdx.x] = make_longlong2(total, 0);
+        return;
+    }
+    const int64_t base = chunks[blockIdx.x].x;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const unsigned b = __ballot_sync(0xffffffffu, (keep >> k) & 1u);
+        int at = before;
+        for (int x = 0; x < KH_TPB / 32; ++x) {
+            if (x < warp) at += wc[k][x];
+            before += wc[k][x];
+        }
+        if ((keep >> k) & 1u) {
+            const int64_t p = base + at + __popc(b & ((1u << lane) - 1u));
+            u[p] = r[k];
+            v[p] = w[k];
+        }
     }
 }
 
 }  // namespace
 
 // Scratch of one extracting context: visited stamps and local ids over the
-// resident graph's nodes, the visit list (at most cap entries).
+// resident graph's nodes, the nodes in the order of discovery and in
+// ascending order (at most cap), the state on the device.
 struct KhopScratch {
-    DevBuf<int32_t> stamp, local, vis;
-    DevBuf<int64_t> deg, dscan, tot;
-    DevBuf<unsigned long long> cnt;
+    DevBuf<int32_t> stamp, local, found, vis, hubs;
+    DevBuf<int64_t> dscan;
+    DevBuf<longlong2> tiles, chunks;
+    DevBuf<KhState> state;
     int32_t epoch = 0;
     int64_t cap = 0;
-    void reserve(bgl_ctx *c, int64_t n_res, int64_t cap_) {
+    void reserve(bgl_ctx *c, const bgl_graph *R, int64_t cap_) {
+        const int64_t n_res = R->n;
         if (stamp.n < (size_t)n_res) {
             stamp.reset(c->alloc, n_res);
             local.reset(c->alloc, n_res);
+            tiles.reset(c->alloc, (n_res + KH_TILE - 1) / KH_TILE);
+            hubs.reset(c->alloc, 2 * R->n_undir / KH_HUB_DEG + 1);
             BGL_CUDA(cudaMemsetAsync(stamp.p, 0, sizeof(int32_t) * n_res, c->stream));
             epoch = 0;
         }
         if (cap < cap_) {
+            found.reset(c->alloc, cap_ + 1);
             vis.reset(c->alloc, cap_ + 1);
-            deg.reset(c->alloc, cap_ + 1);
             dscan.reset(c->alloc, cap_ + 1);
             cap = cap_;
         }
-        if (!tot.p) tot.reset(c->alloc, 1);
-        if (!cnt.p) cnt.reset(c->alloc, 1);
+        if (!state.p) state.reset(c->alloc, 1);
     }
 };
 
@@ -184,65 +379,58 @@ static int64_t khop_extract(bgl_ctx *ctx, const bgl_graph *R, KhopScratch &ws, i
     BGL_REQUIRE(hops >= 0, "khop: hops must be >= 0");
     BGL_REQUIRE(cap >= 1, "khop: max_nodes must be >= 1");
     cudaStream_t s = ctx->stream;
-    ws.reserve(ctx, R->n, cap);
+    cap = std::min(cap, R->n);                     // (no neighbourhood is larger than the graph)
+    ws.reserve(ctx, R, cap);
     const int32_t epoch = ++ws.epoch;
-    kh_seed_kernel<<<1, 1, 0, s>>>(ws.stamp.p, ws.vis.p, (int32_t)seed, epoch);
+    kh_seed_kernel<<<1, 1, 0, s>>>(ws.stamp.p, ws.found.p, (int32_t)seed, epoch, ws.state.p);
     BGL_LAUNCH_CHECK();
-    int64_t total = 1, f0 = 0, nf = 1;
-    for (int h = 0; h < hops && nf > 0; ++h) {
-        kh_deg_kernel<<<kh_blocks(nf), KH_TPB, 0, s>>>(ws.vis.p + f0, nf, R->off.p, ws.deg.p);
-        BGL_LAUNCH_CHECK();
-        scan_exclusive_i64(ctx, ws.deg.p, ws.dscan.p, nf, ws.tot.p);
-        int64_t E = 0;
-        BGL_CUDA(cudaMemcpyAsync(&E, ws.tot.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        BGL_CUDA(cudaMemsetAsync(ws.cnt.p, 0, sizeof(unsigned long long), s));
+    KhState st{};
+    auto fetch = [&] {
+        BGL_CUDA(cudaMemcpyAsync(&st, ws.state.p, sizeof(KhState), cudaMemcpyDeviceToHost, s));
         BGL_CUDA(cudaStreamSynchronize(s));
-        if (E == 0) break;
-        kh_expand_kernel<<<kh_blocks(E), KH_TPB, 0, s>>>(ws.vis.p + f0, nf, ws.dscan.p, E, R->off.p, R->adj.p,
-                                                         ws.stamp.p, epoch, ws.vis.p, total, cap, ws.cnt.p);
+    };
+    const unsigned grid = (unsigned)(4 * ctx->num_sms);
+    for (int h = 0; h < hops; ++h) {
+        kh_hop_kernel<<<grid, KH_TPB, 0, s>>>(R->off.p, R->adj.p, ws.stamp.p, epoch, ws.found.p, cap, ws.hubs.p,
+                                              ws.state.p);
         BGL_LAUNCH_CHECK();
-        unsigned long long add = 0;
-        BGL_CUDA(cudaMemcpyAsync(&add, ws.cnt.p, sizeof(add), cudaMemcpyDeviceToHost, s));
-        BGL_CUDA(cudaStreamSynchronize(s));
-        if (total + (int64_t)add > cap) return -1;
-        f0 = total;
-        nf = (int64_t)add;
-        total += nf;
+        kh_hub_kernel<<<grid, KH_TPB, 0, s>>>(R->off.p, R->adj.p, ws.stamp.p, epoch, ws.found.p, cap, ws.hubs.p,
+                                              ws.state.p);
+        BGL_LAUNCH_CHECK();
+        if (h % 8 == 7) {                          // many hops: stop once nothing is new
+            fetch();
+            if (st.f0 == st.f1 || (int64_t)st.count > cap) break;
+        }
     }
-    const int64_t n = total;
-    // ascending node ids: local id = rank
-    DevBuf<uint32_t> keys(ctx->alloc, n);
-    BGL_CUDA(cudaMemcpyAsync(keys.p, ws.vis.p, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-    radix_sort_u32(ctx, keys.p, nullptr, n, std::max(1, bits_for((uint64_t)R->n)));
-    BGL_CUDA(cudaMemcpyAsync(ws.vis.p, keys.p, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-    kh_local_kernel<<<kh_blocks(n), KH_TPB, 0, s>>>(ws.vis.p, n, ws.local.p);
+    const unsigned tiles = (unsigned)((R->n + KH_TILE - 1) / KH_TILE);
+    kh_mark_kernel<<<tiles, KH_TPB, 0, s>>>(ws.stamp.p, epoch, R->n, R->off.p, ws.tiles.p, nullptr, nullptr, nullptr, 0);
     BGL_LAUNCH_CHECK();
-    // adjacency entries of the neighbourhood's nodes: degree prefix sums
-    kh_deg_kernel<<<kh_blocks(n), KH_TPB, 0, s>>>(ws.vis.p, n, R->off.p, ws.deg.p);
+    kh_tiles_kernel<<<1, KH_TPB, 0, s>>>(ws.tiles.p, tiles, ws.state.p, 0);
     BGL_LAUNCH_CHECK();
-    scan_exclusive_i64(ctx, ws.deg.p, ws.dscan.p, n, ws.tot.p);
-    int64_t E = 0;
-    BGL_CUDA(cudaMemcpyAsync(&E, ws.tot.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    BGL_CUDA(cudaStreamSynchronize(s));
+    kh_mark_kernel<<<tiles, KH_TPB, 0, s>>>(ws.stamp.p, epoch, R->n, R->off.p, ws.tiles.p, ws.vis.p, ws.local.p,
+                                            ws.dscan.p, cap);
+    BGL_LAUNCH_CHECK();
+    fetch();
+    if ((int64_t)st.count > cap) return -1;
+    const int64_t n = (int64_t)st.count, E = (int64_t)st.entries;
     BGL_REQUIRE(E < (int64_t(1) << 31), "khop: more than 2^31 adjacency entries in the neighbourhood");
     m = 0;
-    DevBuf<int32_t> keep(ctx->alloc, std::max<int64_t>(E, 1)), kpos(ctx->alloc, std::max<int64_t>(E, 1));
-    DevBuf<int32_t> ktot(ctx->alloc, 1);
+    const int64_t chunks = (E + KH_CHUNK - 1) / KH_CHUNK;
     if (E > 0) {
-        kh_edge_flag_kernel<<<kh_blocks(E), KH_TPB, 0, s>>>(ws.vis.p, n, ws.dscan.p, E, R->off.p, R->adj.p,
-                                                            ws.stamp.p, epoch, ws.local.p, keep.p);
+        ws.chunks.ensure(ctx->alloc, chunks);
+        kh_edge_kernel<<<(unsigned)chunks, KH_TPB, 0, s>>>(ws.vis.p, n, ws.dscan.p, E, R->off.p, R->adj.p, ws.stamp.p,
+                                                           epoch, ws.local.p, ws.chunks.p, nullptr, nullptr);
         BGL_LAUNCH_CHECK();
-        scan_exclusive_i32(ctx, keep.p, kpos.p, E, ktot.p);
-        int32_t m32 = 0;
-        BGL_CUDA(cudaMemcpyAsync(&m32, ktot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        BGL_CUDA(cudaStreamSynchronize(s));
-        m = m32;
+        kh_tiles_kernel<<<1, KH_TPB, 0, s>>>(ws.chunks.p, chunks, ws.state.p, 1);
+        BGL_LAUNCH_CHECK();
+        fetch();
+        m = (int64_t)st.edges;
     }
     u.reset(ctx->alloc, std::max<int64_t>(m, 1));
     v.reset(ctx->alloc, std::max<int64_t>(m, 1));
     if (m > 0) {
-        kh_edge_fill_kernel<<<kh_blocks(E), KH_TPB, 0, s>>>(ws.vis.p, n, ws.dscan.p, E, R->off.p, R->adj.p,
-                                                            ws.stamp.p, epoch, ws.local.p, kpos.p, u.p, v.p);
+        kh_edge_kernel<<<(unsigned)chunks, KH_TPB, 0, s>>>(ws.vis.p, n, ws.dscan.p, E, R->off.p, R->adj.p, ws.stamp.p,
+                                                           epoch, ws.local.p, ws.chunks.p, u.p, v.p);
         BGL_LAUNCH_CHECK();
     }
     return n;
