@@ -321,6 +321,7 @@ void assemble_device(bgl_graph *g, const bgl_params *p, const float2 *xy_comp, f
     meta_keys_kernel<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(C, p->seed, keys.p, order.p);
     BGL_LAUNCH_CHECK();
     radix_sort_u64(ctx, keys.p, order.p, C, 64);
+    sort_check(ctx);
     // levels: items in order, chunks of K
     std::vector<int64_t> counts(1, C);
     while (counts.back() > 1) counts.push_back((counts.back() + K - 1) / K);

@@ -151,7 +151,8 @@ struct bgl_ctx {
     bgl::Allocator *alloc = nullptr;
     std::string last_error;
     int *d_flag = nullptr;        // device error/flag words (4 ints): [0] per-call checks, [1] ForceAtlas2
-                                  // runs, [2] allocation-free iterations (read by bgl_ctx_sync)
+                                  // runs, [2] allocation-free iterations (read by bgl_ctx_sync),
+                                  // [3] radix sorts (sort_check)
     int *h_flag = nullptr;        // pinned mirror
     unsigned char *noalloc_scratch = nullptr;   // device address of the allocation-free scratch array
     // measured exact/FMM choice by component size octave (fmm_min_nodes = -1)
@@ -211,6 +212,9 @@ void scan_exclusive_i32(bgl_ctx *c, const int32_t *in, int32_t *out, int64_t n, 
 // keys/vals are sorted in place (with internal double buffers).  vals may be null.
 void radix_sort_u64(bgl_ctx *c, uint64_t *keys, uint32_t *vals, int64_t n, int bits);
 void radix_sort_u32(bgl_ctx *c, uint32_t *keys, uint32_t *vals, int64_t n, int bits);
+// BGL_ETIMEOUT if a bounded wait of one of these sorts gave up since the last
+// call (synchronises; the sorts themselves do not)
+void sort_check(bgl_ctx *c);
 
 // Preallocated temporaries for sorting up to `cap` 32-bit keys with values,
 // so that a sort can run inside a captured CUDA graph.

@@ -10,6 +10,8 @@
 // packed (src, dst) keys.  Components: atomicMin hooking of roots plus
 // pointer jumping until no edge joins two roots, which leaves every node
 // labelled with the smallest id of its component.
+#include <algorithm>
+
 #include "bgl_internal.cuh"
 
 namespace bgl {
@@ -137,13 +139,22 @@ __global__ void undirected_keys_kernel(const int32_t *__restrict__ src, const in
     keep[2 * i + 1] = ok;
 }
 
-__global__ void csr_rows_kernel(const uint64_t *__restrict__ k, int64_t m, int b, int32_t *__restrict__ adj,
-                                int64_t *__restrict__ cnt) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    uint64_t mask = (uint64_t(1) << b) - 1;
-    adj[i] = (int32_t)(k[i] & mask);
-    atomicAdd((unsigned long long *)&cnt[k[i] >> b], 1ull);
+// adj and off of the CSR from the m sorted keys (row << b | column): a row
+// starts at the first key that is not below it.  (Counting the rows' entries
+// with atomics, most of them on a few hubs' counters, took 86 us for 1.6e6.)
+__global__ void csr_kernel(const uint64_t *__restrict__ k, int64_t m, int b, int64_t n, int32_t *__restrict__ adj,
+                           int64_t *__restrict__ off) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < m) adj[i] = (int32_t)(k[i] & ((uint64_t(1) << b) - 1));
+    if (i > n) return;
+    const uint64_t row = (uint64_t)i << b;
+    int64_t lo = 0, hi = m;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (k[mid] < row) lo = mid + 1;
+        else hi = mid;
+    }
+    off[i] = lo;
 }
 
 __global__ void iota_kernel(int32_t *a, int64_t n) {
@@ -180,9 +191,42 @@ __global__ void jump_kernel(int32_t *parent, int64_t n) {
     parent[v] = find_root(parent, (int32_t)v);
 }
 
-__global__ void comp_size_kernel(const int32_t *__restrict__ label, int64_t n, int32_t *__restrict__ size) {
-    int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < n) atomicAdd(&size[label[v]], 1);
+// Component sizes.  Most nodes of a graph may be in one component, whose
+// counter every node would queue for (377 us for 680,000 nodes), so a block
+// counts the labels of some of its nodes in shared memory, the others one by
+// one.
+constexpr int SIZE_ITEMS = 8, SIZE_CAND = 4;
+
+__global__ void __launch_bounds__(TPB) comp_size_kernel(const int32_t *__restrict__ label, int64_t n,
+                                                       int32_t *__restrict__ size) {
+    __shared__ int32_t cand[SIZE_CAND], count[SIZE_CAND];
+    const int64_t v0 = (int64_t)blockIdx.x * TPB * SIZE_ITEMS;
+    if (threadIdx.x < SIZE_CAND) {
+        const int64_t v = v0 + (int64_t)threadIdx.x * (TPB * SIZE_ITEMS / SIZE_CAND);
+        cand[threadIdx.x] = v < n ? label[v] : -1;
+        count[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    int32_t l[SIZE_ITEMS];
+#pragma unroll
+    for (int k = 0; k < SIZE_ITEMS; ++k) {
+        const int64_t v = v0 + k * TPB + threadIdx.x;
+        l[k] = v < n ? label[v] : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < SIZE_ITEMS; ++k) {
+        bool open = l[k] >= 0;
+#pragma unroll
+        for (int j = 0; j < SIZE_CAND; ++j) {
+            const bool hit = open && l[k] == cand[j];
+            const unsigned m = __ballot_sync(0xffffffffu, hit);
+            if ((threadIdx.x & 31) == 0 && m) atomicAdd(&count[j], __popc(m));
+            open = open && !hit;
+        }
+        if (open) atomicAdd(&size[l[k]], 1);
+    }
+    __syncthreads();
+    if (threadIdx.x < SIZE_CAND && count[threadIdx.x]) atomicAdd(&size[cand[threadIdx.x]], count[threadIdx.x]);
 }
 
 __global__ void root_flag_kernel(const int32_t *__restrict__ label, int64_t n, int32_t *__restrict__ flag) {
@@ -319,11 +363,9 @@ static void finish_edges(bgl_graph *g, uint64_t *ekey, int64_t m, int b) {
     g->n_undir = mu / 2;
     g->adj.reset(A, mu);
     g->off.reset(A, g->n + 1);
-    DevBuf<int64_t> cnt(A, g->n + 1);
-    BGL_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(int64_t) * (g->n + 1), s));
-    csr_rows_kernel<<<blocks_for(mu), TPB, 0, s>>>(k4.p, mu, b, g->adj.p, cnt.p);
+    csr_kernel<<<blocks_for(std::max<int64_t>(mu, g->n + 1)), TPB, 0, s>>>(k4.p, mu, b, g->n, g->adj.p, g->off.p);
     BGL_LAUNCH_CHECK();
-    scan_exclusive_i64(c, cnt.p, g->off.p, g->n + 1, nullptr);
+    sort_check(c);
     g->has_comp = false;
 }
 
@@ -425,7 +467,7 @@ void components_device(bgl_graph *g) {
     // sizes, component order (size desc, label asc)
     DevBuf<int32_t> size(A, n), flag(A, n), fscan(A, n), tot(A, 1);
     BGL_CUDA(cudaMemsetAsync(size.p, 0, sizeof(int32_t) * (n > 0 ? n : 1), s));
-    comp_size_kernel<<<blocks_for(n), TPB, 0, s>>>(g->label.p, n, size.p);
+    comp_size_kernel<<<blocks_for(n, TPB * SIZE_ITEMS), TPB, 0, s>>>(g->label.p, n, size.p);
     root_flag_kernel<<<blocks_for(n), TPB, 0, s>>>(g->label.p, n, flag.p);
     BGL_LAUNCH_CHECK();
     scan_exclusive_i32(c, flag.p, fscan.p, n, tot.p);
@@ -469,7 +511,7 @@ void components_device(bgl_graph *g) {
     g->h_comp_off.resize(nc + 1);
     BGL_CUDA(cudaMemcpyAsync(g->h_comp_off.data(), g->comp_off.p, sizeof(int64_t) * (nc + 1),
                              cudaMemcpyDeviceToHost, s));
-    BGL_CUDA(cudaStreamSynchronize(s));
+    sort_check(c);
     g->has_comp = true;
     g->kk_max = -1;
 }

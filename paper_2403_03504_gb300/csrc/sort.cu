@@ -1,11 +1,9 @@
 // Device primitives: multi-block exclusive scan and stable LSD radix sort.
 //
 // Scan: reduce-then-scan over tiles of 4096 elements (512 threads x 8).
-// Radix sort: 8-bit digits, tiles of 4096 keys (8 warps x 32 lanes x 16
-// rounds).  Per pass: a per-tile digit histogram (shared-memory integer
-// atomics), one exclusive scan of the digit-major histogram, and a scatter
-// in which each warp ranks its keys by votes on their digits so that equal
-// digits keep their input order (stable).
+// Radix sorts: 8-bit digits, tiles of 4,096 keys, a single kernel a pass
+// (onesweep, below), in which each warp ranks its keys by votes on their
+// digits so that equal digits keep their input order (stable).
 #include <algorithm>
 
 #include "bgl_internal.cuh"
@@ -159,119 +157,7 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d, bool ok) {
     return m;
 }
 
-constexpr int RS_THREADS = 256;
-constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ITEMS = 16;
-constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
-
-template <typename K>
-__global__ void radix_hist_kernel(const K *__restrict__ keys, int64_t n, int shift, int32_t *__restrict__ hist,
-                                  int64_t ntiles) {
-    __shared__ int32_t h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-#pragma unroll 4
-    for (int i = 0; i < RS_ITEMS; ++i) {
-        int64_t k = base + (int64_t)i * RS_THREADS + threadIdx.x;
-        if (k < n) atomicAdd(&h[(unsigned)((keys[k] >> shift) & 0xFF)], 1);
-    }
-    __syncthreads();
-    hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
-}
-
-template <typename K>
-__global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(const K *__restrict__ kin, const uint32_t *__restrict__ vin,
-                                                              K *__restrict__ kout, uint32_t *__restrict__ vout,
-                                                              int64_t n, int shift,
-                                                              const int32_t *__restrict__ offs, int64_t ntiles) {
-    __shared__ int32_t cnt[RS_WARPS][256];
-    __shared__ int32_t gbase[256];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) (&cnt[0][0])[i] = 0;
-    gbase[threadIdx.x] = offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
-    __syncthreads();
-    const unsigned lt = (1u << lane) - 1u;
-    const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * 32 * RS_ITEMS;
-    K key[RS_ITEMS];
-    uint32_t val[RS_ITEMS];
-    int32_t rank[RS_ITEMS];
-#pragma unroll
-    for (int r = 0; r < RS_ITEMS; ++r) {
-        int64_t k = wbase + r * 32 + lane;
-        bool ok = k < n;
-        key[r] = ok ? kin[k] : K(0);
-        val[r] = (ok && vin) ? vin[k] : 0u;
-        unsigned d = (unsigned)((key[r] >> shift) & 0xFF);
-        unsigned peers = digit_peers(d, ok);
-        int before = __popc(peers & lt);
-        int cur = ok ? cnt[warp][d] : 0;
-        __syncwarp();
-        if (ok && before == 0) cnt[warp][d] = cur + __popc(peers);
-        __syncwarp();
-        rank[r] = ok ? (cur + before) : -1;
-    }
-    __syncthreads();
-    {   // exclusive prefix over warps for digit threadIdx.x
-        int d = threadIdx.x;
-        int s = 0;
-#pragma unroll
-        for (int w = 0; w < RS_WARPS; ++w) {
-            int c = cnt[w][d];
-            cnt[w][d] = s;
-            s += c;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < RS_ITEMS; ++r) {
-        if (rank[r] < 0) continue;
-        unsigned d = (unsigned)((key[r] >> shift) & 0xFF);
-        int64_t dst = (int64_t)gbase[d] + cnt[warp][d] + rank[r];
-        kout[dst] = key[r];
-        if (vout) vout[dst] = val[r];
-    }
-}
-
-template <typename K>
-void radix_sort_buffers(bgl_ctx *c, K *keys, uint32_t *vals, int64_t n, int bits, K *ktmp, uint32_t *vtmp,
-                        int32_t *hist, int32_t *tiles) {
-    int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
-    K *ka = keys, *kb = ktmp;
-    uint32_t *va = vals, *vb = vals ? vtmp : nullptr;
-    int passes = 0;
-    for (int shift = 0; shift < bits; shift += 8, ++passes) {
-        radix_hist_kernel<K><<<(unsigned)ntiles, RS_THREADS, 0, c->stream>>>(ka, n, shift, hist, ntiles);
-        BGL_LAUNCH_CHECK();
-        scan_exclusive<int32_t>(c, hist, hist, 256 * ntiles, nullptr, tiles);
-        radix_scatter_kernel<K><<<(unsigned)ntiles, RS_THREADS, 0, c->stream>>>(ka, va, kb, vb, n, shift, hist,
-                                                                                ntiles);
-        BGL_LAUNCH_CHECK();
-        std::swap(ka, kb);
-        std::swap(va, vb);
-    }
-    if (passes & 1) {
-        BGL_CUDA(cudaMemcpyAsync(keys, ka, sizeof(K) * n, cudaMemcpyDeviceToDevice, c->stream));
-        if (vals) BGL_CUDA(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, c->stream));
-    }
-}
-
-inline int64_t rs_tiles(int64_t n) { return (n + RS_TILE - 1) / RS_TILE; }
-inline int64_t scan_tiles_for(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
-
-template <typename K>
-void radix_sort(bgl_ctx *c, K *keys, uint32_t *vals, int64_t n, int bits) {
-    if (n <= 1 || bits <= 0) return;
-    BGL_REQUIRE(n < (int64_t(1) << 31), "radix sort: more than 2^31 keys");
-    const int64_t ntiles = rs_tiles(n);
-    DevBuf<K> kt(c->alloc, n);
-    DevBuf<uint32_t> vt;
-    if (vals) vt.reset(c->alloc, n);
-    DevBuf<int32_t> hist(c->alloc, 256 * ntiles), tiles(c->alloc, scan_tiles_for(256 * ntiles));
-    radix_sort_buffers<K>(c, keys, vals, n, bits, kt.p, vals ? vt.p : nullptr, hist.p, tiles.p);
-}
-
-// ------------------------------------------------------------------ onesweep (32-bit keys)
+// ------------------------------------------------------------------ onesweep
 //
 // Four 8-bit digit passes.  One histogram kernel counts all four digit
 // histograms at once and its last block turns them into global digit
@@ -285,9 +171,54 @@ void radix_sort(bgl_ctx *c, K *keys, uint32_t *vals, int64_t n, int bits) {
 
 // OS_THREADS, OS_ITEMS, OS_TILE: sort_hist.cuh (a caller's histogram kernel uses the same tiles)
 constexpr int OS_WARPS = OS_THREADS / 32;
-constexpr uint32_t OS_AGG = 1u << 30, OS_INC = 2u << 30, OS_MASK = (1u << 30) - 1u;
+// A look-back word: two flag bits above the count, of 32 bits for counts
+// below 2^30 and of 64 bits for more.
+template <typename W>
+struct OsWord {
+    static constexpr W AGG = W(1) << (8 * sizeof(W) - 2), INC = W(2) << (8 * sizeof(W) - 2), MASK = AGG - 1;
+};
 constexpr long long OS_SPIN = 1ll << 24;
 constexpr int OS_LB = 8;           // look-back window (predecessor tiles per step)
+
+// Decoupled look-back of digit d: publishes the tile's count `own` and returns
+// the sum of the earlier tiles' counts.  OS_LB predecessors per step: their
+// status words are loaded together, then taken newest first until an
+// inclusive one.
+template <typename W>
+__device__ __forceinline__ uint32_t os_look_back(volatile W *st, int tile, int d, uint32_t own, int *err,
+                                                 const OsWait &wait) {
+    uint32_t excl = 0;
+    if (tile == 0) {
+        if (!wait.stall_first) st[d] = OsWord<W>::INC | own;
+        return 0;
+    }
+    st[(int64_t)tile * 256 + d] = OsWord<W>::AGG | own;
+    bool done = false;
+    for (int t = tile - 1; t >= 0 && !done; t -= OS_LB) {
+        W v[OS_LB];
+#pragma unroll
+        for (int w = 0; w < OS_LB; ++w) v[w] = t - w >= 0 ? (W)st[(int64_t)(t - w) * 256 + d] : OsWord<W>::INC;
+#pragma unroll
+        for (int w = 0; w < OS_LB; ++w) {
+            if (done) break;
+            long long it = 0;
+            while ((v[w] & ~OsWord<W>::MASK) == 0) {
+                if (++it > wait.spin) {
+                    atomicOr(err, 1);
+                    v[w] = OsWord<W>::INC;
+                    break;
+                }
+                __nanosleep(32);
+                v[w] = st[(int64_t)(t - w) * 256 + d];
+            }
+            excl += (uint32_t)(v[w] & OsWord<W>::MASK);
+            if (v[w] & OsWord<W>::INC) done = true;
+        }
+    }
+    __threadfence();
+    st[(int64_t)tile * 256 + d] = OsWord<W>::INC | (excl + own);
+    return excl;
+}
 
 // digit histograms of the keys, OS_ITEMS per thread
 __global__ void __launch_bounds__(OS_THREADS) os_hist_kernel(const uint32_t *__restrict__ keys, int64_t n, OsHist h) {
@@ -387,40 +318,7 @@ __global__ void __launch_bounds__(OS_THREADS, OS_THREADS > 512 ? 1 : 2) os_scatt
             if (lane >= o) x += y;
         }
         if (lane == 31) wsum[warp] = x;
-        volatile uint32_t *st = status;
-        const uint32_t own = (uint32_t)s;
-        uint32_t excl = 0;
-        if (tile == 0) {
-            if (!wait.stall_first) st[d] = OS_INC | own;
-        } else {
-            st[(int64_t)tile * 256 + d] = OS_AGG | own;
-            // look back OS_LB predecessors per step: their status words are
-            // loaded together, then taken newest first until an inclusive one
-            bool done = false;
-            for (int t = tile - 1; t >= 0 && !done; t -= OS_LB) {
-                uint32_t v[OS_LB];
-#pragma unroll
-                for (int w = 0; w < OS_LB; ++w) v[w] = t - w >= 0 ? (uint32_t)st[(int64_t)(t - w) * 256 + d] : (uint32_t)OS_INC;
-#pragma unroll
-                for (int w = 0; w < OS_LB; ++w) {
-                    if (done) break;
-                    long long it = 0;
-                    while ((v[w] & ~OS_MASK) == 0) {
-                        if (++it > wait.spin) {
-                            atomicOr(err, 1);
-                            v[w] = OS_INC;
-                            break;
-                        }
-                        __nanosleep(32);
-                        v[w] = st[(int64_t)(t - w) * 256 + d];
-                    }
-                    excl += v[w] & OS_MASK;
-                    if (v[w] & OS_INC) done = true;
-                }
-            }
-            __threadfence();
-            st[(int64_t)tile * 256 + d] = OS_INC | (excl + own);
-        }
+        const uint32_t excl = os_look_back<uint32_t>(status, tile, d, (uint32_t)s, err, wait);
         gofs[d] = base[d] + excl;
     }
     __syncthreads();
@@ -476,7 +374,207 @@ __global__ void __launch_bounds__(OS_THREADS, OS_THREADS > 512 ? 1 : 2) os_scatt
     }
 }
 
+// The sort of the graph build: keys of 32 or 64 bits, with values or without,
+// any number of passes.  One kernel counts the digits of every pass, one
+// kernel a pass moves the keys.  A digit count, a scan of the tiles' counts in
+// three kernels and a scatter took 46 us a pass for 800,000 64-bit keys with
+// values and 60 for 1,600,000 without; a pass takes 18 and 25.
+template <typename K>
+__global__ void __launch_bounds__(OS_THREADS) sweep_hist_kernel(const K *__restrict__ keys, int64_t n, int passes,
+                                                               uint32_t *hist, uint32_t *base, unsigned *counter) {
+    __shared__ uint32_t sh[sizeof(K)][256];
+    __shared__ uint32_t ws[OS_THREADS / 32];
+    __shared__ bool last;
+    for (int i = threadIdx.x; i < passes * 256; i += OS_THREADS) (&sh[0][0])[i] = 0;
+    __syncthreads();
+    const int64_t i0 = (int64_t)blockIdx.x * OS_TILE + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < OS_ITEMS; ++r) {
+        const int64_t i = i0 + (int64_t)r * OS_THREADS;
+        if (i >= n) break;
+        const K k = keys[i];
+        for (int d = 0; d < passes; ++d) atomicAdd(&sh[d][(unsigned)(k >> (8 * d)) & 0xFFu], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < passes * 256; i += OS_THREADS)
+        if ((&sh[0][0])[i]) atomicAdd(&hist[i], (&sh[0][0])[i]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i0b = 0; i0b < passes * 256; i0b += OS_THREADS) {
+        const int i = i0b + threadIdx.x;
+        const uint32_t v = i < passes * 256 ? __ldcg(&hist[i]) : 0u;
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) ws[warp] = x;
+        __syncthreads();
+        uint32_t pre = 0;
+        for (int w = warp & ~7; w < warp; ++w) pre += ws[w];
+        if (i < passes * 256) base[i] = pre + x - v;
+        __syncthreads();
+    }
+}
+
+template <typename K, bool VALS, typename W>
+__global__ void __launch_bounds__(OS_THREADS, 2) sweep_kernel(const K *__restrict__ kin,
+                                                              const uint32_t *__restrict__ vin, K *__restrict__ kout,
+                                                              uint32_t *__restrict__ vout, int64_t n, int shift,
+                                                              const uint32_t *__restrict__ base, W *status,
+                                                              unsigned *ticket, int *err, OsWait wait) {
+    __shared__ __align__(4) uint16_t cnt[OS_WARPS][256];
+    __shared__ uint32_t gofs[256];
+    __shared__ int32_t lstart[256];
+    __shared__ int32_t wsum[8];
+    __shared__ K skey[OS_TILE];
+    __shared__ int tile_s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) tile_s = (*(volatile int *)err & 1) ? -1 : (int)atomicAdd(ticket, 1u);
+    for (int i = threadIdx.x; i < OS_WARPS * 128; i += OS_THREADS) reinterpret_cast<uint32_t *>(cnt)[i] = 0;
+    __syncthreads();
+    const int tile = tile_s;
+    if (tile < 0) return;              // a wait gave up: see os_scatter_kernel
+    const int64_t t0 = (int64_t)tile * OS_TILE;
+    const int tcount = (int)(n - t0 < OS_TILE ? n - t0 : OS_TILE);
+    const unsigned lt = (1u << lane) - 1u;
+    const int w0 = warp * 32 * OS_ITEMS;
+    K key[OS_ITEMS];
+    uint32_t val[OS_ITEMS];
+    int32_t rank[OS_ITEMS];
+#pragma unroll
+    for (int r = 0; r < OS_ITEMS; ++r) {
+        const int i = w0 + r * 32 + lane;
+        key[r] = i < tcount ? kin[t0 + i] : K(0);
+        val[r] = VALS && i < tcount ? vin[t0 + i] : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < OS_ITEMS; ++r) {
+        const bool ok = w0 + r * 32 + lane < tcount;
+        const unsigned d = (unsigned)(key[r] >> shift) & 0xFFu;
+        const unsigned peers = digit_peers(d, ok);
+        const int before = __popc(peers & lt);
+        const int cur = ok ? cnt[warp][d] : 0;
+        __syncwarp();
+        if (ok && before == 0) cnt[warp][d] = (uint16_t)(cur + __popc(peers));
+        __syncwarp();
+        rank[r] = ok ? cur + before : -1;
+    }
+    __syncthreads();
+    const bool digit = threadIdx.x < 256;
+    int s = 0, x = 0;
+    if (digit) {
+        const int d = threadIdx.x;
+#pragma unroll
+        for (int w = 0; w < OS_WARPS; ++w) {
+            const int c = cnt[w][d];
+            cnt[w][d] = (uint16_t)s;
+            s += c;
+        }
+        x = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        gofs[d] = base[d] + os_look_back<W>(status, tile, d, (uint32_t)s, err, wait);
+    }
+    __syncthreads();
+    if (digit) {
+        int pre = 0;
+        for (int w = 0; w < warp; ++w) pre += wsum[w];
+        lstart[threadIdx.x] = pre + x - s;
+    }
+    __syncthreads();
+    // keys to their tile-local sorted position, then coalesced runs to
+    // global; the values the same way through the same memory
+    int lp[OS_ITEMS];
+#pragma unroll
+    for (int r = 0; r < OS_ITEMS; ++r) {
+        const unsigned d = (unsigned)(key[r] >> shift) & 0xFFu;
+        lp[r] = lstart[d] + cnt[warp][d] + rank[r];
+        if (rank[r] >= 0) skey[lp[r]] = key[r];
+    }
+    __syncthreads();
+    uint32_t dst[OS_ITEMS];
+#pragma unroll
+    for (int r = 0; r < OS_ITEMS; ++r) {
+        const int i = r * OS_THREADS + threadIdx.x;
+        const K k = i < tcount ? skey[i] : K(0);
+        const unsigned d = (unsigned)(k >> shift) & 0xFFu;
+        dst[r] = gofs[d] + (uint32_t)(i - lstart[d]);
+        if (i < tcount) kout[dst[r]] = k;
+    }
+    if constexpr (VALS) {
+        uint32_t *sval = reinterpret_cast<uint32_t *>(skey);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < OS_ITEMS; ++r)
+            if (rank[r] >= 0) sval[lp[r]] = val[r];
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < OS_ITEMS; ++r) {
+            const int i = r * OS_THREADS + threadIdx.x;
+            if (i < tcount) vout[dst[r]] = sval[i];
+        }
+    }
+}
+
 inline int64_t os_tiles(int64_t n) { return (n + OS_TILE - 1) / OS_TILE; }
+
+// Sorts in place on bits [0, bits), look-back words of type W.  A wait that
+// gives up sets the context's d_flag[3], which sort_check reports.
+template <typename K, bool VALS, typename W>
+void radix_sort_words(bgl_ctx *c, K *keys, uint32_t *vals, int64_t n, int bits) {
+    const int64_t nt = os_tiles(n);
+    const int passes = (bits + 7) / 8;
+    DevBuf<K> kt(c->alloc, n);
+    DevBuf<uint32_t> vt;
+    if (VALS) vt.reset(c->alloc, n);
+    // digit counts, pass tickets and arrival counter (zero at first), digit bases
+    const size_t counts = (size_t)passes * 256;
+    DevBuf<uint32_t> ws(c->alloc, counts + 16), base(c->alloc, counts);
+    BGL_CUDA(cudaMemsetAsync(ws.p, 0, ws.bytes(), c->stream));
+    unsigned *tickets = ws.p + counts;
+    // look-back words, zero before their pass: for every pass, or for many tiles one set for all
+    const bool each = nt > 16384;
+    DevBuf<W> status(c->alloc, 256 * (size_t)nt * (each ? 1 : passes));
+    if (!each) BGL_CUDA(cudaMemsetAsync(status.p, 0, status.bytes(), c->stream));
+    sweep_hist_kernel<K><<<(unsigned)nt, OS_THREADS, 0, c->stream>>>(keys, n, passes, ws.p, base.p, tickets + 15);
+    BGL_LAUNCH_CHECK();
+    OsWait wait;
+    wait.spin = OS_SPIN;
+    K *ka = keys, *kb = kt.p;
+    uint32_t *va = vals, *vb = vt.p;
+    for (int d = 0; d < passes; ++d) {
+        if (each) BGL_CUDA(cudaMemsetAsync(status.p, 0, status.bytes(), c->stream));
+        sweep_kernel<K, VALS, W><<<(unsigned)nt, OS_THREADS, 0, c->stream>>>(
+            ka, va, kb, vb, n, 8 * d, base.p + 256 * d, status.p + (each ? 0 : (size_t)d * 256 * nt), tickets + d,
+            c->d_flag + 3, wait);
+        BGL_LAUNCH_CHECK();
+        std::swap(ka, kb);
+        std::swap(va, vb);
+    }
+    if (passes & 1) {
+        BGL_CUDA(cudaMemcpyAsync(keys, ka, sizeof(K) * n, cudaMemcpyDeviceToDevice, c->stream));
+        if (VALS) BGL_CUDA(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, c->stream));
+    }
+}
+
+template <typename K, bool VALS>
+void radix_sort(bgl_ctx *c, K *keys, uint32_t *vals, int64_t n, int bits) {
+    if (n <= 1 || bits <= 0) return;
+    BGL_REQUIRE(n < (int64_t(1) << 31), "radix sort: more than 2^31 keys");
+    if (n < (int64_t(1) << 30)) radix_sort_words<K, VALS, uint32_t>(c, keys, vals, n, bits);
+    else radix_sort_words<K, VALS, unsigned long long>(c, keys, vals, n, bits);
+}
 
 }  // namespace
 
@@ -487,10 +585,19 @@ void scan_exclusive_i32(bgl_ctx *c, const int32_t *in, int32_t *out, int64_t n, 
     scan_exclusive<int32_t>(c, in, out, n, d_total);
 }
 void radix_sort_u64(bgl_ctx *c, uint64_t *keys, uint32_t *vals, int64_t n, int bits) {
-    radix_sort<uint64_t>(c, keys, vals, n, bits);
+    if (vals) radix_sort<uint64_t, true>(c, keys, vals, n, bits);
+    else radix_sort<uint64_t, false>(c, keys, nullptr, n, bits);
 }
 void radix_sort_u32(bgl_ctx *c, uint32_t *keys, uint32_t *vals, int64_t n, int bits) {
-    radix_sort<uint32_t>(c, keys, vals, n, bits);
+    if (vals) radix_sort<uint32_t, true>(c, keys, vals, n, bits);
+    else radix_sort<uint32_t, false>(c, keys, nullptr, n, bits);
+}
+void sort_check(bgl_ctx *c) {
+    BGL_CUDA(cudaMemcpyAsync(c->h_flag + 3, c->d_flag + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    BGL_CUDA(cudaStreamSynchronize(c->stream));
+    if (!c->h_flag[3]) return;
+    BGL_CUDA(cudaMemsetAsync(c->d_flag + 3, 0, sizeof(int), c->stream));
+    fail(BGL_ETIMEOUT, "radix sort: a bounded device-side wait gave up");
 }
 
 void SortWorkspace::reserve(Allocator *a, int64_t n, cudaStream_t s) {
