@@ -94,6 +94,54 @@ void Allocator::free(void *p) {
     live_.erase(it);
 }
 
+StreamPool::~StreamPool() {
+    for (auto &kv : streams_) cudaStreamDestroy(kv.second);
+    for (auto e : events_) cudaEventDestroy(e);
+}
+
+cudaStream_t StreamPool::stream(int priority) {
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        auto it = streams_.find(priority);
+        if (it != streams_.end()) {
+            cudaStream_t s = it->second;
+            streams_.erase(it);
+            return s;
+        }
+    }
+    cudaStream_t s = nullptr;
+    BGL_CUDA(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, priority));
+    return s;
+}
+
+void StreamPool::give(cudaStream_t s, int priority) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const bool idle = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+    std::lock_guard<std::mutex> lk(mu_);
+    if (idle && streams_.size() < KEEP) streams_.emplace(priority, s);
+    else cudaStreamDestroy(s);
+}
+
+cudaEvent_t StreamPool::event() {
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        if (!events_.empty()) {
+            cudaEvent_t e = events_.back();
+            events_.pop_back();
+            return e;
+        }
+    }
+    cudaEvent_t e = nullptr;
+    BGL_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    return e;
+}
+
+void StreamPool::give(cudaEvent_t e) {
+    std::lock_guard<std::mutex> lk(mu_);
+    if (events_.size() < KEEP) events_.push_back(e);
+    else cudaEventDestroy(e);
+}
+
 void check_params(const bgl_params *p) {
     BGL_REQUIRE(p != nullptr, "params is NULL");
     BGL_REQUIRE(p->kk_max_nodes >= 0 && p->kk_max_nodes <= 255, "kk_max_nodes must be in [0, 255]");
@@ -199,29 +247,15 @@ void layout_device(bgl_graph *g, const bgl_params *p, float *d_xy_out) {
     const int64_t q_fa2 = g->h_comp_off[g->n_fa2];
     std::unique_ptr<KkRun, void (*)(KkRun *)> kk(kk_prepare(g, g->n_fa2, g->n_comp), kk_destroy);
     const int nk = kk_classes(kk.get());
-    std::vector<cudaStream_t> ks;
-    std::vector<cudaEvent_t> kev;
-    auto release = [&] {
-        for (auto e : kev) cudaEventDestroy(e);
-        for (auto st : ks) cudaStreamDestroy(st);
-        kev.clear();
-        ks.clear();
-    };
+    std::vector<PoolStream> ks(nk);
+    std::vector<PoolEvent> kev(nk + 1);
     try {
         // the classes of larger components, whose chains of node steps are the
         // longest, get their SMs first
         int lowest = 0, highest = 0;
         BGL_CUDA(cudaDeviceGetStreamPriorityRange(&lowest, &highest));
-        for (int i = 0; i < nk; ++i) {
-            cudaStream_t st;
-            BGL_CUDA(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, std::min(lowest, highest + i)));
-            ks.push_back(st);
-        }
-        for (int i = 0; i < nk + 1; ++i) {
-            cudaEvent_t e;
-            BGL_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-            kev.push_back(e);
-        }
+        for (int i = 0; i < nk; ++i) ks[i].take(c, std::min(lowest, highest + i));
+        for (auto &e : kev) e.take(c);
         // small components: Kamada-Kawai, one stream per size class, forked
         // from and joined back to stream s
         SideWork kk_work = [&](cudaStream_t s) {
@@ -245,10 +279,8 @@ void layout_device(bgl_graph *g, const bgl_params *p, float *d_xy_out) {
     } catch (...) {
         // nothing may still write to the scratch when it goes back to the allocator
         cudaDeviceSynchronize();
-        release();
         throw;
     }
-    release();
     if (g->n > 0 && p->assemble) {
         assemble_device(g, p, xy.p, reinterpret_cast<float2 *>(d_xy_out), nullptr);
     } else if (g->n > 0) {

@@ -139,6 +139,26 @@ struct DevBuf {
     size_t bytes() const { return sizeof(T) * n; }
 };
 
+// The streams and events that a layout needs for itself, kept by the context
+// between calls (making and destroying them took some 100 us of a call):
+// at most KEEP of each, any priority, given back when a plan or a run ends.
+// One that is still part of a stream capture (a call that failed) is
+// destroyed instead.
+class StreamPool {
+  public:
+    ~StreamPool();
+    cudaStream_t stream(int priority);
+    void give(cudaStream_t s, int priority);
+    cudaEvent_t event();                      // without timing
+    void give(cudaEvent_t e);
+
+  private:
+    static constexpr size_t KEEP = 32;
+    std::mutex mu_;
+    std::multimap<int, cudaStream_t> streams_;
+    std::vector<cudaEvent_t> events_;
+};
+
 }  // namespace bgl
 
 // ------------------------------------------------------------- handles
@@ -149,6 +169,7 @@ struct bgl_ctx {
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
     bgl::Allocator *alloc = nullptr;
+    bgl::StreamPool pool;
     std::string last_error;
     int *d_flag = nullptr;        // device error/flag words (4 ints): [0] per-call checks, [1] ForceAtlas2
                                   // runs, [2] allocation-free iterations (read by bgl_ctx_sync),
@@ -161,6 +182,39 @@ struct bgl_ctx {
 };
 
 namespace bgl {
+// a stream and an event from a context's pool, given back at the end
+struct PoolStream {
+    bgl_ctx *c = nullptr;
+    int priority = 0;
+    cudaStream_t s = nullptr;
+    PoolStream() = default;
+    PoolStream(const PoolStream &) = delete;
+    PoolStream &operator=(const PoolStream &) = delete;
+    void take(bgl_ctx *ctx, int prio = 0) {
+        c = ctx;
+        priority = prio;
+        s = ctx->pool.stream(prio);
+    }
+    ~PoolStream() {
+        if (s) c->pool.give(s, priority);
+    }
+    operator cudaStream_t() const { return s; }
+};
+struct PoolEvent {
+    bgl_ctx *c = nullptr;
+    cudaEvent_t e = nullptr;
+    PoolEvent() = default;
+    PoolEvent(const PoolEvent &) = delete;
+    PoolEvent &operator=(const PoolEvent &) = delete;
+    void take(bgl_ctx *ctx) {
+        c = ctx;
+        e = ctx->pool.event();
+    }
+    ~PoolEvent() {
+        if (e) c->pool.give(e);
+    }
+    operator cudaEvent_t() const { return e; }
+};
 // device address of the allocation-free iteration's scratch array on the
 // current device (cudaGetSymbolAddress; allocates nothing)
 void *noalloc_scratch_address();
@@ -228,8 +282,6 @@ struct SortWorkspace {
 // (v = the value of sorted key i, as int bits) instead of the sorted values.
 void radix_sort_u32_ws(bgl_ctx *c, SortWorkspace &ws, uint32_t *keys, uint32_t *vals, int64_t n, int bits,
                        const float2 *gxy = nullptr, const float *gmass = nullptr, float4 *gpts = nullptr);
-// nonzero if a bounded wait of a workspace sort gave up (synchronises)
-int sort_workspace_error(bgl_ctx *c, SortWorkspace &ws);
 // The same sort in two halves, so that a caller's kernel can count the digit
 // histograms while it makes the keys: radix_sort_u32_ws_begin clears the
 // counts and returns them; every block of the caller's kernel (OS_THREADS)

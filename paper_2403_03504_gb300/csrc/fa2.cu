@@ -19,6 +19,7 @@
 // The sequence has fixed launch shapes, so it is captured once as the body of
 // a device-side WHILE loop in a CUDA graph: one launch runs all iterations.  Every sum has a fixed order, so
 // runs are bitwise reproducible.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 
@@ -491,24 +492,18 @@ __global__ void attraction_gravity_kernel(const float2 *__restrict__ xy, const f
     fa[ch.q - qbase] = make_float2(sx - km * p.x, sy - km * p.y);
 }
 
-__global__ void heavy_flag_kernel(const int64_t *__restrict__ coff, int64_t q0, int64_t n, int32_t *__restrict__ flag) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// A node of more than HEAVY_DEG adjacency entries: its place and entries
+struct HeavyNode {
+    int64_t q, e0, e1;
+};
+__global__ void heavy_kernel(const int64_t *__restrict__ coff, int64_t q0, int64_t n, HeavyNode *out, int64_t cap,
+                             unsigned long long *count) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    flag[i] = (coff[q0 + i + 1] - coff[q0 + i]) > HEAVY_DEG;
-}
-
-__global__ void heavy_list_kernel(const int32_t *__restrict__ flag, const int32_t *__restrict__ fscan, int64_t q0,
-                                  int64_t n, int32_t *__restrict__ heavy) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && flag[i]) heavy[fscan[i]] = (int32_t)(q0 + i);
-}
-
-__global__ void heavy_rows_kernel(const int32_t *__restrict__ heavy, const int64_t *__restrict__ coff, int64_t nh,
-                                  int64_t *__restrict__ rows) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nh) return;
-    rows[2 * i] = coff[heavy[i]];
-    rows[2 * i + 1] = coff[heavy[i] + 1];
+    const int64_t e0 = coff[q0 + i], e1 = coff[q0 + i + 1];
+    if (e1 - e0 <= HEAVY_DEG) return;
+    const unsigned long long k = atomicAdd(count, 1ull);
+    if ((int64_t)k < cap) out[k] = HeavyNode{q0 + i, e0, e1};
 }
 
 // K3 for the FMM's components (the exact kernel sums its own): tiles of 256
@@ -792,8 +787,8 @@ struct Fa2Run {
     int64_t n_chunks = 0;
     std::vector<FmmPlan *> fmm;   // one per FMM component
     std::vector<int64_t> fmm_comp;
-    cudaStream_t side = nullptr;  // attraction + gravity, beside the repulsion
-    cudaEvent_t ev_fork = nullptr, ev_fa = nullptr;
+    PoolStream side;              // attraction + gravity, beside the repulsion
+    PoolEvent ev_fork, ev_fa;
     // A run whose only component is on the FMM path iterates fused: the FMM's
     // combine pass sums swing and traction and sets s_G, and one kernel moves
     // the points and makes the next evaluation's root square (no swing/traction
@@ -872,16 +867,13 @@ struct Fa2Run {
         BGL_CUDA(cudaMemsetAsync(iter.p, 0, sizeof(int), s));
         loop.reset(A, 1);
         if (!fmm.empty()) heavy_setup();
-        BGL_CUDA(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
-        BGL_CUDA(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
-        BGL_CUDA(cudaEventCreateWithFlags(&ev_fa, cudaEventDisableTiming));
+        side.take(g->ctx);
+        ev_fork.take(g->ctx);
+        ev_fa.take(g->ctx);
         BGL_CUDA(cudaStreamSynchronize(s));
     }
     ~Fa2Run() {
         for (auto *pl : fmm) fmm_destroy(pl);
-        if (ev_fork) cudaEventDestroy(ev_fork);
-        if (ev_fa) cudaEventDestroy(ev_fa);
-        if (side) cudaStreamDestroy(side);
     }
 
     // the FMM components' nodes of high degree: chunks of HEAVY_CHUNK adjacency entries
@@ -889,34 +881,33 @@ struct Fa2Run {
         Allocator *A = g->ctx->alloc;
         cudaStream_t s = g->ctx->stream;
         const int64_t nf = q_fmm - q0;
-        DevBuf<int32_t> flag(A, nf), fscan(A, nf), tot(A, 1);
-        heavy_flag_kernel<<<nblocks(nf, 256), 256, 0, s>>>(g->coff.p, q0, nf, flag.p);
+        // the count and the first of them in one copy; there are at most 2 E / HEAVY_DEG
+        constexpr int64_t FIRST = 256;
+        const int64_t cap = std::max<int64_t>(FIRST, 2 * g->n_undir / HEAVY_DEG + 1);
+        DevBuf<HeavyNode> heavy(A, cap + 1);
+        unsigned long long *count = reinterpret_cast<unsigned long long *>(heavy.p);
+        BGL_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned long long), s));
+        heavy_kernel<<<nblocks(nf, 256), 256, 0, s>>>(g->coff.p, q0, nf, heavy.p + 1, cap, count);
         BGL_LAUNCH_CHECK();
-        scan_exclusive_i32(g->ctx, flag.p, fscan.p, nf, tot.p);
-        int32_t nh = 0;
-        BGL_CUDA(cudaMemcpyAsync(&nh, tot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        std::vector<HeavyNode> hn(FIRST + 1);
+        BGL_CUDA(cudaMemcpyAsync(hn.data(), heavy.p, sizeof(HeavyNode) * hn.size(), cudaMemcpyDeviceToHost, s));
         BGL_CUDA(cudaStreamSynchronize(s));
-        std::vector<HeavyChunk> hc;
-        if (nh > 0) {
-            DevBuf<int32_t> heavy(A, nh);
-            heavy_list_kernel<<<nblocks(nf, 256), 256, 0, s>>>(flag.p, fscan.p, q0, nf, heavy.p);
-            BGL_LAUNCH_CHECK();
-            DevBuf<int64_t> hrow(A, 2 * (size_t)nh);
-            heavy_rows_kernel<<<nblocks(nh, 256), 256, 0, s>>>(heavy.p, g->coff.p, nh, hrow.p);
-            BGL_LAUNCH_CHECK();
-            std::vector<int32_t> hq(nh);
-            std::vector<int64_t> ho(2 * (size_t)nh);
-            BGL_CUDA(cudaMemcpyAsync(hq.data(), heavy.p, sizeof(int32_t) * nh, cudaMemcpyDeviceToHost, s));
-            BGL_CUDA(cudaMemcpyAsync(ho.data(), hrow.p, sizeof(int64_t) * 2 * nh, cudaMemcpyDeviceToHost, s));
+        const int32_t nh = (int32_t) * reinterpret_cast<unsigned long long *>(hn.data());
+        if (nh > FIRST) {
+            hn.resize(nh + 1);
+            BGL_CUDA(cudaMemcpyAsync(hn.data(), heavy.p, sizeof(HeavyNode) * hn.size(), cudaMemcpyDeviceToHost, s));
             BGL_CUDA(cudaStreamSynchronize(s));
-            for (int32_t h = 0; h < nh; ++h) {
-                const int64_t r0 = ho[2 * h], r1 = ho[2 * h + 1];
-                const int32_t first = (int32_t)hc.size();
-                const int32_t nchunk = (int32_t)((r1 - r0 + HEAVY_CHUNK - 1) / HEAVY_CHUNK);
-                for (int32_t j = 0; j < nchunk; ++j)
-                    hc.push_back(HeavyChunk{hq[h], h, first, nchunk, r0 + (int64_t)j * HEAVY_CHUNK,
-                                            std::min<int64_t>(r1, r0 + (int64_t)(j + 1) * HEAVY_CHUNK)});
-            }
+        }
+        hn.erase(hn.begin());
+        hn.resize(nh);
+        std::sort(hn.begin(), hn.end(), [](const HeavyNode &x, const HeavyNode &y) { return x.q < y.q; });
+        std::vector<HeavyChunk> hc;
+        for (int32_t h = 0; h < nh; ++h) {
+            const int32_t first = (int32_t)hc.size();
+            const int32_t nchunk = (int32_t)((hn[h].e1 - hn[h].e0 + HEAVY_CHUNK - 1) / HEAVY_CHUNK);
+            for (int32_t j = 0; j < nchunk; ++j)
+                hc.push_back(HeavyChunk{(int32_t)hn[h].q, h, first, nchunk, hn[h].e0 + (int64_t)j * HEAVY_CHUNK,
+                                        std::min<int64_t>(hn[h].e1, hn[h].e0 + (int64_t)(j + 1) * HEAVY_CHUNK)});
         }
         n_chunks = (int64_t)hc.size();
         chunks.reset(A, hc.size());
@@ -972,7 +963,7 @@ struct Fa2Run {
         }
         for (size_t k = 0; k < fmm.size(); ++k) {
             BGL_RANGE("ForceAtlas2: repulsion by the FMM (Section 3.2.1)");
-            fmm_repulsion(fmm[k], xy, qbase, f.p, q0, att ? fa.p : nullptr, att ? ev_fa : nullptr);
+            fmm_repulsion(fmm[k], xy, qbase, f.p, q0, att ? fa.p : nullptr, att ? (cudaEvent_t)ev_fa : nullptr);
         }
         if (att && !fmm.empty()) BGL_CUDA(cudaStreamWaitEvent(s, ev_fa, 0));
         if (exact.n_blk > 0) {

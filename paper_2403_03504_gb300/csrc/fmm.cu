@@ -2335,13 +2335,8 @@ struct FmmPlan {
     int hmask = 0;
     DevBuf<float> binom;
     SortWorkspace sortws;
-    cudaStream_t side = nullptr;          // second stream for the concurrent branch
-    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    ~FmmPlan() {
-        for (auto &e : ev)
-            if (e) cudaEventDestroy(e);
-        if (side) cudaStreamDestroy(side);
-    }
+    PoolStream side;          // second stream for the concurrent branch
+    PoolEvent ev[4];
 };
 
 FmmPlan *fmm_create(bgl_graph *g, const bgl_params *p, int64_t c) {
@@ -2447,8 +2442,8 @@ FmmPlan *fmm_create(bgl_graph *g, const bgl_params *p, int64_t c) {
         }
         pl->binom.reset(A, BN * BN);
         BGL_CUDA(cudaMemcpyAsync(pl->binom.p, bn.data(), sizeof(float) * bn.size(), cudaMemcpyHostToDevice, s));
-        BGL_CUDA(cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking));
-        for (auto &e : pl->ev) BGL_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        pl->side.take(ctx);
+        for (auto &e : pl->ev) e.take(ctx);
         BGL_CUDA(cudaStreamSynchronize(s));
         pl->grid_p = ctx->num_sms * 8;
     } catch (...) {
@@ -2876,7 +2871,6 @@ int fmm_error(FmmPlan *pl) {
     int e = 0;
     BGL_CUDA(cudaMemcpyAsync(&e, pl->err.p, sizeof(int), cudaMemcpyDeviceToHost, pl->g->ctx->stream));
     BGL_CUDA(cudaStreamSynchronize(pl->g->ctx->stream));
-    if (sort_workspace_error(pl->g->ctx, pl->sortws)) e |= ERR_SPIN;
     // a failed evaluation may have stopped before its combine pass: empty
     // every child slot again so that the plan stays usable
     if (e) {

@@ -665,14 +665,6 @@ void radix_sort_u32_ws(bgl_ctx *c, SortWorkspace &ws, uint32_t *keys, uint32_t *
     radix_sort_u32_ws_scatter(c, ws, keys, vals, n, gxy, gmass, gpts);
 }
 
-int sort_workspace_error(bgl_ctx *c, SortWorkspace &ws) {
-    int e = 0;
-    int *err = reinterpret_cast<int *>(reinterpret_cast<unsigned *>(ws.hist.p + 8 * 256) + 5);
-    BGL_CUDA(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    BGL_CUDA(cudaStreamSynchronize(c->stream));
-    return e;
-}
-
 int bits_for(uint64_t v) {
     int b = 0;
     while (b < 64 && (v >> b) != 0) ++b;
