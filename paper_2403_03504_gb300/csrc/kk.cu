@@ -46,6 +46,15 @@ __global__ void init_positions_kernel(const int32_t *__restrict__ nodes, const i
     xy[q - qbase] = initial_position(seed, seed_id_of(sid, nodes[q]));
 }
 
+// rsqrtf for a normal argument: r^2 is at least 1e-30, so what rsqrtf does
+// for denormal ones is left out (20,000 components of 3 to 200 nodes 37.9 ms
+// with it, 33.9 without, the same bits)
+__device__ __forceinline__ float kk_rsqrt(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 template <int G>
 __device__ __forceinline__ float group_sum(float v, unsigned mask) {
 #pragma unroll
@@ -420,7 +429,7 @@ __global__ void kk_kernel(KKArgs a) {
                 for (int k = 0; k < M; ++k) {
                     const float2 d = __ffma2_rn(pi[k], make_float2(-1.f, -1.f), pm);   // p_m - p_i, exact sign flip
                     const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, 1e-30f));
-                    const float rinv = rsqrtf(r2);
+                    const float rinv = kk_rsqrt(r2);
                     // w = k l / r^3 (k l first: zero for the node itself, whose
                     // 1/r^3 would overflow), c = k - w r^2 = k (1 - l / r)
                     const float w = (kl[k].y * rinv) * (rinv * rinv);
