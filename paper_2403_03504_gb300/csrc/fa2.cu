@@ -558,18 +558,6 @@ __global__ void swing_traction_kernel(SwingArgs a, const Tile *__restrict__ tile
     }
 }
 
-// Control of the device-side loop: count the iteration and keep looping
-// while below `iters` (count null: no loop).
-struct LoopCtl {
-    cudaGraphConditionalHandle h = 0;
-    int *count = nullptr;
-    int iters = 0;
-};
-__device__ __forceinline__ void loop_step(const LoopCtl &l) {
-    const int k = ++*l.count;
-    cudaGraphSetConditional(l.h, k < l.iters ? 1u : 0u);
-}
-
 // K4: node speeds and the position update; the first thread also steps the
 // loop (LOOP; a kernel without it can be profiled)
 template <bool LOOP>
@@ -985,7 +973,7 @@ struct Fa2Run {
             // K3 in the FMM's combine pass, K4 with the next root square
             forces(0);
             BGL_RANGE("ForceAtlas2: node update (Section 3.2)");
-            fmm_update_root(fmm[0], xy, qbase, f.p, fprev.p, q0);
+            fmm_update_root(fmm[0], xy, qbase, f.p, fprev.p, q0, loop_ctl);
             return;
         }
         const SwingArgs a = swing_args(d_stats);
@@ -1004,13 +992,6 @@ struct Fa2Run {
         BGL_LAUNCH_CHECK();
     }
 };
-
-namespace {
-
-// End of a loop iteration (fused runs, whose last kernel is the FMM's).
-__global__ void loop_ctrl_kernel(LoopCtl loop) { loop_step(loop); }
-
-}  // namespace
 
 // With BGL_HOST_LOOP=1 in the environment, the iterations are launched
 // from the host as one captured-iteration graph each instead of a device-side
@@ -1087,11 +1068,10 @@ static void run_iterations_host(Fa2Run &run, int iters, double *d_stats, const S
 
 // Iterations per turn of the device-side loop.  A turn costs some 4 us beside
 // its kernels: of a 25 us iteration of exact sums four to a turn save 3.5 us
-// (871 nodes: 24.8 us an iteration with one, 22.6 two, 21.5 four, 20.9 eight),
-// but every captured iteration also costs the instantiation of its kernels:
-// an FMM iteration of nineteen takes 30 us longer to instantiate than it saves
-// in ten turns (8,888 nodes: 106.0 and 104.0 us an iteration with one and two).
-static int loop_unroll(const Fa2Run &run) { return run.fmm.empty() ? 4 : 1; }
+// (871 nodes: 24.8 us an iteration with one, 22.6 two, 21.5 four, 20.9 eight).
+// Every captured iteration also costs the instantiation of its kernels, some
+// 30 us for an FMM iteration, which two to a turn win back in 24 iterations.
+static int loop_unroll(const Fa2Run &run, int iters) { return run.fmm.empty() ? 4 : (iters >= 24 ? 2 : 1); }
 
 // `n` iterations captured on s into graph `into` (null: a new graph, which
 // is returned); loop: stepped by the last one.  Adds the kernels to `kernels`.
@@ -1109,10 +1089,6 @@ static cudaGraph_t capture_iterations(Fa2Run &run, double *d_stats, int n, cudaG
     cudaGraph_t captured = nullptr;
     try {
         for (int k = 0; k < n; ++k) run.iteration(d_stats, k + 1 < n ? LoopCtl{} : loop);
-        if (run.fused && loop.count) {
-            loop_ctrl_kernel<<<1, 1, 0, s>>>(loop);
-            BGL_LAUNCH_CHECK();
-        }
     } catch (...) {
         ctx->alloc->forbid = false;
         cudaStreamEndCapture(s, &captured);
@@ -1152,7 +1128,7 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
     BGL_CUDA(cudaGraphCreate(&graph, 0));
     int64_t kernels = 0;
     try {
-        const int unroll = loop_unroll(run), turns = iters / unroll, rest = iters - turns * unroll;
+        const int unroll = loop_unroll(run, iters), turns = iters / unroll, rest = iters - turns * unroll;
         cudaGraphNode_t rnode = nullptr;
         if (rest > 0) {
             cudaGraph_t child = capture_iterations(run, d_stats, rest, nullptr, LoopCtl{}, kernels);

@@ -7,8 +7,21 @@
 //   s_n = ks s_G / (1 + s_G sqrt(swing_n)), at most ksmax / |F_t(n)|;
 //   p_n += s_n F_t(n).
 #pragma once
+#include <cuda_runtime.h>
 
 namespace bgl {
+
+// Control of the device-side loop: count the iteration and keep looping
+// while below `iters` (count null: no loop).
+struct LoopCtl {
+    cudaGraphConditionalHandle h = 0;
+    int *count = nullptr;
+    int iters = 0;
+};
+__device__ __forceinline__ void loop_step(const LoopCtl &l) {
+    const int k = ++*l.count;
+    cudaGraphSetConditional(l.h, k < l.iters ? 1u : 0u);
+}
 
 // swing and traction terms of one node
 __device__ __forceinline__ void fa2_swing_terms(float2 F, float2 P, float m, int variant, float &sw, float &tr) {

@@ -536,6 +536,11 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_count_kernel(const uint32_t
     if (threadIdx.x < NLEV) tcnt[threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
 }
 
+// Trees of up to this many tiles have no scan kernel (tree_emit_kernel<true>):
+// the tree phase of 27,980 points (28 tiles) takes 28.1 us with it and 23.0
+// without, of 69,696 (69) 28.1 and 22.8, of 125,799 (123) 27.1 and 23.3.
+constexpr int TREE_OWN_TILES = 128;
+
 // Exclusive scan of the (level, tile) counts (one block of SCAN_THREADS,
 // counts staged in shared memory with coalesced loads, SCAN_ITEMS
 // consecutive counts per thread); level offsets.
@@ -620,9 +625,14 @@ __global__ void __launch_bounds__(SCAN_THREADS) tree_scan_kernel(int *tcnt, int 
 // its boxes as it made them waited for a probe and an exchange at each, up to
 // four a level (11.3 us in a tree of 301 boxes).  Levels above the deepest leaf level met in the tile
 // (of its points and of the point before it) hold no box start or end.
+//
+// OWN: of few tiles, each block sums the (level, tile) counts that come
+// before its own itself, and block 0 does the rest of tree_scan_kernel's work.
+template <bool OWN>
 __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const int8_t *__restrict__ cl,
                                                                 const int8_t *__restrict__ lam,
-                                                                const int *__restrict__ tcnt, int ntiles, int Bmax) {
+                                                                const int *__restrict__ tcnt, int ntiles, int Bmax,
+                                                                const int *gmax, int *sortskip) {
     if (aborted(T.err)) return;
     constexpr int NW = TREE_THREADS / 32;
     constexpr int R = TREE_TILE / TREE_THREADS;        // rounds per warp
@@ -632,10 +642,44 @@ __global__ void __launch_bounds__(TREE_THREADS) tree_emit_kernel(Tree T, const i
     __shared__ int smax;
     __shared__ int stc[NLEV];          // the tile's offset at every level, loaded once
     if (threadIdx.x == 0) smax = 0;
-    if (threadIdx.x < NLEV) stc[threadIdx.x] = tcnt[threadIdx.x * ntiles + blockIdx.x];
-    __syncthreads();
     const unsigned epoch = *T.epoch;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (OWN) {
+        __shared__ int sall[NLEV];     // boxes of the level
+        constexpr int M = TREE_OWN_TILES / 32;
+        for (int L = warp; L < NLEV; L += NW) {
+            int v[M], pre = 0, all = 0;
+#pragma unroll
+            for (int m = 0; m < M; ++m) v[m] = m * 32 + lane < ntiles ? tcnt[L * ntiles + m * 32 + lane] : 0;
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                all += v[m];
+                pre += m * 32 + lane < (int)blockIdx.x ? v[m] : 0;
+            }
+            all = __reduce_add_sync(0xffffffffu, all);
+            pre = __reduce_add_sync(0xffffffffu, pre);
+            if (lane == 0) {
+                stc[L] = pre;
+                sall[L] = all;
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const int all = lane < NLEV ? sall[lane] : 0, upto = warp_incl_scan(all);
+            if (lane < NLEV) stc[lane] += upto - all;
+            if (blockIdx.x == 0) {
+                if (lane < NLEV) T.levoff[lane] = upto - all;
+                if (lane == NLEV - 1) {
+                    T.levoff[NLEV] = upto;
+                    if (upto > Bmax) atomicOr(T.err, ERR_BOX_OVERFLOW);
+                    *sortskip = *gmax <= 7 ? 2 : 0;
+                }
+            }
+        }
+    } else {
+        if (threadIdx.x < NLEV) stc[threadIdx.x] = tcnt[threadIdx.x * ntiles + blockIdx.x];
+    }
+    __syncthreads();
     const int t0 = blockIdx.x * TREE_TILE;
     const unsigned lt = (1u << lane) - 1u;
     int c[R], la[R], lp[R];
@@ -1881,10 +1925,16 @@ __global__ void __launch_bounds__(256) combine_kernel(LeafArgs la, int n) {
 // Several points a thread, as in combine_kernel (one: 13.1 us for 556,277).
 constexpr int UPDATE_POINTS = 4;
 
+// (LOOP: the first thread also steps the device-side loop)
+template <bool LOOP>
 __global__ void __launch_bounds__(256) update_root_kernel(float2 *xy, const float2 *__restrict__ f, float2 *fprev, int n,
                                                          const double *sg, float ks, float ksmax, int *bad,
                                                          float4 *__restrict__ part, unsigned *counter, Root *root,
-                                                         int *err, unsigned *epoch, int *tickets, OsHist h) {
+                                                         int *err, unsigned *epoch, int *tickets, OsHist h,
+                                                         LoopCtl loop) {
+    if constexpr (LOOP) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) loop_step(loop);
+    }
     evaluation_clear(tickets, h);
     const float g = (float)*sg;
     float mnx = INFINITY, mxx = -INFINITY, mny = INFINITY, mxy = -INFINITY;
@@ -2561,10 +2611,17 @@ static void phase_tree(FmmPlan *pl, const Tree &T, cudaStream_t s) {
     tree_count_kernel<<<pl->ntiles, TREE_THREADS, 0, s>>>(pl->key.p, pl->n, pl->S, pl->cl.p, pl->lam.p, pl->tcnt.p,
                                                           pl->ntiles, pl->sortskip.p, pl->tickets.p + 6, pl->err.p);
     BGL_LAUNCH_CHECK();
+    if (pl->ntiles <= TREE_OWN_TILES) {
+        tree_emit_kernel<true><<<pl->ntiles, TREE_THREADS, 0, s>>>(T, pl->cl.p, pl->lam.p, pl->tcnt.p, pl->ntiles,
+                                                                   pl->Bmax, pl->tickets.p + 6, pl->sortskip.p);
+        BGL_LAUNCH_CHECK();
+        return;
+    }
     tree_scan_kernel<<<1, SCAN_THREADS, 0, s>>>(pl->tcnt.p, pl->ntiles, pl->levoff.p, pl->Bmax, pl->err.p,
                                                 pl->tickets.p + 6, pl->sortskip.p);
     BGL_LAUNCH_CHECK();
-    tree_emit_kernel<<<pl->ntiles, TREE_THREADS, 0, s>>>(T, pl->cl.p, pl->lam.p, pl->tcnt.p, pl->ntiles, pl->Bmax);
+    tree_emit_kernel<false><<<pl->ntiles, TREE_THREADS, 0, s>>>(T, pl->cl.p, pl->lam.p, pl->tcnt.p, pl->ntiles,
+                                                                pl->Bmax, nullptr, nullptr);
     BGL_LAUNCH_CHECK();
 }
 
@@ -2845,12 +2902,14 @@ void fmm_root(FmmPlan *pl, const float2 *xy, int64_t qbase) {
     BGL_LAUNCH_CHECK();
 }
 
-void fmm_update_root(FmmPlan *pl, float2 *xy, int64_t qbase, const float2 *f, float2 *fprev, int64_t fbase) {
+void fmm_update_root(FmmPlan *pl, float2 *xy, int64_t qbase, const float2 *f, float2 *fprev, int64_t fbase,
+                     const LoopCtl &loop) {
     bgl_ctx *ctx = pl->g->ctx;
     const OsHist h = radix_sort_u32_ws_begin(ctx, pl->sortws, pl->n, false);
-    update_root_kernel<<<nblk(pl->n, 256 * UPDATE_POINTS), 256, 0, ctx->stream>>>(
+    (loop.count ? update_root_kernel<true> : update_root_kernel<false>)<<<nblk(pl->n, 256 * UPDATE_POINTS), 256, 0, ctx->stream>>>(
         xy + (pl->q0 - qbase), f + (pl->q0 - fbase), fprev + (pl->q0 - fbase), pl->n, pl->fz.sg, pl->fz.ks,
-        pl->fz.ksmax, pl->fz.bad, pl->part.p, pl->counter.p, pl->root.p, pl->err.p, pl->epoch.p, pl->tickets.p, h);
+        pl->fz.ksmax, pl->fz.bad, pl->part.p, pl->counter.p, pl->root.p, pl->err.p, pl->epoch.p, pl->tickets.p, h,
+        loop);
     BGL_LAUNCH_CHECK();
 }
 

@@ -1,6 +1,7 @@
 // Fast Multipole Method for the ForceAtlas2 repulsion (Section 3.2.1).
 #pragma once
 #include "bgl_internal.cuh"
+#include "fa2_update.cuh"
 
 namespace bgl {
 
@@ -38,8 +39,10 @@ struct FmmFuse {
 void fmm_fuse(FmmPlan *pl, const FmmFuse &fz);
 // the root square of positions xy (before the first fused evaluation)
 void fmm_root(FmmPlan *pl, const float2 *xy, int64_t qbase);
-// p += s F, F_{t-1} <- F for every point, and the next root square
-void fmm_update_root(FmmPlan *pl, float2 *xy, int64_t qbase, const float2 *f, float2 *fprev, int64_t fbase);
+// p += s F, F_{t-1} <- F for every point, and the next root square; steps
+// the device-side loop if there is one
+void fmm_update_root(FmmPlan *pl, float2 *xy, int64_t qbase, const float2 *f, float2 *fprev, int64_t fbase,
+                     const LoopCtl &loop);
 
 // Counts and per-phase device times of `reps` evaluations (synchronises);
 // out[15]: boxes, leaves, depth, P2P pairs, M2L translations, M2P terms,
