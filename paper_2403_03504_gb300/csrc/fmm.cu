@@ -50,6 +50,8 @@
 
 #include <cstdlib>
 
+#include <cooperative_groups.h>
+
 #include "fa2_update.cuh"
 #include "fmm.cuh"
 #include "p2p.cuh"
@@ -58,6 +60,8 @@
 namespace bgl {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int MAXLEV = 16;
 constexpr int NLEV = MAXLEV + 1;
@@ -414,6 +418,23 @@ __global__ void bbox_kernel(const float2 *__restrict__ xy, int n, float4 *__rest
     bbox_reduce_root(mnx, mxx, mny, mxy, part, counter, root, err, epoch);
 }
 
+__device__ __forceinline__ int warp_incl_scan(int v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    return v;
+}
+
+// Morton key of a point: its cell of the root square's 65536 x 65536
+__device__ __forceinline__ uint32_t point_key(float2 p, float ox, float oy, float sc) {
+    const float fx = floorf((p.x - ox) * sc), fy = floorf((p.y - oy) * sc);
+    const int qx = (int)fminf(fmaxf(fx, 0.f), 65535.f), qy = (int)fminf(fmaxf(fy, 0.f), 65535.f);
+    return spread_bits((uint32_t)qx) | (spread_bits((uint32_t)qy) << 1);
+}
+
 constexpr int KEY_ITEMS = OS_ITEMS;      // one key block per radix tile
 
 __global__ void __launch_bounds__(OS_THREADS) keys_kernel(const float2 *__restrict__ xy, int n, const Root *__restrict__ root,
@@ -431,9 +452,7 @@ __global__ void __launch_bounds__(OS_THREADS) keys_kernel(const float2 *__restri
 #pragma unroll
     for (int r = 0; r < KEY_ITEMS; ++r) {
         const int i = i0 + r * OS_THREADS;
-        const float fx = floorf((p[r].x - ox) * sc), fy = floorf((p[r].y - oy) * sc);
-        const int qx = (int)fminf(fmaxf(fx, 0.f), 65535.f), qy = (int)fminf(fmaxf(fy, 0.f), 65535.f);
-        k[r] = spread_bits((uint32_t)qx) | (spread_bits((uint32_t)qy) << 1);
+        k[r] = point_key(p[r], ox, oy, sc);
         if (i < n) {
             key[i] = k[r];
             idx[i] = (uint32_t)i;
@@ -445,14 +464,149 @@ __global__ void __launch_bounds__(OS_THREADS) keys_kernel(const float2 *__restri
 }
 
 
-__device__ __forceinline__ int warp_incl_scan(int v) {
-    const int lane = threadIdx.x & 31;
+// Keys, sort and gather of a component of up to SMALL_TILES radix tiles in one
+// kernel: a thread-block cluster with a block per tile makes the keys, and
+// each pass ranks a tile's keys, exchanges the blocks' digit counts through
+// distributed shared memory (no look-back, no separate digit count) and moves
+// the keys through global memory.  Same order as the separate kernels (a
+// stable sort on the same bits).  On a few tiles those are all latency: keys,
+// two passes that return at once and two that do not; an iteration on 8,888
+// points takes 87.1 us with them and 79.5 with this, on 27,980 104.5 and 94.7.
+constexpr int SMALL_TILES = 8;         // the portable cluster size
+
+__global__ void __launch_bounds__(OS_THREADS) points_small_kernel(const float2 *__restrict__ xy,
+                                                                 const float *__restrict__ mass, int n,
+                                                                 const Root *__restrict__ root, uint32_t *key_out,
+                                                                 uint32_t *k0, uint32_t *v0, uint32_t *k1,
+                                                                 uint32_t *v1, float4 *__restrict__ pts,
+                                                                 const int *__restrict__ sortskip) {
+    constexpr int NW = OS_THREADS / 32;
+    __shared__ __align__(4) uint16_t cnt[NW][256];
+    __shared__ uint32_t gofs[256], tcount[256];
+    __shared__ int32_t lstart[256], wsum[8], gsum[8];
+    __shared__ uint32_t skey[OS_TILE], sval[OS_TILE];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank_c = (int)cluster.block_rank(), blocks = (int)cluster.num_blocks();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int t0 = rank_c * OS_TILE;
+    const int tcnt_ = min(OS_TILE, n - t0);
+    const int w0 = warp * 32 * OS_ITEMS;
+    const int skip = *sortskip;
+    uint32_t key[OS_ITEMS], val[OS_ITEMS];
+    {
+        const float ox = root->oxf, oy = root->oyf, sc = root->scale;
+        float2 p[OS_ITEMS];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
+        for (int r = 0; r < OS_ITEMS; ++r) {
+            const int i = w0 + r * 32 + lane;
+            p[r] = i < tcnt_ ? xy[t0 + i] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int r = 0; r < OS_ITEMS; ++r) {
+            key[r] = point_key(p[r], ox, oy, sc);
+            val[r] = (uint32_t)(t0 + w0 + r * 32 + lane);
+        }
     }
-    return v;
+    for (int d = skip; d < 4; ++d) {
+        const int shift = 8 * d;
+        if (d > skip) {
+            const uint32_t *kin = (d - skip - 1) & 1 ? k1 : k0, *vin = (d - skip - 1) & 1 ? v1 : v0;
+#pragma unroll
+            for (int r = 0; r < OS_ITEMS; ++r) {
+                const int i = w0 + r * 32 + lane;
+                key[r] = i < tcnt_ ? __ldcg(&kin[t0 + i]) : 0u;        // (other blocks' writes: not from L1)
+                val[r] = i < tcnt_ ? __ldcg(&vin[t0 + i]) : 0u;
+            }
+        }
+        for (int i = threadIdx.x; i < NW * 128; i += OS_THREADS) reinterpret_cast<uint32_t *>(cnt)[i] = 0;
+        __syncthreads();
+        int32_t rank[OS_ITEMS];
+#pragma unroll
+        for (int r = 0; r < OS_ITEMS; ++r) {
+            const bool ok = w0 + r * 32 + lane < tcnt_;
+            const unsigned g = (key[r] >> shift) & 0xFFu;
+            const unsigned peers = digit_peers(g, ok);
+            const int before = __popc(peers & lt);
+            const int cur = ok ? cnt[warp][g] : 0;
+            __syncwarp();
+            if (ok && before == 0) cnt[warp][g] = (uint16_t)(cur + __popc(peers));
+            __syncwarp();
+            rank[r] = ok ? cur + before : -1;
+        }
+        __syncthreads();
+        const bool digit = threadIdx.x < 256;
+        int s = 0, x = 0;
+        if (digit) {
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const int c = cnt[w][threadIdx.x];
+                cnt[w][threadIdx.x] = (uint16_t)s;
+                s += c;
+            }
+            tcount[threadIdx.x] = (uint32_t)s;
+        }
+        cluster.sync();
+        int all = 0, pre = 0, y = 0;
+        if (digit) {
+            for (int b = 0; b < blocks; ++b) {
+                const int c = (int)cluster.map_shared_rank(&tcount[0], b)[threadIdx.x];
+                pre += b < rank_c ? c : 0;
+                all += c;
+            }
+            x = warp_incl_scan(s);
+            y = warp_incl_scan(all);
+            if (lane == 31) {
+                wsum[warp] = x;
+                gsum[warp] = y;
+            }
+        }
+        __syncthreads();
+        if (digit) {
+            int px = 0, py = 0;
+            for (int w = 0; w < warp; ++w) {
+                px += wsum[w];
+                py += gsum[w];
+            }
+            lstart[threadIdx.x] = px + x - s;
+            gofs[threadIdx.x] = (uint32_t)(py + y - all + pre);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < OS_ITEMS; ++r) {
+            if (rank[r] < 0) continue;
+            const unsigned g = (key[r] >> shift) & 0xFFu;
+            const int lp = lstart[g] + cnt[warp][g] + rank[r];
+            skey[lp] = key[r];
+            sval[lp] = val[r];
+        }
+        __syncthreads();
+        uint32_t *kout = d == 3 ? key_out : ((d - skip) & 1 ? k1 : k0), *vout = (d - skip) & 1 ? v1 : v0;
+        uint32_t ok_[OS_ITEMS], ov[OS_ITEMS];
+        float2 p[OS_ITEMS];
+        float m[OS_ITEMS];
+#pragma unroll
+        for (int r = 0; r < OS_ITEMS; ++r) {
+            const int i = r * OS_THREADS + threadIdx.x;
+            ok_[r] = i < tcnt_ ? skey[i] : 0u;
+            ov[r] = i < tcnt_ ? sval[i] : 0u;
+            p[r] = d == 3 && i < tcnt_ ? xy[ov[r]] : make_float2(0.f, 0.f);
+            m[r] = d == 3 && i < tcnt_ ? mass[ov[r]] : 0.f;
+        }
+#pragma unroll
+        for (int r = 0; r < OS_ITEMS; ++r) {
+            const int i = r * OS_THREADS + threadIdx.x;
+            if (i >= tcnt_) continue;
+            const unsigned g = (ok_[r] >> shift) & 0xFFu;
+            const uint32_t dst = gofs[g] + (uint32_t)(i - lstart[g]);
+            kout[dst] = ok_[r];
+            if (d == 3) pts[dst] = make_float4(p[r].x, p[r].y, m[r], __int_as_float((int)ov[r]));
+            else vout[dst] = ov[r];
+        }
+        // the pass's writes before the next one's reads, and no block writes
+        // its counts again, or leaves, while another reads them
+        cluster.sync();
+    }
 }
 
 // ---------------------------------------------------------------- tree build
@@ -2594,6 +2748,25 @@ static void phase_points(FmmPlan *pl, const float2 *xl, cudaStream_t s) {
             bbox_kernel<<<bbox_blocks(pl), 256, 0, s>>>(xl, n, pl->part.p, pl->counter.p, pl->root.p, pl->err.p,
                                                        pl->epoch.p, pl->tickets.p, h);
             BGL_LAUNCH_CHECK();
+        }
+        // (the test aid of the look-back's waits needs the passes that have one)
+        if (n <= SMALL_TILES * OS_TILE && !pl->wait.stall_first) {
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = nblk(n, OS_TILE);
+            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(nblk(n, OS_TILE));
+            cfg.blockDim = dim3(OS_THREADS);
+            cfg.stream = s;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            BGL_CUDA(cudaLaunchKernelEx(&cfg, points_small_kernel, xl, ml, n, (const Root *)pl->root.p, pl->key.p,
+                                        pl->sortws.keys.p, pl->sortws.vals.p, pl->sortws.keys2.p, pl->sortws.vals2.p,
+                                        pl->pts.p, (const int *)pl->sortskip.p));
+            BGL_LAUNCH_CHECK();
+            ctx->stream = keep;
+            return;
         }
         keys_kernel<<<nblk(n, OS_TILE), OS_THREADS, 0, s>>>(xl, n, pl->root.p, pl->key.p, pl->idx.p, h);
         BGL_LAUNCH_CHECK();

@@ -143,20 +143,6 @@ void scan_exclusive(bgl_ctx *c, const T *in, T *out, int64_t n, T *d_total, T *t
 
 // ------------------------------------------------------------------ radix sort
 
-// The lanes with the same 8-bit digit, of those with `ok` set (the result is
-// meaningless in the others).  Eight votes: __match_any_sync takes several
-// times as long (it was 40 % of a radix pass's time).
-__device__ __forceinline__ unsigned digit_peers(unsigned d, bool ok) {
-    unsigned m = __ballot_sync(0xffffffffu, ok);
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const bool set = (d >> b) & 1u;
-        const unsigned v = __ballot_sync(0xffffffffu, set);
-        m &= set ? v : ~v;
-    }
-    return m;
-}
-
 // ------------------------------------------------------------------ onesweep
 //
 // Four 8-bit digit passes.  One histogram kernel counts all four digit

@@ -12,6 +12,20 @@ constexpr int OS_ITEMS = OS_TILE / OS_THREADS;
 static_assert(OS_THREADS % 256 == 0 && OS_ITEMS >= 1 && OS_ITEMS <= 32,
               "whole groups of 256 digits; a thread's keys are tracked in a 32-bit mask");
 
+// The lanes with the same 8-bit digit, of those with `ok` set (the result is
+// meaningless in the others).  Eight votes: __match_any_sync takes several
+// times as long (it was 40 % of a radix pass's time).
+__device__ __forceinline__ unsigned digit_peers(unsigned d, bool ok) {
+    unsigned m = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool set = (d >> b) & 1u;
+        const unsigned v = __ballot_sync(0xffffffffu, set);
+        m &= set ? v : ~v;
+    }
+    return m;
+}
+
 // Adds the block's keys (key[r] for the bits r of `valid`) to the four 8-bit
 // digit histograms of h (shared-memory counts, then one global atomic per
 // non-empty bin); the last block to arrive writes the exclusive digit bases
