@@ -175,6 +175,7 @@ struct bgl_ctx {
                                   // runs, [2] allocation-free iterations (read by bgl_ctx_sync),
                                   // [3] radix sorts (sort_check)
     int *h_flag = nullptr;        // pinned mirror
+    bool sort_waits = false;      // a radix sort of several tiles ran since the last sort_check
     unsigned char *noalloc_scratch = nullptr;   // device address of the allocation-free scratch array
     // measured exact/FMM choice by component size octave (fmm_min_nodes = -1)
     std::mutex tune_mu;
@@ -266,9 +267,14 @@ void scan_exclusive_i32(bgl_ctx *c, const int32_t *in, int32_t *out, int64_t n, 
 // keys/vals are sorted in place (with internal double buffers).  vals may be null.
 void radix_sort_u64(bgl_ctx *c, uint64_t *keys, uint32_t *vals, int64_t n, int bits);
 void radix_sort_u32(bgl_ctx *c, uint32_t *keys, uint32_t *vals, int64_t n, int bits);
-// BGL_ETIMEOUT if a bounded wait of one of these sorts gave up since the last
-// call (synchronises; the sorts themselves do not)
+// The sorts wait for each other's tiles, with a bound.  After a wait that gave
+// up the output is not a permutation of the input, so whatever uses sorted
+// values or keys as indices comes after sort_check (synchronises if there
+// was anything to wait for; BGL_ETIMEOUT), or after sort_fetch, the
+// caller's own synchronisation and sort_fetched.
 void sort_check(bgl_ctx *c);
+void sort_fetch(bgl_ctx *c);
+void sort_fetched(bgl_ctx *c);
 
 // Preallocated temporaries for sorting up to `cap` 32-bit keys with values,
 // so that a sort can run inside a captured CUDA graph.

@@ -326,7 +326,9 @@ static void finish_edges(bgl_graph *g, uint64_t *ekey, int64_t m, int b) {
     scan_exclusive_i32(c, hd.p, hs.p, m, tot.p);
     int32_t md = 0;
     BGL_CUDA(cudaMemcpyAsync(&md, tot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    sort_fetch(c);
     BGL_CUDA(cudaStreamSynchronize(s));
+    sort_fetched(c);
     DevBuf<uint64_t> uk(A, md);
     compact_kernel<uint64_t><<<blocks_for(m), TPB, 0, s>>>(ekey, hd.p, hs.p, m, uk.p);
     BGL_LAUNCH_CHECK();
@@ -356,7 +358,9 @@ static void finish_edges(bgl_graph *g, uint64_t *ekey, int64_t m, int b) {
     scan_exclusive_i32(c, h3.p, s3.p, mk, tot.p);
     int32_t mu = 0;
     BGL_CUDA(cudaMemcpyAsync(&mu, tot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    sort_fetch(c);
     BGL_CUDA(cudaStreamSynchronize(s));
+    sort_fetched(c);
     DevBuf<uint64_t> k4(A, mu);
     compact_kernel<uint64_t><<<blocks_for(mk), TPB, 0, s>>>(k3.p, h3.p, s3.p, mk, k4.p);
     BGL_LAUNCH_CHECK();
@@ -365,7 +369,6 @@ static void finish_edges(bgl_graph *g, uint64_t *ekey, int64_t m, int b) {
     g->off.reset(A, g->n + 1);
     csr_kernel<<<blocks_for(std::max<int64_t>(mu, g->n + 1)), TPB, 0, s>>>(k4.p, mu, b, g->n, g->adj.p, g->off.p);
     BGL_LAUNCH_CHECK();
-    sort_check(c);
     g->has_comp = false;
 }
 
@@ -404,11 +407,13 @@ void graph_build_device(bgl_graph *g, int64_t T, int64_t n_in, int64_t n_out, co
     scan_exclusive_i32(c, head.p, hscan.p, M, tot.p);
     int32_t U = 0;
     BGL_CUDA(cudaMemcpyAsync(&U, tot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    sort_fetch(c);
+    BGL_CUDA(cudaStreamSynchronize(s));
+    sort_fetched(c);
     BGL_CUDA(cudaMemsetAsync(isfirst.p, 0, sizeof(int32_t) * (M > 0 ? M : 1), s));
     mark_first_kernel<<<blocks_for(M), TPB, 0, s>>>(head.p, spos.p, M, isfirst.p);
     BGL_LAUNCH_CHECK();
     scan_exclusive_i32(c, isfirst.p, rank.p, M, nullptr);
-    BGL_CUDA(cudaStreamSynchronize(s));
     g->n_addr = U;
     g->n = T + U;
     g->addr.reset(A, U);
@@ -480,6 +485,7 @@ void components_device(bgl_graph *g) {
     comp_key_kernel<<<blocks_for(n), TPB, 0, s>>>(flag.p, fscan.p, size.p, n, b, ckey.p);
     BGL_LAUNCH_CHECK();
     radix_sort_u64(c, ckey.p, nullptr, nc, 2 * b);
+    sort_check(c);
     g->comp_label.reset(A, nc);
     g->comp_off.reset(A, nc + 1);
     DevBuf<int64_t> csize(A, nc + 1);
@@ -492,6 +498,7 @@ void components_device(bgl_graph *g) {
     node_key_kernel<<<blocks_for(n), TPB, 0, s>>>(g->label.p, cidx.p, n, nkey.p, nval.p);
     BGL_LAUNCH_CHECK();
     radix_sort_u32(c, nkey.p, nval.p, n, nc > 1 ? bits_for((uint64_t)(nc - 1)) : 0);
+    sort_check(c);
     g->nodes.reset(A, n);
     g->pos.reset(A, n);
     g->node_comp.reset(A, n);
@@ -511,7 +518,7 @@ void components_device(bgl_graph *g) {
     g->h_comp_off.resize(nc + 1);
     BGL_CUDA(cudaMemcpyAsync(g->h_comp_off.data(), g->comp_off.p, sizeof(int64_t) * (nc + 1),
                              cudaMemcpyDeviceToHost, s));
-    sort_check(c);
+    BGL_CUDA(cudaStreamSynchronize(s));
     g->has_comp = true;
     g->kk_max = -1;
 }

@@ -535,6 +535,7 @@ void radix_sort_words(bgl_ctx *c, K *keys, uint32_t *vals, int64_t n, int bits) 
     if (!each) BGL_CUDA(cudaMemsetAsync(status.p, 0, status.bytes(), c->stream));
     sweep_hist_kernel<K><<<(unsigned)nt, OS_THREADS, 0, c->stream>>>(keys, n, passes, ws.p, base.p, tickets + 15);
     BGL_LAUNCH_CHECK();
+    if (nt > 1) c->sort_waits = true;      // (one tile waits for nobody)
     OsWait wait;
     wait.spin = OS_SPIN;
     K *ka = keys, *kb = kt.p;
@@ -578,12 +579,23 @@ void radix_sort_u32(bgl_ctx *c, uint32_t *keys, uint32_t *vals, int64_t n, int b
     if (vals) radix_sort<uint32_t, true>(c, keys, vals, n, bits);
     else radix_sort<uint32_t, false>(c, keys, nullptr, n, bits);
 }
-void sort_check(bgl_ctx *c) {
-    BGL_CUDA(cudaMemcpyAsync(c->h_flag + 3, c->d_flag + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    BGL_CUDA(cudaStreamSynchronize(c->stream));
+void sort_fetch(bgl_ctx *c) {
+    if (c->sort_waits)
+        BGL_CUDA(cudaMemcpyAsync(c->h_flag + 3, c->d_flag + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+}
+void sort_fetched(bgl_ctx *c) {
+    if (!c->sort_waits) return;
+    c->sort_waits = false;
     if (!c->h_flag[3]) return;
+    c->h_flag[3] = 0;
     BGL_CUDA(cudaMemsetAsync(c->d_flag + 3, 0, sizeof(int), c->stream));
     fail(BGL_ETIMEOUT, "radix sort: a bounded device-side wait gave up");
+}
+void sort_check(bgl_ctx *c) {
+    if (!c->sort_waits) return;
+    sort_fetch(c);
+    BGL_CUDA(cudaStreamSynchronize(c->stream));
+    sort_fetched(c);
 }
 
 void SortWorkspace::reserve(Allocator *a, int64_t n, cudaStream_t s) {
