@@ -181,32 +181,17 @@ __global__ void __launch_bounds__(NA_TILE)
     cluster.sync();                                      // no block leaves while block 0 reads its memory
 }
 
-// swing / traction partial sums per tile into the static scratch; the last
-// block sums the tiles in order and sets s_G = min(tau trc / swg, 1.5 s_G)
-__global__ void na_swing_traction_kernel(const float2 *__restrict__ f, const float2 *__restrict__ fprev,
-                                         const float *__restrict__ mass, int64_t n, int variant, double tau,
-                                         double *sg, unsigned char *scratch) {
+// Swing and traction sums of the nodes of the block's tile (256 threads; the
+// result in thread 0): each thread's terms in order, lanes by an exchange
+// sum, warps in order.  F and P are the thread's forces and previous forces.
+constexpr int NA_PER = NA_RED_TILE / 256;
+__device__ __forceinline__ double2 na_tile_sums(const float2 (&F)[NA_PER], const float2 (&P)[NA_PER],
+                                                const float (&m)[NA_PER], int64_t q0, int64_t t1, int variant) {
     __shared__ double ws[32], wt[32];
-    __shared__ bool last;
-    unsigned *counter = reinterpret_cast<unsigned *>(scratch);
-    double2 *partial = reinterpret_cast<double2 *>(scratch + NA_COUNTER_BYTES);
-    const int64_t t0 = (int64_t)blockIdx.x * NA_RED_TILE;
-    const int64_t t1 = t0 + NA_RED_TILE < n ? t0 + NA_RED_TILE : n;
-    // the tile's loads in flight together, then each thread's terms in order
-    constexpr int PER = NA_RED_TILE / 256;
-    float2 F[PER], P[PER];
-    float m[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int64_t q = t0 + k * 256 + threadIdx.x;
-        F[k] = q < t1 ? f[q] : make_float2(0.f, 0.f);
-        P[k] = q < t1 ? fprev[q] : make_float2(0.f, 0.f);
-        m[k] = variant == 1 && q < t1 ? mass[q] : 0.f;
-    }
     double sw = 0.0, tr = 0.0;
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        if (t0 + k * 256 + (int64_t)threadIdx.x >= t1) break;
+    for (int k = 0; k < NA_PER; ++k) {
+        if (q0 + k * 256 >= t1) break;
         const float s = sqrtf((F[k].x - P[k].x) * (F[k].x - P[k].x) + (F[k].y - P[k].y) * (F[k].y - P[k].y));
         const float u = sqrtf((F[k].x + P[k].x) * (F[k].x + P[k].x) + (F[k].y + P[k].y) * (F[k].y + P[k].y));
         if (variant == 1) {
@@ -228,13 +213,108 @@ __global__ void na_swing_traction_kernel(const float2 *__restrict__ f, const flo
         wt[warp] = tr;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0, u = 0.0;
+    double s = 0.0, u = 0.0;
+    if (threadIdx.x == 0)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
             s += ws[w];
             u += wt[w];
         }
-        partial[blockIdx.x] = make_double2(s, u);
+    return make_double2(s, u);
+}
+
+// s_G = min(tau trc / swg, 1.5 s_G)
+__device__ __forceinline__ double na_speed(double swg, double trc, double g, double tau) {
+    double s_new = swg > 0.0 ? tau * trc / swg : 1.5 * g;
+    if (s_new > 1.5 * g) s_new = 1.5 * g;
+    return s_new;
+}
+
+// the node's move at global speed g
+__device__ __forceinline__ float2 na_move(float2 p, float2 F, float2 P, float g, float ks, float ksmax, int *bad) {
+    float sw = sqrtf((F.x - P.x) * (F.x - P.x) + (F.y - P.y) * (F.y - P.y));
+    float s = ks * g / (1.f + g * sqrtf(sw));
+    float fn = sqrtf(F.x * F.x + F.y * F.y);
+    if (fn > 0.f && s > ksmax / fn) s = ksmax / fn;
+    p.x += s * F.x;
+    p.y += s * F.y;
+    if (!isfinite(p.x) || !isfinite(p.y)) *bad = 1;
+    return p;
+}
+
+// Swing, traction, global speed and update of a component of up to NA_CLUSTER
+// tiles in one kernel: a cluster with a block per tile, the tiles' sums read
+// through distributed shared memory and added in tile order by every block.
+// Each node's forces are read once.  The sums and the update as two kernels
+// are all latency at this size (8.6 + 3.5 us and a launch between them at
+// 2,821 nodes): a whole iteration on 2,821 nodes 29.0 us with two kernels and
+// 27.9 with this one, on 8,192 48.5 and 46.6, on 16,384 (eight tiles, the most
+// a cluster holds) 124.6 and 122.8.
+__global__ void __launch_bounds__(256) na_swing_update_kernel(const float2 *__restrict__ f, float2 *__restrict__ fprev,
+                                                              const float *__restrict__ mass,
+                                                              float2 *__restrict__ xy, int64_t n, int variant,
+                                                              double tau, double *sg, float ks, float ksmax,
+                                                              int *bad) {
+    __shared__ double2 tile;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int64_t t0 = (int64_t)blockIdx.x * NA_RED_TILE;
+    const int64_t t1 = t0 + NA_RED_TILE < n ? t0 + NA_RED_TILE : n;
+    const int64_t q0 = t0 + threadIdx.x;
+    float2 F[NA_PER], P[NA_PER], p[NA_PER];
+    float m[NA_PER];
+#pragma unroll
+    for (int k = 0; k < NA_PER; ++k) {
+        const int64_t q = q0 + k * 256;
+        F[k] = q < t1 ? f[q] : make_float2(0.f, 0.f);
+        P[k] = q < t1 ? fprev[q] : make_float2(0.f, 0.f);
+        m[k] = variant == 1 && q < t1 ? mass[q] : 0.f;
+        p[k] = q < t1 ? xy[q] : make_float2(0.f, 0.f);
+    }
+    const double g0 = *sg;
+    const double2 own = na_tile_sums(F, P, m, q0, t1, variant);
+    if (threadIdx.x == 0) tile = own;
+    cluster.sync();                        // the tiles' sums; every thread has read *sg
+    double swg = 0.0, trc = 0.0;
+    for (unsigned k = 0; k < gridDim.x; ++k) {
+        const double2 v = *cluster.map_shared_rank(&tile, k);
+        swg += v.x;
+        trc += v.y;
+    }
+    const double s_new = na_speed(swg, trc, g0, tau);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *sg = s_new;
+    const float g = (float)s_new;
+#pragma unroll
+    for (int k = 0; k < NA_PER; ++k) {
+        const int64_t q = q0 + k * 256;
+        if (q >= t1) break;
+        xy[q] = na_move(p[k], F[k], P[k], g, ks, ksmax, bad);
+        fprev[q] = F[k];
+    }
+    cluster.sync();                        // no block leaves while another reads its sum
+}
+
+// Larger components: partial sums per tile into the static scratch; the last
+// block sums the tiles in order and sets s_G
+__global__ void na_swing_traction_kernel(const float2 *__restrict__ f, const float2 *__restrict__ fprev,
+                                         const float *__restrict__ mass, int64_t n, int variant, double tau,
+                                         double *sg, unsigned char *scratch) {
+    __shared__ bool last;
+    unsigned *counter = reinterpret_cast<unsigned *>(scratch);
+    double2 *partial = reinterpret_cast<double2 *>(scratch + NA_COUNTER_BYTES);
+    const int64_t t0 = (int64_t)blockIdx.x * NA_RED_TILE;
+    const int64_t t1 = t0 + NA_RED_TILE < n ? t0 + NA_RED_TILE : n;
+    // the tile's loads in flight together, then each thread's terms in order
+    float2 F[NA_PER], P[NA_PER];
+    float m[NA_PER];
+#pragma unroll
+    for (int k = 0; k < NA_PER; ++k) {
+        const int64_t q = t0 + k * 256 + threadIdx.x;
+        F[k] = q < t1 ? f[q] : make_float2(0.f, 0.f);
+        P[k] = q < t1 ? fprev[q] : make_float2(0.f, 0.f);
+        m[k] = variant == 1 && q < t1 ? mass[q] : 0.f;
+    }
+    const double2 own = na_tile_sums(F, P, m, t0 + threadIdx.x, t1, variant);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = own;
         __threadfence();
         last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
@@ -251,10 +331,7 @@ __global__ void na_swing_traction_kernel(const float2 *__restrict__ f, const flo
         swg += tiles[k].x;
         trc += tiles[k].y;
     }
-    double g = *sg;
-    double s_new = swg > 0.0 ? tau * trc / swg : 1.5 * g;
-    if (s_new > 1.5 * g) s_new = 1.5 * g;
-    *sg = s_new;
+    *sg = na_speed(swg, trc, *sg, tau);
     *counter = 0u;
 }
 
@@ -265,17 +342,8 @@ __global__ void na_update_kernel(const float2 *__restrict__ f, float2 *__restric
     if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<unsigned *>(scratch) = 0u;
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
-    float2 F = f[q], P = fprev[q];
-    float g = (float)*sg;
-    float sw = sqrtf((F.x - P.x) * (F.x - P.x) + (F.y - P.y) * (F.y - P.y));
-    float s = ks * g / (1.f + g * sqrtf(sw));
-    float fn = sqrtf(F.x * F.x + F.y * F.y);
-    if (fn > 0.f && s > ksmax / fn) s = ksmax / fn;
-    float2 p = xy[q];
-    p.x += s * F.x;
-    p.y += s * F.y;
-    if (!isfinite(p.x) || !isfinite(p.y)) *bad = 1;
-    xy[q] = p;
+    const float2 F = f[q];
+    xy[q] = na_move(xy[q], F, fprev[q], (float)*sg, ks, ksmax, bad);
     fprev[q] = F;
 }
 
@@ -316,7 +384,18 @@ void fa2_iteration_noalloc(bgl_ctx *c, int64_t n, const int64_t *d_off, const in
     BGL_CUDA(cudaLaunchKernelEx(&cfg, na_force_kernel, (const float2 *)d_xy, d_mass, d_off, d_adj, n, (float)p->kr,
                                 (float)p->kg, d_f));
     BGL_LAUNCH_CHECK();
-    na_swing_traction_kernel<<<na_blocks(n, NA_RED_TILE), 256, 0, s>>>(d_f, d_fprev, d_mass, n, p->swing_variant,
+    const unsigned tiles = na_blocks(n, NA_RED_TILE);
+    if (tiles <= NA_CLUSTER) {
+        attr.val.clusterDim.x = tiles;
+        cfg.gridDim = dim3(tiles);
+        cfg.blockDim = dim3(256);
+        BGL_CUDA(cudaLaunchKernelEx(&cfg, na_swing_update_kernel, (const float2 *)d_f, d_fprev, d_mass, d_xy, n,
+                                    (int)p->swing_variant, p->tau, d_sg, (float)p->ks, (float)p->ksmax,
+                                    c->d_flag + 2));
+        BGL_LAUNCH_CHECK();
+        return;
+    }
+    na_swing_traction_kernel<<<tiles, 256, 0, s>>>(d_f, d_fprev, d_mass, n, p->swing_variant,
                                                                        p->tau, d_sg, scratch);
     BGL_LAUNCH_CHECK();
     na_update_kernel<<<na_blocks(n, 256), 256, 0, s>>>(d_f, d_fprev, d_xy, d_sg, n, (float)p->ks, (float)p->ksmax,

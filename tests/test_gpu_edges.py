@@ -1,7 +1,7 @@
 """Edges of the kernels' tiles, splits and dispatch rules: the exact sum (target
 tiles of 128 and 256, source stages of 1,024, one block for all stages above
 65,536 nodes, attraction by lane, warp and block), the allocation-free
-iteration (cluster sizes 2 to 8), the FMM's small-tree paths (cluster sort up
+iteration (cluster sizes 1 to 8), the FMM's small-tree paths (cluster sort up
 to 32,768 points, rows of leaves, trees of up to 128 tiles), the radix sorts of
 the graph build (tiles of 4,096 keys) and the k-hop kernels (hubs, many hops,
 caps).  Against the oracle at the tolerances of the other tests: exact forces
@@ -159,4 +159,37 @@ def test_khop_hubs_many_hops_and_caps(ctx, seed, hops):
     assert np.array_equal(g.khop(seed, hops, len(ids))[0], ids)
     if len(ids) > 1:
         assert g.khop(seed, hops, len(ids) - 1) is None
+    g.destroy()
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n", [255, 2048, 2049, 16384, 16385])
+def test_noalloc_speed_and_update_at_tile_and_cluster_edges(ctx, n, variant):
+    """Up to eight tiles of 2,048 nodes the sums and the update are one cluster
+    kernel, above it two kernels: s_G of the second call against the FP64 sums
+    of the GPU's own forces (1e-5), positions against bgl_fa2_step (1e-3 of the
+    diagonal)."""
+    import torch
+    bgl = _bgl()
+    g, off, adj, mass = _component(ctx, n, *_hub_graph(n, 20))
+    xy = synth.points(n, n, "uniform", scale=30.0)
+    dev = [torch.from_numpy(a).cuda() for a in (off, adj, mass.astype(np.float32), xy)]
+    f, fp = torch.zeros(n, 2, device="cuda"), torch.zeros(n, 2, device="cuda")
+    sg = torch.ones(1, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    p = bgl.params(repulsion=bgl.REP_EXACT, swing_variant=variant)
+    forces = []
+    for _ in range(2):
+        ctx.fa2_iteration_noalloc(n, dev[0], dev[1], dev[2], dev[3], fp, f, sg, p)
+        ctx.sync()
+        forces.append(f.cpu().numpy().astype(np.float64))
+        assert np.array_equal(fp.cpu().numpy(), f.cpu().numpy())
+    f1, f2 = forces
+    w = mass if variant else np.ones(n)
+    swg, trc = np.sum(w * np.hypot(*(f2 - f1).T)), np.sum((0.5 if variant else 1.0) * w * np.hypot(*(f2 + f1).T))
+    first = 0.5 if variant else 1.0                 # of the first call, where swing equals traction
+    assert float(sg.cpu()[0]) == pytest.approx(min(trc / swg, 1.5 * first), rel=1e-5)
+    want, _ = g.fa2_step(0, p, 2, xy)
+    err = np.max(np.hypot(*(dev[3].cpu().numpy() - want).T))
+    assert err <= 1e-3 * np.hypot(*np.ptp(want, axis=0))
     g.destroy()
