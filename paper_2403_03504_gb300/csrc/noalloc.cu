@@ -6,8 +6,8 @@
 // a latency-bound loop cannot afford the device-wide synchronisation that
 // cudaMalloc and cudaFree may cause.  bgl_fa2_iteration_noalloc serves them:
 // the caller passes every input and output, and the only scratch the
-// iteration needs -- the per-tile swing/traction partial sums and the
-// arrival counter of their reduction -- lives in one file-scope device
+// iteration needs -- above eight tiles the per-tile swing/traction partial
+// sums and the arrival counter of their reduction -- lives in one file-scope device
 // array of fixed size (NOALLOC_SCRATCH_BYTES), which every GPU that loads
 // this library holds until the process exits.
 //
