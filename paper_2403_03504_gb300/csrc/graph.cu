@@ -497,6 +497,9 @@ void components_device(bgl_graph *g) {
     Allocator *A = c->alloc;
     cudaStream_t s = c->stream;
     const int64_t n = g->n;
+    // the arrays are rebuilt in place: until they are whole the graph has no
+    // components, so that after a failure nothing uses them
+    g->has_comp = false;
     g->label.reset(A, n);
     iota_kernel<<<blocks_for(n), TPB, 0, s>>>(g->label.p, n);
     BGL_LAUNCH_CHECK();
