@@ -480,7 +480,9 @@ int64_t bgl_launch_count(void);
  * `after` more successful device allocations on this context, the next one
  * fails as if the device were out of memory, so the call making it returns
  * BGL_ENOMEM with its outputs untouched; the aid then turns itself off.
- * after = -1 turns it off at once.  No GPU fault is involved. */
+ * after = -1 turns it off at once.  The workers of a server start with the
+ * setting that its resident graph's context has in bgl_server_create.  No GPU
+ * fault is involved. */
 bgl_status bgl_debug_fail_alloc(bgl_ctx *ctx, int64_t after);
 
 #ifdef __cplusplus

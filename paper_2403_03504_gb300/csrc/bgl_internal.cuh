@@ -123,8 +123,8 @@ struct DevBuf {
     void reset(Allocator *al, size_t count) {
         release();
         a = al;
-        n = count;
         p = static_cast<T *>(al->alloc(sizeof(T) * (count > 0 ? count : 1)));
+        n = count;      // (still 0 after a refused allocation)
     }
     // grow-only: keeps the block when it is already big enough
     void ensure(Allocator *al, size_t count) {

@@ -348,18 +348,23 @@ struct KhopScratch {
     DevBuf<longlong2> tiles, chunks;
     DevBuf<KhState> state;
     int32_t epoch = 0;
-    int64_t cap = 0;
+    // nodes and visit list entries that the arrays are whole for: a serving
+    // worker goes on after a refused allocation, and what was being made then
+    // is made again
+    int64_t nodes = 0, cap = 0;
     void reserve(bgl_ctx *c, const bgl_graph *R, int64_t cap_) {
-        const int64_t n_res = R->n;
-        if (stamp.n < (size_t)n_res) {
-            stamp.reset(c->alloc, n_res);
-            local.reset(c->alloc, n_res);
-            tiles.reset(c->alloc, (n_res + KH_TILE - 1) / KH_TILE);
+        if (nodes < R->n) {
+            nodes = 0;
+            stamp.reset(c->alloc, R->n);
+            local.reset(c->alloc, R->n);
+            tiles.reset(c->alloc, (R->n + KH_TILE - 1) / KH_TILE);
             hubs.reset(c->alloc, 2 * R->n_undir / KH_HUB_DEG + 1);
-            BGL_CUDA(cudaMemsetAsync(stamp.p, 0, sizeof(int32_t) * n_res, c->stream));
+            BGL_CUDA(cudaMemsetAsync(stamp.p, 0, sizeof(int32_t) * R->n, c->stream));
             epoch = 0;
+            nodes = R->n;
         }
         if (cap < cap_) {
+            cap = 0;
             found.reset(c->alloc, cap_ + 1);
             vis.reset(c->alloc, cap_ + 1);
             dscan.reset(c->alloc, cap_ + 1);
@@ -718,6 +723,7 @@ bgl_status bgl_server_create(bgl_graph *resident, int32_t slots, int64_t hbm_bud
             bgl_server_destroy(srv);
             return st;
         }
+        c->alloc->fail_after.store(resident->ctx->alloc->fail_after.load());     // test aid
         srv->s.ctxs.push_back(c);
     }
     // the resident graph must be complete before other streams read it

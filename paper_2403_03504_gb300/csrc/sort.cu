@@ -600,6 +600,7 @@ void sort_check(bgl_ctx *c) {
 
 void SortWorkspace::reserve(Allocator *a, int64_t n, cudaStream_t s) {
     if (n <= cap) return;
+    cap = 0;
     keys.reset(a, n);
     vals.reset(a, n);
     keys2.reset(a, n);

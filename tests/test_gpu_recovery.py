@@ -4,7 +4,10 @@ only a later call would meet.
 * bgl_components on a graph that has components rebuilds their arrays in
   place: a call that fails partway (a refused allocation) leaves the graph
   without components, so that the calls that need them return BGL_ESTATE
-  until bgl_components has succeeded again."""
+  until bgl_components has succeeded again.
+* A serving worker keeps its k-hop scratch between requests: after a request
+  that a refused allocation ended, while the scratch was made or grown, the
+  next requests get the same neighbourhoods and layouts as ever."""
 import numpy as np
 import pytest
 
@@ -60,4 +63,44 @@ def test_failed_components_leave_the_graph_without_any(ctx):
             break
     ctx.debug_fail_alloc(-1)
     assert refused >= 15                 # every allocation of the call was refused once
+    g.destroy()
+
+
+def test_serving_worker_goes_on_after_a_refused_allocation(ctx):
+    bgl = _bgl()
+    n = 3000
+    u, v = np.arange(n - 1), np.arange(1, n)
+    hub = np.arange(2, 1300)                                # node 0: more than 1,024 entries
+    g = bgl.Graph.from_edges(ctx, n, np.concatenate([u, np.zeros_like(hub)]), np.concatenate([v, hub]))
+    p = bgl.params(seed=4, fa2_iters=1, kk_sweeps=1)
+    # (the visit list of the third and fourth is larger than those before)
+    requests = [(2500, 3, 10), (2000, 5, 20), (1290, 2, n), (0, 1, n), (2500, 3, 10)]
+
+    def serve(after):
+        ctx.debug_fail_alloc(after)
+        srv = bgl.Server(g, slots=1)
+        ctx.debug_fail_alloc(-1)
+        out = []
+        for seed, hops, cap in requests:
+            rid = srv.submit(seed, hops, p, cap)
+            status, k, _, _ = srv.wait(rid)
+            out.append(srv.fetch(rid, k) if status == 0 else status)
+        srv.close()
+        return out
+
+    want = serve(-1)
+    for (seed, hops, cap), w in zip(requests, want):
+        assert np.array_equal(w[0], g.khop(seed, hops, cap)[0])
+    after, refused = 0, len(requests)
+    while refused:
+        refused = 0
+        for w, got in zip(want, serve(after)):
+            if isinstance(got, int):
+                assert got == ENOMEM
+                refused += 1
+            else:
+                assert np.array_equal(got[0], w[0]) and np.array_equal(got[1], w[1]), after
+        assert refused <= 1
+        after += 1
+    assert 100 < after < 2000            # every allocation of the five requests was refused once
     g.destroy()
