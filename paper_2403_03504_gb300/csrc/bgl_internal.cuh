@@ -317,6 +317,10 @@ struct OsWait {
     long long spin = 0;
     int stall_first = 0;
 };
+// The waits of a sort that starts now: with BGL_TEST_SORT_STALL=1 in the
+// environment (a test aid) its first tile withholds its counts and the waits
+// on it give up after 4,096 polls, so that the call returns BGL_ETIMEOUT.
+OsWait sort_wait(int *err);
 // d_skip (device int, may be null = 0): the passes below *d_skip (0 or 2)
 // return at once, so the keys end up ordered by their top 32 - 8 * skip
 // bits only (stable: equal top bits keep the input order).  Read by each

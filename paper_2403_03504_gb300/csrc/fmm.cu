@@ -2628,17 +2628,7 @@ FmmPlan *fmm_create(bgl_graph *g, const bgl_params *p, int64_t c) {
         BGL_CUDA(cudaMemsetAsync(pl->epoch.p, 0, sizeof(unsigned), s));
         pl->tickets.reset(A, NTICKETS);
         pl->err.reset(A, 1);
-        pl->wait.err = pl->err.p;
-        {
-            // test aid for the failure path: BGL_TEST_SORT_STALL=1 makes the
-            // sort's first tile withhold its counts and the waits on it give
-            // up after 4,096 polls, so the evaluation reports BGL_ETIMEOUT
-            const char *v = std::getenv("BGL_TEST_SORT_STALL");
-            if (v && v[0] == '1') {
-                pl->wait.stall_first = 1;
-                pl->wait.spin = 1 << 12;
-            }
-        }
+        pl->wait = sort_wait(pl->err.p);
         pl->sortws.reserve(A, n, s);
         BGL_CUDA(cudaMemsetAsync(pl->counter.p, 0, sizeof(unsigned), s));
         BGL_CUDA(cudaMemsetAsync(pl->arrive.p, 0, sizeof(int) * bmax, s));

@@ -5,6 +5,7 @@
 // (onesweep, below), in which each warp ranks its keys by votes on their
 // digits so that equal digits keep their input order (stable).
 #include <algorithm>
+#include <cstdlib>
 
 #include "bgl_internal.cuh"
 #include "sort_hist.cuh"
@@ -536,15 +537,14 @@ void radix_sort_words(bgl_ctx *c, K *keys, uint32_t *vals, int64_t n, int bits) 
     sweep_hist_kernel<K><<<(unsigned)nt, OS_THREADS, 0, c->stream>>>(keys, n, passes, ws.p, base.p, tickets + 15);
     BGL_LAUNCH_CHECK();
     if (nt > 1) c->sort_waits = true;      // (one tile waits for nobody)
-    OsWait wait;
-    wait.spin = OS_SPIN;
+    const OsWait wait = sort_wait(c->d_flag + 3);
     K *ka = keys, *kb = kt.p;
     uint32_t *va = vals, *vb = vt.p;
     for (int d = 0; d < passes; ++d) {
         if (each) BGL_CUDA(cudaMemsetAsync(status.p, 0, status.bytes(), c->stream));
         sweep_kernel<K, VALS, W><<<(unsigned)nt, OS_THREADS, 0, c->stream>>>(
             ka, va, kb, vb, n, 8 * d, base.p + 256 * d, status.p + (each ? 0 : (size_t)d * 256 * nt), tickets + d,
-            c->d_flag + 3, wait);
+            wait.err, wait);
         BGL_LAUNCH_CHECK();
         std::swap(ka, kb);
         std::swap(va, vb);
@@ -578,6 +578,17 @@ void radix_sort_u64(bgl_ctx *c, uint64_t *keys, uint32_t *vals, int64_t n, int b
 void radix_sort_u32(bgl_ctx *c, uint32_t *keys, uint32_t *vals, int64_t n, int bits) {
     if (vals) radix_sort<uint32_t, true>(c, keys, vals, n, bits);
     else radix_sort<uint32_t, false>(c, keys, nullptr, n, bits);
+}
+OsWait sort_wait(int *err) {
+    OsWait w;
+    w.err = err;
+    w.spin = OS_SPIN;
+    const char *v = std::getenv("BGL_TEST_SORT_STALL");
+    if (v && v[0] == '1') {
+        w.stall_first = 1;
+        w.spin = 1 << 12;
+    }
+    return w;
 }
 void sort_fetch(bgl_ctx *c) {
     if (c->sort_waits)

@@ -7,7 +7,13 @@ only a later call would meet.
   until bgl_components has succeeded again.
 * A serving worker keeps its k-hop scratch between requests: after a request
   that a refused allocation ended, while the scratch was made or grown, the
-  next requests get the same neighbourhoods and layouts as ever."""
+  next requests get the same neighbourhoods and layouts as ever.
+* The radix sorts of the graph build, the components and the assembly wait
+  for each other's tiles, with a bound.  With BGL_TEST_SORT_STALL=1 the first
+  tile withholds its counts and the waits on it give up after 4,096 polls: the
+  call returns BGL_ETIMEOUT before a sorted value indexes anything (in each of
+  the sorts, inputs of two tiles and more), and the same call without the aid
+  gives what it gave before."""
 import numpy as np
 import pytest
 
@@ -104,3 +110,71 @@ def test_serving_worker_goes_on_after_a_refused_allocation(ctx):
         after += 1
     assert 100 < after < 2000            # every allocation of the five requests was refused once
     g.destroy()
+
+
+def _build(ctx):
+    tx = synth.tx_lists(**dict(synth.C1, n_tx=3000))
+    g = _bgl().Graph.build(ctx, tx.in_off, tx.in_addr, tx.out_off, tx.out_addr)
+    out = [g.addresses(), *g.edges(), *g.csr()]
+    g.destroy()
+    return out
+
+
+def _from_edges(ctx, n, u, v):
+    g = _bgl().Graph.from_edges(ctx, n, u, v)
+    out = [*g.edges(), *g.csr()]
+    g.destroy()
+    return out
+
+
+def _pairs(comps, size):
+    """Paths of `size` nodes."""
+    u = np.setdiff1d(np.arange(comps * size), np.arange(1, comps + 1) * size - 1)
+    return comps * size, u, u + 1
+
+
+def _components(ctx, g):
+    labels, n_comp = g.components()
+    return [labels, np.array(n_comp), *g.component_nodes()]
+
+
+def _assembled(ctx, g, out):
+    return [g.layout(_bgl().params(seed=1, kk_sweeps=2, assemble=1), out=out)]
+
+
+@pytest.mark.parametrize("sort", ["addresses", "directed edges", "undirected edges", "component sizes", "nodes",
+                                  "assembly order"])
+def test_a_sort_that_gives_up_is_reported_before_its_output_is_used(ctx, monkeypatch, sort):
+    bgl = _bgl()
+    g, out = None, np.zeros((0, 2), np.float32)
+    if sort == "addresses":
+        call = lambda: _build(ctx)
+    elif sort == "directed edges":
+        rng = np.random.default_rng(1)
+        u, v = rng.integers(0, 9000, (2, 20000))
+        call = lambda: _from_edges(ctx, 9000, u, v)
+    elif sort == "undirected edges":                # one tile of edges, two of both directions
+        n, u, v = _pairs(1, 3001)
+        call = lambda: _from_edges(ctx, n, u, v)
+    else:
+        n, u, v = _pairs(*((2, 4000) if sort == "nodes" else (5000, 2)))
+        g = bgl.Graph.from_edges(ctx, n, u, v)
+        if sort == "assembly order":
+            g.components(labels=False)
+            out = np.zeros((n, 2), np.float32)
+            call = lambda: _assembled(ctx, g, out)
+        else:
+            call = lambda: _components(ctx, g)
+    want = [a.copy() for a in call()]
+    out[:] = 7.5
+    monkeypatch.setenv("BGL_TEST_SORT_STALL", "1")
+    for _ in range(2):
+        _refused(ctx, call, ETIMEOUT)
+    assert np.all(out == 7.5)
+    if g is not None and sort != "assembly order":
+        _refused(ctx, lambda: g.layout(bgl.params()), ESTATE)
+    monkeypatch.delenv("BGL_TEST_SORT_STALL")
+    got = call()
+    assert len(got) == len(want) and all(np.array_equal(a, b) for a, b in zip(got, want))
+    if g is not None:
+        g.destroy()
