@@ -284,15 +284,13 @@ struct SortWorkspace {
     int64_t cap = 0;
     void reserve(Allocator *a, int64_t n, cudaStream_t s);
 };
-// With gpts, the last pass writes gpts[i] = {gxy[v].x, gxy[v].y, gmass[v], v}
-// (v = the value of sorted key i, as int bits) instead of the sorted values.
-void radix_sort_u32_ws(bgl_ctx *c, SortWorkspace &ws, uint32_t *keys, uint32_t *vals, int64_t n, int bits,
-                       const float2 *gxy = nullptr, const float *gmass = nullptr, float4 *gpts = nullptr);
-// The same sort in two halves, so that a caller's kernel can count the digit
-// histograms while it makes the keys: radix_sort_u32_ws_begin clears the
-// counts and returns them; every block of the caller's kernel (OS_THREADS)
-// then calls os_block_hist (sort_hist.cuh) on its keys; and
-// radix_sort_u32_ws_scatter runs the four passes.
+// A sort on a workspace comes in two halves around a kernel of the caller's
+// that makes the keys: radix_sort_u32_ws_begin returns the counts; every block
+// of the caller's kernel (OS_THREADS, one per tile) then calls os_block_hist
+// (sort_hist.cuh) on its keys and zeroes its tile's status words
+// (os_clear_status); and radix_sort_u32_ws_scatter runs the four passes.  The
+// caller zeroes hist and tickets in a kernel that runs before its histogram
+// kernel.
 struct OsHist {
     uint32_t *hist;      // 4 x 256 digit counts
     uint32_t *base;      // 4 x 256 exclusive digit bases (written by the last block)
@@ -301,17 +299,13 @@ struct OsHist {
     uint32_t *status;    // 4 x ntiles x 256 look-back status words
     int64_t ntiles;      // tiles of 4,096 keys
 };
-// With clear = false the caller zeroes hist and tickets in a kernel that
-// runs before its histogram kernel, and each block of the histogram kernel
-// (one per tile) zeroes its tile's status words (os_clear_status).
-OsHist radix_sort_u32_ws_begin(bgl_ctx *c, SortWorkspace &ws, int64_t n, bool clear = true);
-// The bounded waits of the scatter passes: err (null: the workspace's own
-// word) receives bit 1 when a wait gives up, and a pass started after that
-// does nothing; spin is the poll limit (0: the default, about half a second
-// of polling); stall_first = 1 makes the first tile of every pass withhold
-// its counts, so that the waits on it run out -- a test aid for the
-// failure path (BGL_ETIMEOUT), memory-safe because a tile that gives up
-// still writes inside [0, n).
+OsHist radix_sort_u32_ws_begin(SortWorkspace &ws, int64_t n);
+// The bounded waits of the scatter passes: err receives bit 1 when a wait
+// gives up, and a pass started after that does nothing; spin is the poll
+// limit (by default about half a second of polling); stall_first = 1 makes
+// the first tile of every pass withhold its counts, so that the waits on it
+// run out -- a test aid for the failure path (BGL_ETIMEOUT), memory-safe
+// because a tile that gives up still writes inside [0, n).
 struct OsWait {
     int *err = nullptr;
     long long spin = 0;
@@ -321,13 +315,15 @@ struct OsWait {
 // environment (a test aid) its first tile withholds its counts and the waits
 // on it give up after 4,096 polls, so that the call returns BGL_ETIMEOUT.
 OsWait sort_wait(int *err);
+// With gpts, the last pass writes gpts[i] = {gxy[v].x, gxy[v].y, gmass[v], v}
+// (v = the value of sorted key i, as int bits) instead of the sorted values.
 // d_skip (device int, may be null = 0): the passes below *d_skip (0 or 2)
 // return at once, so the keys end up ordered by their top 32 - 8 * skip
 // bits only (stable: equal top bits keep the input order).  Read by each
 // pass when it starts.
 void radix_sort_u32_ws_scatter(bgl_ctx *c, SortWorkspace &ws, uint32_t *keys, uint32_t *vals, int64_t n,
-                               const float2 *gxy = nullptr, const float *gmass = nullptr, float4 *gpts = nullptr,
-                               const int *d_skip = nullptr, OsWait wait = OsWait());
+                               const float2 *gxy, const float *gmass, float4 *gpts, const int *d_skip,
+                               const OsWait &wait);
 
 int bits_for(uint64_t max_value);   // number of bits needed to hold max_value
 

@@ -2740,7 +2740,7 @@ static void phase_points(FmmPlan *pl, const float2 *xl, cudaStream_t s) {
         // tickets, digit counts and look-back words are zeroed by bbox_kernel
         // (by update_root_kernel in a fused iteration, which also made the root)
         // and keys_kernel
-        const OsHist h = radix_sort_u32_ws_begin(ctx, pl->sortws, n, false);
+        const OsHist h = radix_sort_u32_ws_begin(pl->sortws, n);
         if (!pl->fused) {
             bbox_kernel<<<bbox_blocks(pl), 256, 0, s>>>(xl, n, pl->part.p, pl->counter.p, pl->root.p, pl->err.p,
                                                        pl->epoch.p, pl->tickets.p, h);
@@ -3066,7 +3066,7 @@ void fmm_fuse(FmmPlan *pl, const FmmFuse &fz) {
 
 void fmm_root(FmmPlan *pl, const float2 *xy, int64_t qbase) {
     bgl_ctx *ctx = pl->g->ctx;
-    const OsHist h = radix_sort_u32_ws_begin(ctx, pl->sortws, pl->n, false);
+    const OsHist h = radix_sort_u32_ws_begin(pl->sortws, pl->n);
     bbox_kernel<<<bbox_blocks(pl), 256, 0, ctx->stream>>>(xy + (pl->q0 - qbase), pl->n, pl->part.p, pl->counter.p,
                                                           pl->root.p, pl->err.p, pl->epoch.p, pl->tickets.p, h);
     BGL_LAUNCH_CHECK();
@@ -3075,7 +3075,7 @@ void fmm_root(FmmPlan *pl, const float2 *xy, int64_t qbase) {
 void fmm_update_root(FmmPlan *pl, float2 *xy, int64_t qbase, const float2 *f, float2 *fprev, int64_t fbase,
                      const LoopCtl &loop) {
     bgl_ctx *ctx = pl->g->ctx;
-    const OsHist h = radix_sort_u32_ws_begin(ctx, pl->sortws, pl->n, false);
+    const OsHist h = radix_sort_u32_ws_begin(pl->sortws, pl->n);
     (loop.count ? update_root_kernel<true> : update_root_kernel<false>)<<<nblk(pl->n, 256 * UPDATE_POINTS), 256, 0, ctx->stream>>>(
         xy + (pl->q0 - qbase), f + (pl->q0 - fbase), fprev + (pl->q0 - fbase), pl->n, pl->fz.sg, pl->fz.ks,
         pl->fz.ksmax, pl->fz.bad, pl->part.p, pl->counter.p, pl->root.p, pl->err.p, pl->epoch.p, pl->tickets.p, h,

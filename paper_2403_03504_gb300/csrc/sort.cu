@@ -207,20 +207,6 @@ __device__ __forceinline__ uint32_t os_look_back(volatile W *st, int tile, int d
     return excl;
 }
 
-// digit histograms of the keys, OS_ITEMS per thread
-__global__ void __launch_bounds__(OS_THREADS) os_hist_kernel(const uint32_t *__restrict__ keys, int64_t n, OsHist h) {
-    uint32_t k[OS_ITEMS];
-    unsigned valid = 0;
-    const int64_t i0 = (int64_t)blockIdx.x * OS_TILE + threadIdx.x;
-#pragma unroll
-    for (int r = 0; r < OS_ITEMS; ++r) {
-        const int64_t i = i0 + (int64_t)r * OS_THREADS;
-        k[r] = i < n ? keys[i] : 0u;
-        if (i < n) valid |= 1u << r;
-    }
-    os_block_hist<OS_ITEMS>(k, valid, h);
-}
-
 // Buffers of pass d (0..3) when the first `skip` passes are skipped: the
 // first active pass reads the input, the last writes the output, the ones
 // between alternate between the two scratch pairs.
@@ -229,12 +215,12 @@ struct OsBufs {
     uint32_t *k0, *v0, *k1, *v1; // scratch
 };
 
-__global__ void __launch_bounds__(OS_THREADS, OS_THREADS > 512 ? 1 : 2) os_scatter_kernel(OsBufs bf, int d, const int *d_skip, int64_t n,
-                                                                 const uint32_t *__restrict__ base,
-                                                                 uint32_t *status, unsigned *ticket, int *err,
-                                                                 const float2 *__restrict__ gxy,
-                                                                 const float *__restrict__ gmass,
-                                                                 float4 *__restrict__ gpts, OsWait wait) {
+__global__ void __launch_bounds__(OS_THREADS, 2) os_scatter_kernel(OsBufs bf, int d, const int *d_skip, int64_t n,
+                                                                   const uint32_t *__restrict__ base,
+                                                                   uint32_t *status, unsigned *ticket, int *err,
+                                                                   const float2 *__restrict__ gxy,
+                                                                   const float *__restrict__ gmass,
+                                                                   float4 *__restrict__ gpts, OsWait wait) {
     const int skip = d_skip ? *d_skip : 0;
     if (d < skip) return;
     const int shift = 8 * d;
@@ -616,17 +602,15 @@ void SortWorkspace::reserve(Allocator *a, int64_t n, cudaStream_t s) {
     vals.reset(a, n);
     keys2.reset(a, n);
     vals2.reset(a, n);
-    // hist: 4 x 256 digit counts, 4 x 256 digit bases, 4 tickets, 1 counter, error word
-    hist.reset(a, 8 * 256 + 8);
+    // hist: 4 x 256 digit counts, 4 x 256 digit bases, 4 tickets, 1 counter
+    hist.reset(a, 8 * 256 + 5);
     BGL_CUDA(cudaMemsetAsync(hist.p, 0, hist.bytes(), s));
     tiles.reset(a, 4 * 256 * os_tiles(n));   // look-back status words, one block per pass
     cap = n;
 }
 
-OsHist radix_sort_u32_ws_begin(bgl_ctx *c, SortWorkspace &ws, int64_t n, bool clear) {
+OsHist radix_sort_u32_ws_begin(SortWorkspace &ws, int64_t n) {
     BGL_REQUIRE(n <= ws.cap && n < (int64_t(1) << 30), "radix sort: workspace too small");
-    cudaStream_t s = c->stream;
-    const int64_t nt = os_tiles(n);
     OsHist h;
     h.hist = reinterpret_cast<uint32_t *>(ws.hist.p);
     h.base = h.hist + 4 * 256;
@@ -634,45 +618,30 @@ OsHist radix_sort_u32_ws_begin(bgl_ctx *c, SortWorkspace &ws, int64_t n, bool cl
     h.counter = tickets + 4;
     h.tickets = tickets;
     h.status = reinterpret_cast<uint32_t *>(ws.tiles.p);
-    h.ntiles = nt;
-    if (!clear) return h;
-    // counts, pass tickets and look-back status words start at zero
-    BGL_CUDA(cudaMemsetAsync(h.hist, 0, sizeof(uint32_t) * 4 * 256, s));
-    BGL_CUDA(cudaMemsetAsync(tickets, 0, sizeof(unsigned) * 4, s));
-    BGL_CUDA(cudaMemsetAsync(ws.tiles.p, 0, sizeof(uint32_t) * 4 * 256 * nt, s));
+    h.ntiles = os_tiles(n);
     return h;
 }
 
 void radix_sort_u32_ws_scatter(bgl_ctx *c, SortWorkspace &ws, uint32_t *keys, uint32_t *vals, int64_t n,
-                               const float2 *gxy, const float *gmass, float4 *gpts, const int *d_skip, OsWait wait) {
+                               const float2 *gxy, const float *gmass, float4 *gpts, const int *d_skip,
+                               const OsWait &wait) {
+    BGL_REQUIRE(wait.err && wait.spin > 0, "radix sort: waits without a bound or a word for their failure");
     cudaStream_t s = c->stream;
     const int64_t nt = os_tiles(n);
     uint32_t *hist = reinterpret_cast<uint32_t *>(ws.hist.p);
     uint32_t *base = hist + 4 * 256;
     unsigned *tickets = reinterpret_cast<unsigned *>(hist + 8 * 256);
-    int *err = wait.err ? wait.err : reinterpret_cast<int *>(tickets + 5);
-    if (wait.spin <= 0) wait.spin = OS_SPIN;
     uint32_t *status = reinterpret_cast<uint32_t *>(ws.tiles.p);
     const OsBufs bf{keys, vals, ws.keys.p, ws.vals.p, ws.keys2.p, ws.vals2.p};
     for (int d = 0; d < 4; ++d) {
         const bool g = d == 3 && gpts;
         os_scatter_kernel<<<(unsigned)nt, OS_THREADS, 0, s>>>(bf, d, d_skip, n, base + 256 * d,
-                                                              status + (int64_t)d * 256 * nt, tickets + d, err,
+                                                              status + (int64_t)d * 256 * nt, tickets + d, wait.err,
                                                               g ? gxy : nullptr, g ? gmass : nullptr,
                                                               g ? gpts : nullptr, wait);
         BGL_LAUNCH_CHECK();
     }
     // the sorted keys (and values unless gathered) are back in keys / vals
-}
-
-void radix_sort_u32_ws(bgl_ctx *c, SortWorkspace &ws, uint32_t *keys, uint32_t *vals, int64_t n, int bits,
-                       const float2 *gxy, const float *gmass, float4 *gpts) {
-    if (n <= 1 || bits <= 0) return;
-    BGL_REQUIRE(bits == 32 && vals, "radix sort: the workspace sort takes 32-bit keys with values");
-    const OsHist h = radix_sort_u32_ws_begin(c, ws, n);
-    os_hist_kernel<<<(unsigned)os_tiles(n), OS_THREADS, 0, c->stream>>>(keys, n, h);
-    BGL_LAUNCH_CHECK();
-    radix_sort_u32_ws_scatter(c, ws, keys, vals, n, gxy, gmass, gpts);
 }
 
 int bits_for(uint64_t v) {
