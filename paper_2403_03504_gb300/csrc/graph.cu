@@ -521,6 +521,7 @@ void components_device(bgl_graph *g) {
     DevBuf<int32_t> size(A, n), flag(A, n), fscan(A, n), tot(A, 1);
     BGL_CUDA(cudaMemsetAsync(size.p, 0, sizeof(int32_t) * (n > 0 ? n : 1), s));
     comp_size_kernel<<<blocks_for(n, TPB * SIZE_ITEMS), TPB, 0, s>>>(g->label.p, n, size.p);
+    BGL_LAUNCH_CHECK();
     root_flag_kernel<<<blocks_for(n), TPB, 0, s>>>(g->label.p, n, flag.p);
     BGL_LAUNCH_CHECK();
     scan_exclusive_i32(c, flag.p, fscan.p, n, tot.p);
