@@ -14,7 +14,8 @@
 // The kernels are variants of the ones in fa2.cu that need no host-built
 // tile list and no per-call buffers: one component, targets tiled by block
 // index, the stages of a tile's sources spread over a thread-block cluster
-// whose blocks hand their sums over in distributed shared memory.  The
+// whose blocks hand their sums over in distributed shared memory, or, on large
+// components, all in one block.  The
 // formulas of every force term, of the swing/traction sums and of the update
 // are the same; the order and precision of the sums differ (here every thread
 // sums its swing/traction terms in FP64 over tiles of 2,048 nodes and a hub's
@@ -51,6 +52,33 @@ constexpr size_t NOALLOC_SCRATCH_BYTES = NA_COUNTER_BYTES + sizeof(double2) * NA
 // cudaGetSymbolAddress (noalloc_scratch_address, stored in the context).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
 
+// NA_STILE sources from s0 on (cnt of them) to src, by a block of NA_TILE
+__device__ __forceinline__ void na_stage(const float2 *__restrict__ xy, const float *__restrict__ mass, int64_t s0,
+                                         int cnt, float4 *src) {
+#pragma unroll
+    for (int k = 0; k < NA_STILE / NA_TILE; ++k) {
+        const int j = k * NA_TILE + threadIdx.x;
+        if (j < cnt) {
+            const float2 p = xy[s0 + j];
+            src[j] = make_float4(p.x, p.y, mass[s0 + j], 0.f);
+        }
+    }
+}
+
+// A stage's sum v enters the compensated running total s (c: the rounding so far)
+__device__ __forceinline__ void na_add(float v, float &s, float &c) {
+    const float y = v - c, t = s + y;
+    c = (t - s) - y;
+    s = t;
+}
+
+// F of a node at z from its repulsion sum and attraction (the repulsion rounded before the attraction)
+__device__ __forceinline__ float2 na_total(float m, float kr, float kg, float sx, float sy, float2 a, float2 z) {
+    const float km = kr * m, kgm = kg * m;
+    const float2 fr = make_float2(__fmul_rn(km, sx), __fmul_rn(km, sy));
+    return make_float2((fr.x + a.x) - kgm * z.x, (fr.y + a.y) - kgm * z.y);
+}
+
 // Forces of the cluster's NA_TILE targets: repulsion from all n nodes, plus
 // attraction and gravity.
 //
@@ -60,12 +88,11 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH
 // (two buffers, so one barrier a round).  A cluster has a block per stage and
 // one more, up to NA_CLUSTER: on a small component more would only share SMs
 // with the ones that work.  The blocks without a stage, or all of them,
-// share the attraction, entry after entry:
-// a lane for a node of few entries, for the others the warp loads 32 entries
-// at a time and adds them in order through shuffles.  No memory is needed
-// beyond the blocks' own.  One block per 512 targets with all stages, and a
-// kernel with one thread per node for the attraction, took 99.6 and 15.5 us
-// for 2,821 nodes.
+// share the attraction, entry after entry: a lane for a node of few entries,
+// for the others the warp loads 32 entries at a time and adds them in order
+// through shuffles.  No memory is needed beyond the blocks' own.  One block
+// per 512 targets with all stages, and a kernel with one thread per node for
+// the attraction, took 99.6 and 15.5 us for 2,821 nodes.
 __global__ void __launch_bounds__(NA_TILE)
     na_force_kernel(const float2 *__restrict__ xy, const float *__restrict__ mass, const int64_t *__restrict__ off,
                     const int32_t *__restrict__ adj, int64_t n, float kr, float kg, float2 *__restrict__ f) {
@@ -142,14 +169,7 @@ __global__ void __launch_bounds__(NA_TILE)
         const int64_t s0 = (k0 + rank) * NA_STILE;
         const int cnt = (int)(s0 >= n ? 0 : (n - s0 < NA_STILE ? n - s0 : NA_STILE));
         __syncthreads();
-#pragma unroll
-        for (int k = 0; k < NA_STILE / NA_TILE; ++k) {
-            const int j = k * NA_TILE + threadIdx.x;
-            if (j < cnt) {
-                const float2 p = xy[s0 + j];
-                src[j] = make_float4(p.x, p.y, mass[s0 + j], 0.f);
-            }
-        }
+        na_stage(xy, mass, s0, cnt, src);
         __syncthreads();
         float ax = 0.f, ay = 0.f;
         // (the node itself adds 0)
@@ -160,25 +180,123 @@ __global__ void __launch_bounds__(NA_TILE)
             const int m = (int)(stages - k0 < blocks ? stages - k0 : blocks);
             for (int r = 0; r < m; ++r) {                // compensated running total of the stage sums
                 const float2 v = cluster.map_shared_rank(&part[0][0], r)[buf * NA_TILE + threadIdx.x];
-                float y = v.x - cx;
-                float t = sx + y;
-                cx = (t - sx) - y;
-                sx = t;
-                y = v.y - cy;
-                t = sy + y;
-                cy = (t - sy) - y;
-                sy = t;
+                na_add(v.x, sx, cx);
+                na_add(v.y, sy, cy);
             }
         }
     }
     if (rank == 0 && q < n) {
-        const float m = mass[q], km = kr * m;
         const float2 a = cluster.map_shared_rank(&satt[0], first + threadIdx.x / share)[threadIdx.x % share];
-        const float2 fr = make_float2(__fmul_rn(km, sx), __fmul_rn(km, sy));   // rounded before the attraction
-        const float kgm = kg * m;
-        f[q] = make_float2((fr.x + a.x) - kgm * z.x, (fr.y + a.y) - kgm * z.y);
+        f[q] = na_total(mass[q], kr, kg, sx, sy, a, z);
     }
     cluster.sync();                                      // no block leaves while block 0 reads its memory
+}
+
+// Attraction of the warp's nodes q, a lane each (ok: the lane has one), in
+// the order and the manner of na_force_kernel, which has it written out: with
+// a call of this it ran 3 % slower, at two registers less.
+__device__ __forceinline__ float2 na_attraction(const float2 *__restrict__ xy, const int64_t *__restrict__ off,
+                                                const int32_t *__restrict__ adj, int64_t q, bool ok) {
+    const int lane = threadIdx.x & 31;
+    const int64_t e0 = ok ? off[q] : 0, deg = ok ? off[q + 1] - e0 : 0;
+    const float2 p = ok ? xy[q] : make_float2(0.f, 0.f);
+    float ax = 0.f, ay = 0.f;
+    if (deg <= NA_LANE_DEG) {
+        float2 o[NA_LANE_DEG];
+#pragma unroll
+        for (int e = 0; e < NA_LANE_DEG; ++e) o[e] = e < deg ? xy[adj[e0 + e]] : p;
+#pragma unroll
+        for (int e = 0; e < NA_LANE_DEG; ++e) {
+            if (e < deg) {
+                ax -= p.x - o[e].x;
+                ay -= p.y - o[e].y;
+            }
+        }
+    }
+    unsigned more = __ballot_sync(0xffffffffu, deg > NA_LANE_DEG);
+    while (more) {
+        const int l = __ffs(more) - 1;
+        more &= more - 1;
+        const int64_t f0 = __shfl_sync(0xffffffffu, e0, l), d = __shfl_sync(0xffffffffu, deg, l);
+        const float px = __shfl_sync(0xffffffffu, p.x, l), py = __shfl_sync(0xffffffffu, p.y, l);
+        float sx = 0.f, sy = 0.f;
+        constexpr int C = 4;                             // loads of four rounds in flight
+        for (int64_t c0 = 0; c0 < d; c0 += 32 * C) {
+            float2 t[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int64_t e = c0 + c * 32 + lane;
+                const float2 o = e < d ? xy[adj[f0 + e]] : make_float2(px, py);
+                t[c] = make_float2(px - o.x, py - o.y);
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int m = (int)min((int64_t)32, d - c0 - c * 32);
+#pragma unroll 8
+                for (int j = 0; j < m; ++j) {
+                    sx -= __shfl_sync(0xffffffffu, t[c].x, j);
+                    sy -= __shfl_sync(0xffffffffu, t[c].y, j);
+                }
+            }
+        }
+        if (lane == l) {
+            ax = sx;
+            ay = sy;
+        }
+    }
+    return make_float2(ax, ay);
+}
+
+// The same for a component with targets enough to fill the chip without a
+// split of the stages: a block has 2 NA_TILE targets, two a thread in packed
+// FP32x2 arithmetic, and all stages, so that a source is read from shared
+// memory once for two pairs and no block waits for another.  Bound by issue and
+// the MUFU; the sums are the cluster kernel's bit for bit.  The line lies where
+// the blocks are some seven an SM: on 131,072 nodes 5.73 ms an iteration with
+// the clusters and 5.97 with this, on 196,608 12.8 and 12.9, on 262,144 22.8
+// and 19.8, on 1,048,576 363 and 270 (two scalar targets a thread in blocks
+// of 512, with the attraction in a kernel of its own: 339).
+constexpr int64_t NA_WIDE_MIN = 1 << 18;
+
+__global__ void __launch_bounds__(NA_TILE)
+    na_force_wide_kernel(const float2 *__restrict__ xy, const float *__restrict__ mass,
+                         const int64_t *__restrict__ off, const int32_t *__restrict__ adj, int64_t n, float kr,
+                         float kg, float2 *__restrict__ f) {
+    __shared__ float4 src[NA_STILE];
+    const int64_t q0 = (int64_t)blockIdx.x * (2 * NA_TILE) + threadIdx.x;
+    float2 z[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) z[r] = q0 + r * NA_TILE < n ? xy[q0 + r * NA_TILE] : make_float2(0.f, 0.f);
+    // negated targets and sums: each operation is the sign mirror of p2p_chain's
+    const float2 nzx = make_float2(-z[0].x, -z[1].x), nzy = make_float2(-z[0].y, -z[1].y);
+    float sx[2] = {0.f, 0.f}, sy[2] = {0.f, 0.f}, cx[2] = {0.f, 0.f}, cy[2] = {0.f, 0.f};
+    for (int64_t s0 = 0; s0 < n; s0 += NA_STILE) {
+        const int cnt = (int)(n - s0 < NA_STILE ? n - s0 : NA_STILE);
+        __syncthreads();
+        na_stage(xy, mass, s0, cnt, src);
+        __syncthreads();
+        float2 gx = make_float2(0.f, 0.f), gy = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int j = 0; j < cnt; ++j) {
+            const float4 q = src[j];
+            const float2 dx = __fadd2_rn(make_float2(q.x, q.x), nzx), dy = __fadd2_rn(make_float2(q.y, q.y), nzy);
+            const float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+            const float2 inv = make_float2(rcp_approx(fmaxf(r2.x, 1e-30f)), rcp_approx(fmaxf(r2.y, 1e-30f)));
+            const float2 w = __fmul2_rn(make_float2(q.z, q.z), inv);
+            gx = __ffma2_rn(w, dx, gx);
+            gy = __ffma2_rn(w, dy, gy);
+        }
+        na_add(-gx.x, sx[0], cx[0]);
+        na_add(-gx.y, sx[1], cx[1]);
+        na_add(-gy.x, sy[0], cy[0]);
+        na_add(-gy.y, sy[1], cy[1]);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int64_t q = q0 + r * NA_TILE;
+        const float2 a = na_attraction(xy, off, adj, q, q < n);
+        if (q < n) f[q] = na_total(mass[q], kr, kg, sx[r], sy[r], a, z[r]);
+    }
 }
 
 // Swing and traction sums of the nodes of the block's tile (256 threads; the
@@ -370,20 +488,25 @@ void fa2_iteration_noalloc(bgl_ctx *c, int64_t n, const int64_t *d_off, const in
     unsigned char *scratch = c->noalloc_scratch;
     BGL_REQUIRE(scratch != nullptr, "noalloc: the context has no scratch address");
     cudaStream_t s = c->stream;
-    const unsigned blocks = (unsigned)std::min<int64_t>(NA_CLUSTER, (n + NA_STILE - 1) / NA_STILE + 1);
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = blocks;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(na_blocks(n, NA_TILE) * blocks);
-    cfg.blockDim = dim3(NA_TILE);
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    BGL_CUDA(cudaLaunchKernelEx(&cfg, na_force_kernel, (const float2 *)d_xy, d_mass, d_off, d_adj, n, (float)p->kr,
-                                (float)p->kg, d_f));
-    BGL_LAUNCH_CHECK();
+    if (n < NA_WIDE_MIN) {
+        attr.val.clusterDim.x = (unsigned)std::min<int64_t>(NA_CLUSTER, (n + NA_STILE - 1) / NA_STILE + 1);
+        cfg.gridDim = dim3(na_blocks(n, NA_TILE) * attr.val.clusterDim.x);
+        cfg.blockDim = dim3(NA_TILE);
+        BGL_CUDA(cudaLaunchKernelEx(&cfg, na_force_kernel, (const float2 *)d_xy, d_mass, d_off, d_adj, n,
+                                    (float)p->kr, (float)p->kg, d_f));
+        BGL_LAUNCH_CHECK();
+    } else {
+        na_force_wide_kernel<<<na_blocks(n, 2 * NA_TILE), NA_TILE, 0, s>>>(d_xy, d_mass, d_off, d_adj, n,
+                                                                          (float)p->kr, (float)p->kg, d_f);
+        BGL_LAUNCH_CHECK();
+    }
     const unsigned tiles = na_blocks(n, NA_RED_TILE);
     if (tiles <= NA_CLUSTER) {
         attr.val.clusterDim.x = tiles;

@@ -1,0 +1,51 @@
+"""Dispatch rules whose line lies above the sizes of the other tests.
+
+* bgl_fa2_iteration_noalloc: from 262,144 nodes on a block has two targets a
+  thread and all stages; below, the stages are spread over a cluster.  Forces
+  against the oracle on sampled nodes, to the 1e-5 of the sum of the terms'
+  sizes that the exact forces are held to elsewhere."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _bgl():
+    import paper_2403_03504_gb300 as bgl
+    return bgl
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = _bgl().Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("n", [262143, 262144, 262273, 262401])
+def test_noalloc_forces_of_large_components(ctx, n):
+    """One node short of the line, on it, and last blocks of 129 and 257 - 256
+    targets; a hub of 3,000 entries and, last, a node of one."""
+    import torch
+    bgl = _bgl()
+    u, v = np.arange(n - 1), np.arange(1, n)
+    hub = np.arange(2, 3000)
+    g = bgl.Graph.from_edges(ctx, n, np.concatenate([u, np.zeros_like(hub)]), np.concatenate([v, hub]))
+    off, adj = g.csr()
+    g.destroy()
+    mass = np.diff(off) + 1.0
+    xy = synth.points(n, n, "uniform", scale=200.0)
+    dev = [torch.from_numpy(a).cuda() for a in (off, adj, mass.astype(np.float32), xy)]
+    f, fp = torch.zeros(n, 2, device="cuda"), torch.zeros(n, 2, device="cuda")
+    sg = torch.ones(1, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    ctx.fa2_iteration_noalloc(n, dev[0], dev[1], dev[2], dev[3], fp, f, sg, bgl.params(repulsion=bgl.REP_EXACT))
+    ctx.sync()
+    tg = np.unique(np.concatenate([np.random.default_rng(n).choice(n, 200, replace=False),
+                                   [0, 1, 2999, 3000, 127, 128, 255, 256, n - 130, n - 129, n - 2, n - 1]]))
+    o = oracle.fa2_forces(xy[:, 0], xy[:, 1], mass, off, adj, targets=tg)
+    ref = o["frep"] + o["fatt"] + o["fgrav"]
+    assert np.max(np.hypot(*(f.cpu().numpy()[tg] - ref).T) / o["sabs"]) <= 1e-5
