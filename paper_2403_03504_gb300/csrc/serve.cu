@@ -19,8 +19,9 @@
 // stamped with a per-worker counter (never cleared).  The visited nodes in
 // ascending id (local id = rank, so the subgraph does not depend on the order
 // of discovery) and their degree prefix sums come from one scan over the
-// marks, and the induced edges, listed per node in adjacency order, from a
-// count and a fill over the entries.
+// marks, or, in a large resident graph, from a sort of the visited nodes; and
+// the induced edges, listed per node in adjacency order, from a count and a
+// fill over the entries.
 #include <chrono>
 #include <condition_variable>
 #include <deque>
@@ -57,6 +58,13 @@ constexpr int KH_LANE_DEG = 8;         // frontier nodes up to this degree: one 
 constexpr int KH_HUB_DEG = 1024;       // above this degree: the whole grid
 constexpr int KH_TILE = 4096;          // nodes per tile of the scan over the marks
 constexpr int KH_CHUNK = 2048;         // adjacency entries per block of the edge kernels
+// Resident graphs from this size on: the visited nodes are sorted by id
+// instead of found by scans over the marks of all nodes, whose time goes with
+// the graph (two extractions of 426 nodes: 449 us with the scans and 529 with
+// the sort on 1,048,576 nodes, 534 and 551 on 8,388,608, 610 and 582 on
+// 16,777,216, 1,816 and 713 on 134,217,728, where one thread an edge and a
+// sort, with the host between the hops, took 1,439).
+constexpr int64_t KH_SORT_MIN = int64_t(1) << 24;
 
 // state of an extraction on the device
 struct KhState {
@@ -225,6 +233,17 @@ __global__ void __launch_bounds__(KH_TPB) kh_mark_kernel(const int32_t *__restri
         ++r;
         e += off[v + 1] - off[v];
     }
+}
+
+// Ranks and degrees of the visited nodes in ascending order
+__global__ void __launch_bounds__(KH_TPB) kh_rank_kernel(const int32_t *__restrict__ vis, int64_t n,
+                                                        const int64_t *__restrict__ off, int32_t *__restrict__ local,
+                                                        int64_t *__restrict__ deg) {
+    const int64_t r = (int64_t)blockIdx.x * KH_TPB + threadIdx.x;
+    if (r >= n) return;
+    const int32_t v = vis[r];
+    local[v] = (int32_t)r;
+    deg[r] = off[v + 1] - off[v];
 }
 
 // one block: the tiles' exclusive sums in place, the totals to st (of the
@@ -407,14 +426,28 @@ static int64_t khop_extract(bgl_ctx *ctx, const bgl_graph *R, KhopScratch &ws, i
             if (st.f0 == st.f1 || (int64_t)st.count > cap) break;
         }
     }
-    const unsigned tiles = (unsigned)((R->n + KH_TILE - 1) / KH_TILE);
-    kh_mark_kernel<<<tiles, KH_TPB, 0, s>>>(ws.stamp.p, epoch, R->n, R->off.p, ws.tiles.p, nullptr, nullptr, nullptr, 0);
-    BGL_LAUNCH_CHECK();
-    kh_tiles_kernel<<<1, KH_TPB, 0, s>>>(ws.tiles.p, tiles, ws.state.p, 0);
-    BGL_LAUNCH_CHECK();
-    kh_mark_kernel<<<tiles, KH_TPB, 0, s>>>(ws.stamp.p, epoch, R->n, R->off.p, ws.tiles.p, ws.vis.p, ws.local.p,
-                                            ws.dscan.p, cap);
-    BGL_LAUNCH_CHECK();
+    if (R->n >= KH_SORT_MIN) {
+        fetch();
+        if ((int64_t)st.count > cap) return -1;
+        const int64_t n = (int64_t)st.count;
+        BGL_CUDA(cudaMemcpyAsync(ws.vis.p, ws.found.p, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
+        radix_sort_u32(ctx, reinterpret_cast<uint32_t *>(ws.vis.p), nullptr, n, bits_for((uint64_t)R->n));
+        sort_check(ctx);
+        DevBuf<int64_t> deg(ctx->alloc, n);
+        kh_rank_kernel<<<kh_blocks(n), KH_TPB, 0, s>>>(ws.vis.p, n, R->off.p, ws.local.p, deg.p);
+        BGL_LAUNCH_CHECK();
+        scan_exclusive_i64(ctx, deg.p, ws.dscan.p, n, reinterpret_cast<int64_t *>(&ws.state.p->entries));
+    } else {
+        const unsigned tiles = (unsigned)((R->n + KH_TILE - 1) / KH_TILE);
+        kh_mark_kernel<<<tiles, KH_TPB, 0, s>>>(ws.stamp.p, epoch, R->n, R->off.p, ws.tiles.p, nullptr, nullptr,
+                                                nullptr, 0);
+        BGL_LAUNCH_CHECK();
+        kh_tiles_kernel<<<1, KH_TPB, 0, s>>>(ws.tiles.p, tiles, ws.state.p, 0);
+        BGL_LAUNCH_CHECK();
+        kh_mark_kernel<<<tiles, KH_TPB, 0, s>>>(ws.stamp.p, epoch, R->n, R->off.p, ws.tiles.p, ws.vis.p, ws.local.p,
+                                                ws.dscan.p, cap);
+        BGL_LAUNCH_CHECK();
+    }
     fetch();
     if ((int64_t)st.count > cap) return -1;
     const int64_t n = (int64_t)st.count, E = (int64_t)st.entries;

@@ -3,7 +3,11 @@
 * bgl_fa2_iteration_noalloc: from 262,144 nodes on a block has two targets a
   thread and all stages; below, the stages are spread over a cluster.  Forces
   against the oracle on sampled nodes, to the 1e-5 of the sum of the terms'
-  sizes that the exact forces are held to elsewhere."""
+  sizes that the exact forces are held to elsewhere.
+* k-hop neighbourhoods in a resident graph of 2^24 nodes and more come from a
+  sort of the visited nodes, in smaller ones from scans over the marks of all:
+  equal to the oracle's on both sides of the line.  A sort that gives up
+  (BGL_TEST_SORT_STALL=1, see test_gpu_recovery.py) is reported."""
 import numpy as np
 import pytest
 
@@ -49,3 +53,29 @@ def test_noalloc_forces_of_large_components(ctx, n):
     o = oracle.fa2_forces(xy[:, 0], xy[:, 1], mass, off, adj, targets=tg)
     ref = o["frep"] + o["fatt"] + o["fgrav"]
     assert np.max(np.hypot(*(f.cpu().numpy()[tg] - ref).T) / o["sabs"]) <= 1e-5
+
+
+@pytest.mark.parametrize("n", [(1 << 24) - 1, 1 << 24])
+def test_khop_in_a_large_graph(ctx, monkeypatch, n):
+    """A path whose node 0 is also joined to 2..1401 and to the last nodes."""
+    bgl = _bgl()
+    u, v = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32)
+    hub = np.concatenate([np.arange(2, 1402), np.arange(n - 40, n)]).astype(np.int32)
+    g = bgl.Graph.from_edges(ctx, n, np.concatenate([u, np.zeros_like(hub)]), np.concatenate([v, hub]))
+    off, adj = g.csr()
+    for seed, hops in ((0, 0), (0, 1), (n - 1, 2), (700, 2), (n // 2, 1), (n // 2, 2500), (n - 50, 11)):
+        ids, edges = oracle.khop(off, adj, seed, hops)
+        got = g.khop(seed, hops, 1 << 30)
+        assert np.array_equal(got[0], ids)
+        assert sorted(zip(np.minimum(got[1], got[2]).tolist(), np.maximum(got[1], got[2]).tolist())) == edges
+        assert np.array_equal(g.khop(seed, hops, len(ids))[0], ids)
+        if len(ids) > 1:
+            assert g.khop(seed, hops, len(ids) - 1) is None
+    if n >= 1 << 24:
+        monkeypatch.setenv("BGL_TEST_SORT_STALL", "1")
+        with pytest.raises(bgl.BglError) as e:
+            g.khop(n // 2, 2500, n)                  # 5,001 nodes: two tiles
+        assert e.value.status == -4
+        monkeypatch.delenv("BGL_TEST_SORT_STALL")
+        assert len(g.khop(n // 2, 2500, n)[0]) == 5001
+    g.destroy()
