@@ -210,6 +210,9 @@ bgl_status bgl_split(bgl_graph *g, int32_t kk_max_nodes, int64_t *n_kk, int64_t 
  * by kk_l * diameter / 2.  Components with one node sit at the origin.
  * xy_out[2 n_nodes] (host) receives x, y of node v at [2v], [2v+1], each in
  * its component's own frame.  Synchronises the stream.
+ * Device memory: components on the exact repulsion keep partial sums while
+ * they run, up to 64 bytes a node, and on those of 8,193 to 65,536 nodes up to
+ * 512 bytes a node but no more than 512 MiB for all of a call together.
  */
 bgl_status bgl_layout(bgl_graph *g, const bgl_params *p, float *xy_out);
 

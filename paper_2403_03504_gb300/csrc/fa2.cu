@@ -35,6 +35,15 @@ namespace {
 constexpr int EX_THREADS = 128, EX_WARPS = EX_THREADS / 32;
 constexpr int EX_STAGE = 1024;                 // sources summed before they enter the compensated total
 constexpr int64_t EX_SPLIT_MAX_N = 1 << 16;    // components up to this size: a block per stage (partial sums in memory)
+// Partial sums take 8 bytes a node and stage: up to 64 a node for components
+// of up to EX_SPLIT_FREE_N nodes, 512 on 65,536.  All components above
+// EX_SPLIT_FREE_N of a run together get EX_PART_BYTES, smallest first: sixteen
+// of 65,536.  More have tiles enough to fill the chip without a split (of
+// 60,000 nodes, times of some iterations split and not: 3 components 24.6 and
+// 34.1 ms, 10 33.5 and 34.6, 16 52.9 and 52.9, 30 52.5 and 48.8, the last with
+// 875 MB of partial sums).
+constexpr int64_t EX_SPLIT_FREE_N = 8 * EX_STAGE;
+constexpr int64_t EX_PART_BYTES = int64_t(512) << 20;
 #ifndef BGL_EXACT_WIDE_WARPS
 #define BGL_EXACT_WIDE_WARPS 3000              // warps at two targets per lane from which a run takes two
 #endif
@@ -583,9 +592,9 @@ inline unsigned nblocks(int64_t n, int t) { return (unsigned)std::max<int64_t>(1
 
 // Blocks of the exact sum over the given components (indices >= c0): for each
 // tile of EX_THREADS R targets one for its attraction, and one for each stage
-// of its sources, or for all of them in a component of more than
-// EX_SPLIT_MAX_N nodes (the partial sums of more would take n^2 / 128 bytes,
-// and it has tiles enough).
+// of its sources, or for all of them in a component of more nodes than
+// split_max (the partial sums would take n^2 / 128 bytes, and there are tiles
+// enough).  The order of the sums is the same either way.
 struct ExactSum {
     DevBuf<ExBlock> blk;
     DevBuf<float2> part, group;
@@ -595,7 +604,20 @@ struct ExactSum {
 
     // reps: every tile so many times (each copy writes the same forces)
     void make(bgl_graph *g, int64_t c0, int64_t c1, const std::vector<int64_t> &comps, int reps = 1) {
-        auto parts_of = [](int64_t n) { return n <= EX_SPLIT_MAX_N ? (n + EX_STAGE - 1) / EX_STAGE : int64_t(1); };
+        int64_t split_max = EX_SPLIT_FREE_N, bytes = 0;
+        for (auto it = comps.rbegin(); it != comps.rend(); ++it) {            // (sizes descend)
+            const int64_t n = g->h_comp_off[*it + 1] - g->h_comp_off[*it];
+            if (n <= EX_SPLIT_FREE_N) continue;
+            bytes += (n + 255) / 256 * 256 * ((n + EX_STAGE - 1) / EX_STAGE) * (int64_t)sizeof(float2) * reps;
+            if (n > EX_SPLIT_MAX_N || bytes > EX_PART_BYTES) {
+                split_max = std::min(split_max, n - 1);                       // (none of this size)
+                break;
+            }
+            split_max = n;
+        }
+        auto parts_of = [split_max](int64_t n) {
+            return n <= split_max ? (n + EX_STAGE - 1) / EX_STAGE : int64_t(1);
+        };
         int64_t wide = 0;
         for (int64_t c : comps) {
             const int64_t n = g->h_comp_off[c + 1] - g->h_comp_off[c];

@@ -7,7 +7,11 @@
 * k-hop neighbourhoods in a resident graph of 2^24 nodes and more come from a
   sort of the visited nodes, in smaller ones from scans over the marks of all:
   equal to the oracle's on both sides of the line.  A sort that gives up
-  (BGL_TEST_SORT_STALL=1, see test_gpu_recovery.py) is reported."""
+  (BGL_TEST_SORT_STALL=1, see test_gpu_recovery.py) is reported.
+* The partial sums of exact components above 8,192 nodes take at most 512 MiB
+  a run, whatever their number (64 bytes a node below), with the same bits as
+  when a component has them all to itself; and a server's footprint estimate
+  bounds what a request of one such component takes."""
 import numpy as np
 import pytest
 
@@ -78,4 +82,47 @@ def test_khop_in_a_large_graph(ctx, monkeypatch, n):
         assert e.value.status == -4
         monkeypatch.delenv("BGL_TEST_SORT_STALL")
         assert len(g.khop(n // 2, 2500, n)[0]) == 5001
+    g.destroy()
+
+
+def _trees(comps, n, arity):
+    """Trees of n nodes, the parent of a tree's node i being (i - 1) // arity."""
+    i = np.arange(1, n)
+    base = np.arange(comps)[:, None] * n
+    return comps * n, (base + (i - 1) // arity).ravel(), (base + i).ravel()
+
+
+def test_partial_sums_of_many_exact_components_are_bounded():
+    import torch
+    bgl = _bgl()
+    comps, size = 30, 60000
+    n, u, v = _trees(comps, size, 3)
+    with bgl.Context(0) as c:
+        g = bgl.Graph.from_edges(c, n, u, v)
+        g.components(labels=False)
+        p = bgl.params(seed=5, fa2_iters=1, repulsion=bgl.REP_EXACT)
+        free = torch.cuda.mem_get_info()[0]
+        xy = g.layout(p)
+        taken = free - torch.cuda.mem_get_info()[0]
+        # positions, forces and tiles: some 70 bytes a node; unbounded partial sums would take 470 more
+        assert taken <= (512 << 20) + 128 * n, taken
+        off, _, nodes = g.component_nodes()
+        for k in (0, comps - 1):
+            ids = nodes[off[k]:off[k + 1]]
+            x, y = oracle.init_positions(5, ids)
+            alone, _ = g.fa2_step(k, p, 1, np.stack([x, y], 1).astype(np.float32))
+            assert np.array_equal(alone, xy[ids])
+        g.destroy()
+
+
+def test_footprint_estimate_bounds_an_exact_request(ctx):
+    bgl = _bgl()
+    n, u, v = _trees(1, 65536, 50)
+    g = bgl.Graph.from_edges(ctx, n, u, v)
+    srv = bgl.Server(g, slots=1)
+    for size, hops in ((n, 3), (2551, 2)):
+        status, k, _, nbytes = srv.wait(srv.submit(0, hops, bgl.params(fa2_iters=1, repulsion=bgl.REP_EXACT)))
+        assert status == 0 and k == size
+        assert 0 < nbytes[1] <= nbytes[0]
+    srv.close()
     g.destroy()
