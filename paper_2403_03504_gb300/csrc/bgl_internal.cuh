@@ -353,8 +353,9 @@ KkRun *kk_prepare(bgl_graph *g, int64_t c0, int64_t c1);
 void kk_destroy(KkRun *run);
 int kk_classes(const KkRun *run);
 void kk_enqueue_distances(const KkRun *run, cudaStream_t s);   // before any class's kk_enqueue
+// placed (may be null) completes once all of the class's blocks have started
 void kk_enqueue(const KkRun *run, int i, const bgl_params *p, float2 *xy, int64_t qbase, bool init, int sweeps,
-                int32_t *d_out, cudaStream_t s);
+                int32_t *d_out, cudaStream_t s, cudaEvent_t placed = nullptr);
 void kk_distances(bgl_graph *g, int64_t c, int32_t *d_out_dev);
 
 // ForceAtlas2 on components [c0, c1) (exact or FMM per component);

@@ -1095,6 +1095,29 @@ static void run_iterations_host(Fa2Run &run, int iters, double *d_stats, const S
 // 30 us for an FMM iteration, which two to a turn win back in 24 iterations.
 static int loop_unroll(const Fa2Run &run, int iters) { return run.fmm.empty() ? 4 : (iters >= 24 ? 2 : 1); }
 
+// Gives every kernel of a graph the shared-memory split that the Kamada-Kawai
+// kernels ask for.  An SM changes its split only when it is empty: beside
+// Kamada-Kawai classes an exact sum that wants another one keeps SMs from
+// them, and their blocks pile up on the others (50 exact iterations of 6,000
+// nodes beside 1,000 components of 3 to 200 nodes: 27.8 to 68 ms without this,
+// 27 to 31 with it; beside 20,000 64 to 89 and 35 to 45).  The FMM's kernels
+// are better with their own (10,000 nodes alone: 4.2 ms, 4.5 with this one;
+// 100,000 beside 100,000 components of 3 to 30: 13.65 and 13.96).
+static void widest_shared_memory(cudaGraph_t graph) {
+    size_t n = 0;
+    BGL_CUDA(cudaGraphGetNodes(graph, nullptr, &n));
+    std::vector<cudaGraphNode_t> nodes(n);
+    if (n) BGL_CUDA(cudaGraphGetNodes(graph, nodes.data(), &n));
+    cudaLaunchAttributeValue v = {};
+    v.sharedMemCarveout = (unsigned)cudaSharedmemCarveoutMaxShared;
+    for (cudaGraphNode_t nd : nodes) {
+        cudaGraphNodeType t;
+        BGL_CUDA(cudaGraphNodeGetType(nd, &t));
+        if (t == cudaGraphNodeTypeKernel)
+            BGL_CUDA(cudaGraphKernelNodeSetAttribute(nd, cudaLaunchAttributePreferredSharedMemoryCarveout, &v));
+    }
+}
+
 // `n` iterations captured on s into graph `into` (null: a new graph, which
 // is returned); loop: stepped by the last one.  Adds the kernels to `kernels`.
 static cudaGraph_t capture_iterations(Fa2Run &run, double *d_stats, int n, cudaGraph_t into, const LoopCtl &loop,
@@ -1149,14 +1172,17 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
     cudaGraphExec_t exec = nullptr;
     BGL_CUDA(cudaGraphCreate(&graph, 0));
     int64_t kernels = 0;
+    const bool widest = run.exact.n_blk > 0 && side;
     try {
         const int unroll = loop_unroll(run, iters), turns = iters / unroll, rest = iters - turns * unroll;
         cudaGraphNode_t rnode = nullptr;
         if (rest > 0) {
-            cudaGraph_t child = capture_iterations(run, d_stats, rest, nullptr, LoopCtl{}, kernels);
-            const cudaError_t e = cudaGraphAddChildGraphNode(&rnode, graph, nullptr, 0, child);
-            cudaGraphDestroy(child);
-            BGL_CUDA(e);
+            struct Child {
+                cudaGraph_t g;
+                ~Child() { cudaGraphDestroy(g); }
+            } child{capture_iterations(run, d_stats, rest, nullptr, LoopCtl{}, kernels)};
+            if (widest) widest_shared_memory(child.g);
+            BGL_CUDA(cudaGraphAddChildGraphNode(&rnode, graph, nullptr, 0, child.g));
         }
         if (turns > 0) {
             LoopCtl ctl;
@@ -1173,6 +1199,7 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
             int64_t per_turn = 0;
             capture_iterations(run, d_stats, unroll, cp.conditional.phGraph_out[0], ctl, per_turn);
             kernels += per_turn * turns;
+            if (widest) widest_shared_memory(cp.conditional.phGraph_out[0]);
         }
         if (side) {
             // the side work, captured on the run's side stream (it may fork

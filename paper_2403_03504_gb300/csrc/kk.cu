@@ -500,6 +500,7 @@ struct KkClass {
     DevBuf<uint8_t> gdist;
     DevBuf<int64_t> gdist_off;
     DevBuf<int> gdiam;
+    int64_t blocks() const { return (c1 - c0 + gpb - 1) / gpb; }
 };
 
 struct KkRun {
@@ -610,19 +611,29 @@ void kk_enqueue_distances(const KkRun *run, cudaStream_t s) {
 
 template <int G, int CPL>
 static void kk_enqueue_class(const KkRun &run, const KkClass &k, const bgl_params *p, float2 *xy, int64_t qbase,
-                             bool init, int sweeps, int32_t *d_out, cudaStream_t s) {
+                             bool init, int sweeps, int32_t *d_out, cudaStream_t s, cudaEvent_t placed) {
     const KKArgs a = kk_args(run, k, p, xy, qbase, init, sweeps, d_out);
-    const int64_t blocks = (a.nc + k.gpb - 1) / k.gpb;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeLaunchCompletionEvent;
+    attr.val.launchCompletionEvent.event = placed;
+    attr.val.launchCompletionEvent.flags = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)k.blocks());
+    cfg.blockDim = dim3(G * k.gpb);
+    cfg.dynamicSmemBytes = k.smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = placed ? 1 : 0;
     bool launched = false;
     if constexpr (CPL % 4 == 0) {
         if (k.gdist.p) {
-            kk_kernel<G, CPL, true><<<(unsigned)blocks, G * k.gpb, k.smem, s>>>(a);
+            BGL_CUDA(cudaLaunchKernelEx(&cfg, kk_kernel<G, CPL, true>, a));
             launched = true;
         }
     }
     if (!launched) {
         BGL_REQUIRE(!k.gdist.p, "kk: distances in global memory need a multiple of 4 nodes per lane");
-        kk_kernel<G, CPL, false><<<(unsigned)blocks, G * k.gpb, k.smem, s>>>(a);
+        BGL_CUDA(cudaLaunchKernelEx(&cfg, kk_kernel<G, CPL, false>, a));
     }
     BGL_LAUNCH_CHECK();
 }
@@ -684,32 +695,32 @@ int kk_classes(const KkRun *run) { return (int)run->cls.size(); }
 
 // launches size class i on stream s
 void kk_enqueue(const KkRun *run, int i, const bgl_params *p, float2 *xy, int64_t qbase, bool init, int sweeps,
-                int32_t *d_out, cudaStream_t s) {
+                int32_t *d_out, cudaStream_t s, cudaEvent_t placed) {
     BGL_RANGE("Kamada-Kawai: Newton sweeps of one size class (Section 3.1)");
     const KkClass &k = *run->cls[i];
     switch (k.G * 64 + k.CPL) {
 #if BGL_KK_WIDE == 2
-        case 8 * 64 + 32: kk_enqueue_class<8, 32>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 8 * 64 + 16: kk_enqueue_class<8, 16>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 8 * 64 + 8: kk_enqueue_class<8, 8>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
+        case 8 * 64 + 32: kk_enqueue_class<8, 32>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 8 * 64 + 16: kk_enqueue_class<8, 16>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 8 * 64 + 8: kk_enqueue_class<8, 8>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
 #elif BGL_KK_WIDE == 1
-        case 16 * 64 + 16: kk_enqueue_class<16, 16>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 16 * 64 + 8: kk_enqueue_class<16, 8>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 16 * 64 + 4: kk_enqueue_class<16, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
+        case 16 * 64 + 16: kk_enqueue_class<16, 16>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 16 * 64 + 8: kk_enqueue_class<16, 8>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 16 * 64 + 4: kk_enqueue_class<16, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
 #else
-        case 32 * 64 + 8: kk_enqueue_class<32, 8>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 32 * 64 + 4: kk_enqueue_class<32, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 32 * 64 + 2: kk_enqueue_class<32, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
+        case 32 * 64 + 8: kk_enqueue_class<32, 8>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 32 * 64 + 4: kk_enqueue_class<32, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 32 * 64 + 2: kk_enqueue_class<32, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
 #endif
 #if BGL_KK_NARROW
-        case 8 * 64 + 4: kk_enqueue_class<8, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 4 * 64 + 4: kk_enqueue_class<4, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
+        case 8 * 64 + 4: kk_enqueue_class<8, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 4 * 64 + 4: kk_enqueue_class<4, 4>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
 #else
-        case 16 * 64 + 2: kk_enqueue_class<16, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        case 8 * 64 + 2: kk_enqueue_class<8, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
+        case 16 * 64 + 2: kk_enqueue_class<16, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        case 8 * 64 + 2: kk_enqueue_class<8, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
 #endif
-        case 4 * 64 + 2: kk_enqueue_class<4, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
-        default: kk_enqueue_class<4, 1>(*run, k, p, xy, qbase, init, sweeps, d_out, s); break;
+        case 4 * 64 + 2: kk_enqueue_class<4, 2>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
+        default: kk_enqueue_class<4, 1>(*run, k, p, xy, qbase, init, sweeps, d_out, s, placed); break;
     }
 }
 

@@ -11,7 +11,10 @@
 * The partial sums of exact components above 8,192 nodes take at most 512 MiB
   a run, whatever their number (64 bytes a node below), with the same bits as
   when a component has them all to itself; and a server's footprint estimate
-  bounds what a request of one such component takes."""
+  bounds what a request of one such component takes.
+* Kamada-Kawai classes of 608 blocks and more fill the chip; beside classes the
+  exact iterations' kernels ask for their shared-memory split: every component
+  gets the layout that it gets alone."""
 import numpy as np
 import pytest
 
@@ -125,4 +128,24 @@ def test_footprint_estimate_bounds_an_exact_request(ctx):
         assert status == 0 and k == size
         assert 0 < nbytes[1] <= nbytes[0]
     srv.close()
+    g.destroy()
+
+
+def test_layout_beside_classes_that_fill_the_chip(ctx):
+    """20,000 components of 3 to 50 nodes (some 900 blocks) beside one of 3,000
+    in the exact sum."""
+    bgl = _bgl()
+    size = 3000
+    sizes, u, v = synth.forest(8, 20000, 3.0, 50.0)
+    base = int(sizes.sum())
+    n, gu, gv = _trees(1, size, 3)
+    g = bgl.Graph.from_edges(ctx, base + n, np.concatenate([u, base + gu]), np.concatenate([v, base + gv]))
+    g.components(labels=False)
+    p = bgl.params(seed=6, fa2_iters=30, kk_sweeps=20, ksmax=0.05, repulsion=bgl.REP_EXACT)
+    xy = g.layout(p)
+    x, y = oracle.init_positions(6, np.arange(base, base + n))
+    alone, _ = g.fa2_step(0, p, 30, np.stack([x, y], 1).astype(np.float32))
+    assert np.array_equal(xy[base:], alone)
+    p.fa2_iters = 0                                  # the classes without iterations beside them
+    assert np.array_equal(xy[:base], g.layout(p)[:base])
     g.destroy()
