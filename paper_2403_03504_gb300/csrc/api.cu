@@ -268,7 +268,9 @@ void layout_device(bgl_graph *g, const bgl_params *p, float *d_xy_out) {
         // 400,000 nodes took 44 to 89 ms and take 38, beside 60,000 38 (now and
         // then 89) and 35.8, alone 34 to 48 and 33.9.
         kk_enqueue_distances(kk.get(), c->stream);
-        SideWork kk_work = [&](cudaStream_t s) {
+        SideWork kk_work;
+        kk_work.blocks = kk_blocks(kk.get());
+        kk_work.enqueue = [&](cudaStream_t s) {
             // one stream per size class, forked from and joined back to stream s
             BGL_CUDA(cudaEventRecord(kev[nk], s));
             for (int i = 0; i < nk; ++i) {
@@ -284,7 +286,7 @@ void layout_device(bgl_graph *g, const bgl_params *p, float *d_xy_out) {
             init_positions(g, p, xy.p, 0, q_fa2);
             fa2_layout(g, p, xy.p, 0, 0, g->n_fa2, p->fa2_iters, nullptr, nk ? kk_work : SideWork());
         } else if (nk) {
-            kk_work(c->stream);
+            kk_work.enqueue(c->stream);
         }
         BGL_CUDA(cudaStreamSynchronize(c->stream));
     } catch (...) {

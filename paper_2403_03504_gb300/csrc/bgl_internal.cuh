@@ -352,6 +352,7 @@ struct KkRun;
 KkRun *kk_prepare(bgl_graph *g, int64_t c0, int64_t c1);
 void kk_destroy(KkRun *run);
 int kk_classes(const KkRun *run);
+int64_t kk_blocks(const KkRun *run);                           // thread blocks of all classes
 void kk_enqueue_distances(const KkRun *run, cudaStream_t s);   // before any class's kk_enqueue
 // placed (may be null) completes once all of the class's blocks have started
 void kk_enqueue(const KkRun *run, int i, const bgl_params *p, float2 *xy, int64_t qbase, bool init, int sweeps,
@@ -365,7 +366,14 @@ void kk_distances(bgl_graph *g, int64_t c, int32_t *d_out_dev);
 // Work that runs beside the ForceAtlas2 iterations: enqueued on the given
 // stream (it may fork to streams of its own and must join back); with the
 // device-side loop it is captured and launched in the same graph.
-using SideWork = std::function<void(cudaStream_t)>;
+struct SideWork {
+    std::function<void(cudaStream_t)> enqueue;
+    int64_t blocks = 0;      // thread blocks of its kernels
+    explicit operator bool() const { return (bool)enqueue; }
+    // whether it leaves little room on the SMs: from four blocks each on (of
+    // four warps and up to some 40 KB)
+    bool fills(const bgl_ctx *c) const { return blocks >= 4 * (int64_t)c->num_sms; }
+};
 void fa2_layout(bgl_graph *g, const bgl_params *p, float2 *xy, int64_t qbase, int64_t c0, int64_t c1, int iters,
                 double *d_stats, const SideWork &side = SideWork());
 // Assembly of the component layouts into one frame (assemble.cu, Section 4):

@@ -1034,7 +1034,7 @@ static void run_iterations_host(Fa2Run &run, int iters, double *d_stats, const S
         BGL_CUDA(cudaEventRecord(run.ev_fork, s));
         BGL_CUDA(cudaStreamWaitEvent(run.side, run.ev_fork, 0));
         try {
-            side(run.side);
+            side.enqueue(run.side);
             BGL_CUDA(cudaEventRecord(side_done, run.side));
         } catch (...) {
             cudaEventDestroy(side_done);
@@ -1157,7 +1157,7 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
     bgl_ctx *ctx = run.g->ctx;
     cudaStream_t s = ctx->stream;
     if (iters <= 0) {
-        if (side) side(s);
+        if (side) side.enqueue(s);
         return;
     }
     BGL_CUDA(cudaMemsetAsync(ctx->d_flag + 1, 0, sizeof(int), s));
@@ -1208,7 +1208,7 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
             BGL_CUDA(cudaStreamBeginCapture(run.side, cudaStreamCaptureModeThreadLocal));
             ctx->alloc->forbid = true;
             try {
-                side(run.side);
+                side.enqueue(run.side);
             } catch (...) {
                 ctx->alloc->forbid = false;
                 cudaGraph_t tmp = nullptr;
@@ -1247,11 +1247,12 @@ static void run_iterations(Fa2Run &run, int iters, double *d_stats, const SideWo
 void fa2_layout(bgl_graph *g, const bgl_params *p, float2 *xy, int64_t qbase, int64_t c0, int64_t c1, int iters,
                 double *d_stats, const SideWork &side) {
     if (c1 <= c0 || iters <= 0) {
-        if (side) side(g->ctx->stream);
+        if (side) side.enqueue(g->ctx->stream);
         return;
     }
     BGL_RANGE("ForceAtlas2 iterations (Section 3.2)");
     Fa2Run run(g, p, xy, qbase, c0, c1);
+    for (FmmPlan *pl : run.fmm) fmm_crowded(pl, side.fills(g->ctx));
     run_iterations(run, iters, d_stats, side);
 }
 

@@ -472,6 +472,10 @@ __global__ void __launch_bounds__(OS_THREADS) keys_kernel(const float2 *__restri
 // stable sort on the same bits).  On a few tiles those are all latency: keys,
 // two passes that return at once and two that do not; an iteration on 8,888
 // points takes 87.1 us with them and 79.5 with this, on 27,980 104.5 and 94.7.
+// But a cluster needs room on all its SMs at once: beside 20,000 Kamada-Kawai
+// components of 3 to 50 nodes 50 iterations on 10,000 points took 7.4 ms with
+// it, 6.5 without (28,000: 7.9 and 7.3), beside 8,000 components 5.19 and 5.30;
+// so beside work that fills the SMs the separate kernels stay.
 constexpr int SMALL_TILES = 8;         // the portable cluster size
 
 __global__ void __launch_bounds__(OS_THREADS) points_small_kernel(const float2 *__restrict__ xy,
@@ -2511,6 +2515,7 @@ static std::vector<uint4> m2l_fragments(int p) {
 struct FmmPlan {
     bgl_graph *g = nullptr;
     OsWait wait;           // bounded waits of the sort: error word, poll limit, test stall
+    bool crowded = false;  // (fmm_crowded)
     bool fused = false;    // fused ForceAtlas2 iteration (fmm_fuse): no bounding-box kernel, swing in combine
     FmmFuse fz;
     DevBuf<double2> spart; // swing/traction partial sums of the combine blocks
@@ -2747,7 +2752,7 @@ static void phase_points(FmmPlan *pl, const float2 *xl, cudaStream_t s) {
             BGL_LAUNCH_CHECK();
         }
         // (the test aid of the look-back's waits needs the passes that have one)
-        if (n <= SMALL_TILES * OS_TILE && !pl->wait.stall_first) {
+        if (n <= SMALL_TILES * OS_TILE && !pl->crowded && !pl->wait.stall_first) {
             cudaLaunchAttribute attr;
             attr.id = cudaLaunchAttributeClusterDimension;
             attr.val.clusterDim.x = nblk(n, OS_TILE);
@@ -3052,6 +3057,8 @@ void fmm_profile(FmmPlan *pl, const float2 *xy, int64_t qbase, int reps, double 
     out[16] = (double)skip_last;
     out[17] = (double)h[6];
 }
+
+void fmm_crowded(FmmPlan *pl, bool crowded) { pl->crowded = crowded; }
 
 void fmm_fuse(FmmPlan *pl, const FmmFuse &fz) {
     bgl_ctx *ctx = pl->g->ctx;

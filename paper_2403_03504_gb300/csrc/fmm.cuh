@@ -37,6 +37,8 @@ struct FmmFuse {
     int *bad = nullptr;              // set when a position becomes non-finite
 };
 void fmm_fuse(FmmPlan *pl, const FmmFuse &fz);
+// whether other work fills the SMs beside the plan's evaluations
+void fmm_crowded(FmmPlan *pl, bool crowded);
 // the root square of positions xy (before the first fused evaluation)
 void fmm_root(FmmPlan *pl, const float2 *xy, int64_t qbase);
 // p += s F, F_{t-1} <- F for every point, and the next root square; steps

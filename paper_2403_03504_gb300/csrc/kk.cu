@@ -693,6 +693,12 @@ void kk_destroy(KkRun *run) { delete run; }
 
 int kk_classes(const KkRun *run) { return (int)run->cls.size(); }
 
+int64_t kk_blocks(const KkRun *run) {
+    int64_t n = 0;
+    for (const auto &k : run->cls) n += k->blocks();
+    return n;
+}
+
 // launches size class i on stream s
 void kk_enqueue(const KkRun *run, int i, const bgl_params *p, float2 *xy, int64_t qbase, bool init, int sweeps,
                 int32_t *d_out, cudaStream_t s, cudaEvent_t placed) {

@@ -12,9 +12,10 @@
   a run, whatever their number (64 bytes a node below), with the same bits as
   when a component has them all to itself; and a server's footprint estimate
   bounds what a request of one such component takes.
-* Kamada-Kawai classes of 608 blocks and more fill the chip; beside classes the
-  exact iterations' kernels ask for their shared-memory split: every component
-  gets the layout that it gets alone."""
+* Kamada-Kawai classes of 608 blocks and more fill the chip, and beside them the
+  FMM of up to 32,768 points has its separate sort; beside classes the exact
+  iterations' kernels ask for their shared-memory split: every component gets
+  the layout that it gets alone."""
 import numpy as np
 import pytest
 
@@ -131,17 +132,17 @@ def test_footprint_estimate_bounds_an_exact_request(ctx):
     g.destroy()
 
 
-def test_layout_beside_classes_that_fill_the_chip(ctx):
-    """20,000 components of 3 to 50 nodes (some 900 blocks) beside one of 3,000
-    in the exact sum."""
+@pytest.mark.parametrize("rep,size", [("exact", 3000), ("fmm", 10000)])
+def test_layout_beside_classes_that_fill_the_chip(ctx, rep, size):
+    """20,000 components of 3 to 50 nodes (some 900 blocks) beside a large one."""
     bgl = _bgl()
-    size = 3000
     sizes, u, v = synth.forest(8, 20000, 3.0, 50.0)
     base = int(sizes.sum())
     n, gu, gv = _trees(1, size, 3)
     g = bgl.Graph.from_edges(ctx, base + n, np.concatenate([u, base + gu]), np.concatenate([v, base + gv]))
     g.components(labels=False)
-    p = bgl.params(seed=6, fa2_iters=30, kk_sweeps=20, ksmax=0.05, repulsion=bgl.REP_EXACT)
+    p = bgl.params(seed=6, fa2_iters=30, kk_sweeps=20, ksmax=0.05,
+                   repulsion=bgl.REP_EXACT if rep == "exact" else bgl.REP_FMM)
     xy = g.layout(p)
     x, y = oracle.init_positions(6, np.arange(base, base + n))
     alone, _ = g.fa2_step(0, p, 30, np.stack([x, y], 1).astype(np.float32))
