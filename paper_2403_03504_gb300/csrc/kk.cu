@@ -414,11 +414,13 @@ __global__ void kk_kernel(KKArgs a) {
             // one overlap the other's (a pair past the component adds exactly
             // 0); with one the largest components' chains of steps took 36.4
             // ms of 2,000 components, with two 32.2, with four 33.4 (more
-            // pairs past the components)
+            // pairs past the components).  Groups of four and eight lanes with
+            // four nodes each have chains enough in a warp: one node (300,000
+            // components of 3 to 20 nodes 12.9 ms, 14.0 with two)
+            constexpr int M = CPL < 2 || (G < 16 && CPL > 2) ? 1 : 2;
 #pragma unroll
-            for (int j0 = 0; j0 < CPL; j0 += 2) {
+            for (int j0 = 0; j0 < CPL; j0 += M) {
                 if (j0 * G >= n) break;                  // the group's component has no node there
-                constexpr int M = CPL < 2 ? CPL : 2;
                 float2 kl[M], pi[M];
 #pragma unroll
                 for (int k = 0; k < M; ++k) {
