@@ -237,7 +237,8 @@ namespace bgl {
 // components and the ForceAtlas2 components are independent (Section 4), so
 // the KK size classes run beside the ForceAtlas2 iterations: each class on
 // a stream of its own, captured into the same CUDA graph as the iteration
-// loop (one graph launch lays out every component).
+// loop (after the distances of the larger ones, one graph launch lays out
+// every component).
 void layout_device(bgl_graph *g, const bgl_params *p, float *d_xy_out) {
     check_params(p);
     require_comp(g);

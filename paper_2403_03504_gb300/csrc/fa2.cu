@@ -1,24 +1,29 @@
 // ForceAtlas2 iteration (Section 3.2) on the device.
 //
 // One iteration over the ForceAtlas2 components [c0, c1):
-//   K1 repulsion      exact: tiles of 512 targets per block, sources of the
-//                     same component staged 1024 at a time in shared memory;
-//                     FMM components run the pipeline in fmm.cu instead.
-//                     f <- F_rep = kr m_i sum_j m_j (p_i - p_j) / |p_i - p_j|^2
-//   K2 attraction     fa <- -sum_{j adjacent} (p_i - p_j) - kg m_i p_i; one
-//      + gravity      thread per node; nodes of degree > 128 in chunks of 2048
-//                     entries, one block each, combined in chunk order.  It
-//                     runs on a second stream beside the repulsion, whose
-//                     final writes add fa: f <- F_rep + fa
-//   K3 swing/traction per-node |F_t - F_{t-1}|, |F_t + F_{t-1}| summed in FP64
-//                     per tile (warp shuffles); the last block to finish sums
-//                     each component's tiles (a warp per component, fixed
-//                     order) and updates s_G = min(tau trc / swg, 1.5 s_G)
+//   K1 repulsion      f <- F_rep = kr m_i sum_j m_j (p_i - p_j) / |p_i - p_j|^2.
+//                     Exact components: exact_kernel, a block per tile of 128
+//                     or 256 targets and stage of 1,024 sources, or per tile
+//                     with all sources (ExactSum).  FMM components: fmm.cu.
+//   K2 attraction     -sum_{j adjacent} (p_i - p_j) - kg m_i p_i, added to f.
+//      + gravity      Exact: blocks of their own in exact_kernel's launch;
+//                     the tile's last block to finish adds what they sum.
+//                     FMM: attraction_gravity_kernel on a second stream beside
+//                     the evaluation, whose final kernel adds fa.  Nodes of
+//                     degree > 128 in chunks of 2,048 entries, in chunk order
+//   K3 swing/traction |F_t - F_{t-1}|, |F_t + F_{t-1}| summed in FP32 over 32
+//                     nodes and in FP64 above (SwingArgs); a component's last
+//                     block to finish sets s_G = min(tau trc / swg, 1.5 s_G).
+//                     Exact: in exact_kernel.  FMM: in combine_kernel (fmm.cu)
+//                     for a component that runs alone, else
+//                     swing_traction_kernel
 //   K4 update         s_n = ks s_G / (1 + s_G sqrt|F_t - F_{t-1}|), capped at
 //                     ksmax / |F_t|; p_n += s_n F_t; F_{t-1} <- F_t
-// The sequence has fixed launch shapes, so it is captured once as the body of
-// a device-side WHILE loop in a CUDA graph: one launch runs all iterations.  Every sum has a fixed order, so
-// runs are bitwise reproducible.
+//                     (update_kernel; with the next root square in
+//                     update_root_kernel, fmm.cu, for an FMM component alone)
+// The sequence has fixed launch shapes, so a few iterations are captured as
+// the body of a device-side WHILE loop in a CUDA graph: one launch runs them
+// all.  Every sum has a fixed order, so runs are bitwise reproducible.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>

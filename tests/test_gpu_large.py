@@ -8,6 +8,7 @@
   sort of the visited nodes, in smaller ones from scans over the marks of all:
   equal to the oracle's on both sides of the line.  A sort that gives up
   (BGL_TEST_SORT_STALL=1, see test_gpu_recovery.py) is reported.
+  Either way a hop may meet several hubs.
 * The partial sums of exact components above 8,192 nodes take at most 512 MiB
   a run, whatever their number (64 bytes a node below), with the same bits as
   when a component has them all to itself; and a server's footprint estimate
@@ -149,4 +150,23 @@ def test_layout_beside_classes_that_fill_the_chip(ctx, rep, size):
     assert np.array_equal(xy[base:], alone)
     p.fa2_iters = 0                                  # the classes without iterations beside them
     assert np.array_equal(xy[:base], g.layout(p)[:base])
+    g.destroy()
+
+
+@pytest.mark.parametrize("hops", [1, 2, 3, 4])
+def test_khop_over_several_hubs_in_several_hops(ctx, hops):
+    """Hubs of 1,100 to 5,100 entries (more than a block's 1,024), two of them
+    met in the first hop and two more in each of the next ones."""
+    bgl = _bgl()
+    rng = np.random.default_rng(3)
+    n, hubs = 30000, 8
+    degree = 1100 + 570 * np.arange(hubs)
+    u = np.concatenate([np.repeat(np.arange(hubs), degree), np.arange(hubs - 2), [hubs, hubs]])
+    v = np.concatenate([rng.integers(hubs + 1, n, degree.sum()), np.arange(2, hubs), [0, 1]])
+    g = bgl.Graph.from_edges(ctx, n, u, v)
+    off, adj = g.csr()
+    ids, edges = oracle.khop(off, adj, hubs, hops)
+    got = g.khop(hubs, hops, n)
+    assert np.array_equal(got[0], ids)
+    assert sorted(zip(np.minimum(got[1], got[2]).tolist(), np.maximum(got[1], got[2]).tolist())) == edges
     g.destroy()
